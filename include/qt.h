@@ -72,7 +72,10 @@ typedef int32_t qt_status;
 
 /* search forms (qt_options.form) */
 #define QT_FORM_AUTO 0        /* library picks the fastest certified form: TC_RECHECK for
-                                 3 <= d <= 10, F32_RECHECK otherwise                      */
+                                 3 <= d <= 10, F32_RECHECK otherwise; for d <= 2 and grids
+                                 of at most 1024 points the FP32 screen runs only over the
+                                 few points that a table of the grid leaves (located search,
+                                 Algorithms II and III and given samples)                  */
 #define QT_FORM_PLAIN_F64 1   /* brute force, exact FP64 distances                       */
 #define QT_FORM_F32_RECHECK 2 /* FP32 brute-force screen, FP64 recheck of near ties      */
 #define QT_FORM_TC_RECHECK 3  /* tensor-core (tcgen05) screen, FP64 recheck              */

@@ -72,12 +72,15 @@ struct qt_ctx {
     std::map<std::string, DevBuf> dev;
     std::map<std::string, HostBuf> host;
     cudaStream_t cap_stream = nullptr;
-    cudaEvent_t ev_tables = nullptr;   // last use of the pinned descriptor tables
+    cudaEvent_t ev_tables = nullptr;   // end of the last forward step (workspace and tables in use until then)
+    cudaEvent_t ev_up[2] = {nullptr, nullptr};   // last upload from each of the two pinned table blocks
+    int up = 0;
     cudaEvent_t ev_k0 = nullptr, ev_k1 = nullptr;   // around the forward kernel (stats.ms)
     bool timed = false;
     // cached graph of the last forward call
     cudaGraphExec_t gexec = nullptr;
-    std::vector<unsigned char> gkey;
+    std::vector<unsigned char> gkey;   // what the captured graph does
+    std::vector<unsigned char> seen;   // what the last step launched directly did
     // autotuner cache: key -> samples per thread
     std::map<TuneKey, int> tune;
     int last_form = 0;
@@ -174,8 +177,11 @@ qt_status host_get(qt_ctx* ctx, const char* name, size_t bytes, void** out)
 {
     HostBuf& b = ctx->host[name];
     if (b.bytes < bytes) {
-        if (ctx->ev_tables) cudaEventSynchronize(ctx->ev_tables);
-        if (b.p) cudaFreeHost(b.p);
+        if (b.p) {
+            // an upload may still read it
+            if (ctx->ev_tables) cudaEventSynchronize(ctx->ev_tables);
+            cudaFreeHost(b.p);
+        }
         b.p = nullptr;
         b.bytes = 0;
         size_t want = std::max<size_t>(bytes, 256);
@@ -250,6 +256,8 @@ extern "C" qt_status qt_create(qt_ctx** out, int32_t device)
     ctx->smem_optin = prop.sharedMemPerBlockOptin;
     if (cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_tables, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_up[0], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_up[1], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreate(&ctx->ev_k0) != cudaSuccess || cudaEventCreate(&ctx->ev_k1) != cudaSuccess) {
         delete ctx;
         return QT_ECUDA;
@@ -270,6 +278,8 @@ extern "C" qt_status qt_destroy(qt_ctx* ctx)
         if (kv.second.p) cudaFreeHost(kv.second.p);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->ev_tables) cudaEventDestroy(ctx->ev_tables);
+    for (int u = 0; u < 2; ++u)
+        if (ctx->ev_up[u]) cudaEventDestroy(ctx->ev_up[u]);
     if (ctx->ev_k0) cudaEventDestroy(ctx->ev_k0);
     if (ctx->ev_k1) cudaEventDestroy(ctx->ev_k1);
     delete ctx;
@@ -324,6 +334,39 @@ struct Plan {
     std::vector<LayerDesc> layers;
     std::vector<GridInfo> grids;
     long long count_entries = 0;
+    // located search (d <= 2)
+    std::vector<CellGrid> cells;
+    long long cell_entries = 0, cell_floats = 0, cell_tile = 0;
+    int cell_g0 = 0, cell_g1 = 0;      // grids whose tables the step needs
+};
+
+// Device buffers of the located search.
+struct CellBufs {
+    void *tab = nullptr, *rec = nullptr, *pool = nullptr;
+    uint32_t pool_words = 0;
+};
+
+// The host's tables of a step, uploaded as one block: the zeroed status, the layer
+// and grid descriptors, the sampler's parameters and the located search's grids.
+// (Six separate copies and memsets cost 10 us of a 120 us call.)
+struct Tables {
+    size_t status = 0, layers = 0, grids = 0, pf = 0, pd = 0, cells = 0, near = 0, bytes = 0;
+    Tables(const Plan& P, bool with_near)
+    {
+        const size_t pcount = (size_t)std::max(1, P.n) * P.pstride;
+        auto take = [&](size_t n) {
+            const size_t at = bytes;
+            bytes = (bytes + n + 127) / 128 * 128;
+            return at;
+        };
+        status = take(sizeof(DevStatus));
+        layers = take(sizeof(LayerDesc) * P.layers.size());
+        grids = take(sizeof(GridInfo) * P.grids.size());
+        pf = take(pcount * 4);
+        pd = take(pcount * 8);
+        cells = take(sizeof(CellGrid) * P.cells.size());
+        near = take(with_near ? (size_t)P.n * kCellNearStride * 4 : 0);
+    }
 };
 
 struct FwdIO {
@@ -339,6 +382,49 @@ struct FwdIO {
 
 qt_status make_plan_full(qt_ctx* ctx, int d, int n, const int64_t* Ns, const double* mus, long long M,
                          const qt_options* o, bool from_arrays, Plan& P, int algo);
+
+// Bins along each axis of a grid's table: about 20 per point for d = 2 (the 2-factor
+// grids: 2.6 candidates per search, against 4.3 at 8 per point), at most 104 x 104, so
+// that the tables of two grids fit one CTA's shared memory; 16 per point for d = 1.
+void cell_bins(int d, long long N, int* nb0, int* nb1)
+{
+    if (d == 1) {
+        *nb0 = (int)std::min<long long>(8192, round_up(16 * N, 64));
+        *nb1 = 1;
+    } else {
+        const int nb = (int)std::ceil(std::sqrt(20.0 * (double)N));
+        *nb0 = *nb1 = (int)std::min<long long>(104, round_up(std::max(nb, 8), 8));
+    }
+}
+
+size_t cell_bytes(int d, long long N)
+{
+    if (N <= 1) return 0;
+    int a, b;
+    cell_bins(d, N, &a, &b);
+    return (size_t)a * b * 8 + (size_t)round_up(N * d, 4) * 4;
+}
+
+// Whether the automatic form takes the located search: d <= 2, indices of ten
+// bits, two tables within one CTA's shared memory and all of them within 1 GiB.  It
+// is the faster one at every size measured (us per call, brute force / located:
+// 4 dates x 3000 pairs on 64 points 125 / 66, 365 x 10^5 on 500 points 5500 / 1200,
+// 100 x 10^7 on 500 points 142900 / 19500, ten FP64 dates x 10^6 on 100 points
+// 3190 / 290); callers that name a form, a tile or the shared-memory histogram get
+// the brute-force kernels.
+bool cells_apply(size_t smem, int d, int n, const int64_t* Ns, const qt_options* o)
+{
+    if (o->form != QT_FORM_AUTO || d > 2 || o->tile_samples_per_thread > 0 || (o->flags & QT_FLAG_SMEM_HIST)) return false;
+    size_t total = 0, pair = 0, prev = 0;
+    for (int k = 0; k <= n; ++k) {
+        if (Ns[k] > kCellMaxN) return false;
+        const size_t b = cell_bytes(d, Ns[k]);
+        pair = std::max(pair, b + prev);
+        total += b;
+        prev = b;
+    }
+    return total <= (1ull << 30) && pair + 16 * 1024 <= smem;
+}
 
 // Work items per launch of the tensor-core form: all of them when the screen
 // kernel draws its own samples, as many as 2 GiB of drawn samples hold with the
@@ -368,6 +454,8 @@ qt_status make_plan(qt_ctx* ctx, int d, int n, const int64_t* Ns, const double* 
         if (k != only_layer) P.layers[k].items = 0;
     }
     P.layers[only_layer].coff = 0;
+    P.cell_g0 = only_layer;
+    P.cell_g1 = only_layer + 2;
     P.total_items = items;
     P.count_entries = (long long)P.layers[only_layer].NA * P.layers[only_layer].NB;
     if (P.form == kTcRecheck) P.tc_chunk_items = tc_chunk(P, o);
@@ -391,8 +479,10 @@ qt_status make_plan_full(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
         if (from_arrays) return fail(ctx, QT_EUNSUPPORTED, "the path-wise form draws its own paths");
         form = QT_FORM_F32_RECHECK;
     }
+    const bool cells = cells_apply(ctx->smem_optin, d, n, Ns, o);
     // automatic choice: the fastest certified form measured on GB300 -- the
-    // tensor-core screen for 3 <= d <= 10, the FP32 screen otherwise
+    // tensor-core screen for 3 <= d <= 10, the FP32 screen otherwise (for d <= 2 on
+    // the few candidates that the located search leaves)
     if (form == QT_FORM_AUTO) form = (d >= 3 && d <= 10) ? QT_FORM_TC_RECHECK : QT_FORM_F32_RECHECK;
     if (form != QT_FORM_PLAIN_F64 && form != QT_FORM_F32_RECHECK && form != QT_FORM_TC_RECHECK &&
         form != QT_FORM_ROUTER_CERT)
@@ -437,6 +527,74 @@ qt_status make_plan_full(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
         roff += G.Npad;
     }
     P.total_recs = roff;
+    if (cells) {
+        const bool f32 = o->sample_prec == QT_PREC_F32;
+        P.form = algo == 2 ? kPathCells : kCells;
+        P.block = kCellThreads;
+        P.cells.resize(P.ngrids);
+        size_t one = 0, pair = 0, prev = 0;
+        for (int g = 0; g < P.ngrids; ++g) {
+            CellGrid& C = P.cells[g];
+            memset(&C, 0, sizeof C);
+            for (int l = 0; l < d; ++l) C.mu[l] = P.grids[g].mu[l];
+            C.N = (int)Ns[g];
+            C.goff = P.grids[g].goff;
+            C.toff = P.cell_entries;
+            C.roff = P.cell_floats;
+            if (C.N > 1) {
+                cell_bins(d, C.N, &C.nb0, &C.nb1);
+                P.cell_entries += (long long)C.nb0 * C.nb1;
+                P.cell_floats += round_up((long long)C.N * d, 4);
+            }
+            const size_t b = cell_bytes(d, C.N);
+            one = std::max(one, b);
+            pair = std::max(pair, b + prev);
+            prev = b;
+        }
+        P.cell_g0 = 0;
+        P.cell_g1 = P.ngrids;
+        P.S = 1;
+        // CTAs of 1024 threads share two tables among 32 warps; few samples spread
+        // over more SMs in CTAs of 256 (4 x 3000 pairs: 12 or 48 CTAs)
+        P.tile = M * n >= 2ll * ctx->num_sms * kCellThreads ? kCellThreads : 256;
+        P.block = P.tile;
+        if (algo == 2) {
+            // one wave of CTAs over equal tiles of paths, S per thread at most
+            const int smax = f32 ? 8 : 4;
+            const long long G = ctx->num_sms, full = G * kCellThreads * smax;
+            const long long waves = (M + full - 1) / full;
+            P.cell_tile = round_up((M + G * waves - 1) / (G * waves), 32);
+            P.S = P.cell_tile <= kCellThreads ? 1 : smax;
+        }
+        P.grid_bytes = algo == 2 ? 2 * (size_t)round_up((long long)one, 128) : (size_t)round_up((long long)pair, 128);
+        P.layers.resize(n);
+        long long item = 0, coff = 0;
+        size_t hmax = 0;
+        const long long items_per_layer = (M + P.tile - 1) / P.tile;
+        for (int k = 0; k < n; ++k) {
+            LayerDesc& L = P.layers[k];
+            memset(&L, 0, sizeof L);
+            L.NA = (int)Ns[k];
+            L.NB = (int)Ns[k + 1];
+            L.gridA = k;
+            L.gridB = k + 1;
+            L.coff = coff;
+            L.item_begin = item;
+            L.items = (int)items_per_layer;
+            // a private histogram where a layer's counts are so few that the L2
+            // reductions of all CTAs would meet on them (the first layer: 1 x N_1)
+            const long long ent = (long long)L.NA * L.NB;
+            L.hist_smem = algo != 2 && !(o->flags & QT_FLAG_GLOBAL_HIST) && ent <= 2048 && M >= 16 * ent;
+            if (L.hist_smem) hmax = std::max(hmax, (size_t)ent * 4);
+            item += items_per_layer;
+            coff += ent;
+        }
+        P.total_items = algo == 2 ? (M + P.cell_tile - 1) / P.cell_tile : item;
+        P.count_entries = coff;
+        P.hist_bytes = round_up((long long)hmax, 16);
+        P.dyn_smem = P.grid_bytes + P.hist_bytes;
+        return QT_OK;
+    }
     if (algo == 2) {
         // Algorithm II: a CTA carries a tile of paths through every layer; the
         // FP32 records of one grid per shared-memory buffer, two buffers
@@ -656,26 +814,26 @@ bool stream_is_capturing(cudaStream_t st)
     return cs != cudaStreamCaptureStatusNone;
 }
 
-// Enqueue the whole forward step on `st`: table uploads, zeroing, record
+// Enqueue the whole forward step on `st`: table upload, zeroing, record
 // preparation, the persistent kernel.
 qt_status enqueue_forward(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long M, unsigned long long seed,
-                          const qt_options* o, int source, void* dparams_f, void* dparams_d, const void* hparams_f,
-                          const void* hparams_d, size_t pcount, void* dlayers, void* dgrids, const void* hlayers,
-                          const void* hgrids, void* drec32, void* drec64, DevStatus* dstatus, cudaStream_t st,
-                          void* dtiles, void* dtcitems)
+                          const qt_options* o, int source, const Tables& T, const void* htables, void* dtables,
+                          void* drec32, void* drec64, cudaStream_t st, void* dtiles, void* dtcitems,
+                          const CellBufs& cb, cudaEvent_t uploaded)
 {
-    QT_CUDA(cudaMemcpyAsync(dparams_f, hparams_f, pcount * 4, cudaMemcpyHostToDevice, st));
-    QT_CUDA(cudaMemcpyAsync(dparams_d, hparams_d, pcount * 8, cudaMemcpyHostToDevice, st));
-    QT_CUDA(cudaMemcpyAsync(dlayers, hlayers, sizeof(LayerDesc) * P.layers.size(), cudaMemcpyHostToDevice, st));
-    QT_CUDA(cudaMemcpyAsync(dgrids, hgrids, sizeof(GridInfo) * P.grids.size(), cudaMemcpyHostToDevice, st));
-    QT_CUDA(cudaMemsetAsync(dstatus, 0, sizeof(DevStatus), st));
+    unsigned char* dt = (unsigned char*)dtables;
+    DevStatus* dstatus = (DevStatus*)(dt + T.status);
+    void *dlayers = dt + T.layers, *dgrids = dt + T.grids, *dparams_f = dt + T.pf, *dparams_d = dt + T.pd;
+    QT_CUDA(cudaMemcpyAsync(dtables, htables, T.bytes, cudaMemcpyHostToDevice, st));
+    if (uploaded) QT_CUDA(cudaEventRecord(uploaded, st));
     const size_t csize = o->counts_type == QT_COUNTS_U32 ? 4 : 8;
     QT_CUDA(cudaMemsetAsync(io.counts, 0, csize * (size_t)P.count_entries, st));
     if (io.dump && io.dump->count > 0) {
         QT_CUDA(cudaMemsetAsync(io.dump->i, 0xFF, sizeof(int32_t) * (size_t)io.dump->count * P.n, st));
         QT_CUDA(cudaMemsetAsync(io.dump->j, 0xFF, sizeof(int32_t) * (size_t)io.dump->count * P.n, st));
     }
-    {
+    const bool cells = P.form == kCells || P.form == kPathCells;
+    if (!cells) {
         const int blk = 256;
         const long long nb = (P.total_recs + blk - 1) / blk;
         prep_records_kernel<<<(unsigned)nb, blk, 0, st>>>(
@@ -734,6 +892,21 @@ qt_status enqueue_forward(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long
         fp.dumpJ = io.dump->j;
     }
     fp.status = dstatus;
+    if (cells) {
+        fp.cells = (CellGrid*)(dt + T.cells);
+        fp.cell_tab = (unsigned long long*)cb.tab;
+        fp.cell_rec = (float*)cb.rec;
+        fp.cell_pool = (uint16_t*)cb.pool;
+        fp.cell_cursor = &dstatus->cell_cursor;
+        fp.cell_pool_cap = cb.pool_words;
+        fp.cell_g0 = P.cell_g0;
+        fp.cell_g1 = P.cell_g1;
+        fp.cell_near = (const float*)(dt + T.near);
+        fp.cell_tile = P.cell_tile;
+        fp.cell_ipl = P.cell_g1 - P.cell_g0 == P.ngrids ? P.layers[0].items : 0;
+        cudaError_t ce = launch_build_cells(P.d, fp, ctx->num_sms, st);
+        if (ce != cudaSuccess) return fail(ctx, QT_ECUDA, "table kernel launch: %s", cudaGetErrorString(ce));
+    }
     if (P.form == kRouterCert) {
         router_fill_params(static_cast<const qt_router*>(o->router), fp);
         long long pts = 0;
@@ -812,6 +985,45 @@ void key_append(std::vector<unsigned char>& k, const void* p, size_t n)
     k.insert(k.end(), b, b + n);
 }
 
+// FP64 layers of the located search: the pair (X - mu_A, Y - mu_B) as FP32 maps of
+// the normals, combined in FP64 (block layout: pair_near in qt_cells.cuh), and each
+// grid's bound on the resulting error: the normals' (2^-20 of their radius, at most
+// 8.6) through the maps, and a few FP32 roundings.
+void combine_near(const Plan& P, const double* params, float* out, CellGrid* cells)
+{
+    const int d = P.d;
+    for (int k = 0; k < P.n; ++k) {
+        const double* p = params + (long long)k * P.pstride;
+        const double *m = p, *b = p + d, *L = p + 2 * d, *A = L + d * d, *T = A + d * d;
+        float* o = out + (long long)k * kCellNearStride;
+        memset(o, 0, kCellNearStride * sizeof(float));
+        float *cA = o, *oL = o + d, *cB = oL + d * d, *oAL = cB + d, *oT = oAL + d * d;
+        const CellGrid& GA = P.cells[k];
+        const CellGrid& GB = P.cells[k + 1];
+        double errA = 0.0, errB = 0.0;
+        for (int l = 0; l < d; ++l) {
+            const double a = m[l] - (double)GA.mu[l];
+            double c = b[l] - (double)GB.mu[l], sa = 0.0, sb = 0.0;
+            for (int q = 0; q < d; ++q) {
+                c += A[l * d + q] * m[q];
+                double al = 0.0;
+                for (int r = 0; r < d; ++r) al += A[l * d + r] * L[r * d + q];
+                oL[l * d + q] = (float)L[l * d + q];
+                oAL[l * d + q] = (float)al;
+                oT[l * d + q] = (float)T[l * d + q];
+                sa += std::fabs(L[l * d + q]);
+                sb += std::fabs(al) + std::fabs(T[l * d + q]);
+            }
+            cA[l] = (float)a;
+            cB[l] = (float)c;
+            errA = std::max(errA, 8.6 * sa * 0x1.6p-20 + std::fabs(a) * 0x1p-22);
+            errB = std::max(errB, 8.6 * sb * 0x1.6p-20 + std::fabs(c) * 0x1p-22);
+        }
+        cells[k].err = std::max(cells[k].err, (float)(1.01 * errA));
+        cells[k + 1].err = std::max(cells[k + 1].err, (float)(1.01 * errB));
+    }
+}
+
 // Upload the tables of plan P and run it on `st`, directly or through the
 // cached CUDA graph.  `tag` prefixes the workspace names (the autotuner keeps
 // its own buffers so that it never invalidates the cached graph).
@@ -821,18 +1033,23 @@ qt_status run_plan(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long M, uns
 {
     qt_status s;
     const int n = P.n;
-    void *dlayers, *dgrids, *dpf, *dpd, *drec32 = nullptr, *drec64 = nullptr, *dstatus;
-    const size_t pbytes = (size_t)std::max(1, n) * P.pstride;
-    if ((s = dev_get(ctx, (tag + "layers").c_str(), sizeof(LayerDesc) * P.layers.size(), &dlayers))) return s;
-    if ((s = dev_get(ctx, (tag + "grids").c_str(), sizeof(GridInfo) * P.grids.size(), &dgrids))) return s;
-    if ((s = dev_get(ctx, (tag + "params_f").c_str(), pbytes * 4, &dpf))) return s;
-    if ((s = dev_get(ctx, (tag + "params_d").c_str(), pbytes * 8, &dpd))) return s;
-    if (P.form != kPlainF64) {
+    void *dtables, *drec32 = nullptr, *drec64 = nullptr;
+    CellBufs cb;
+    const bool near = source == kSampler && o->sample_prec == QT_PREC_F64 && P.form == kCells;
+    const Tables T(P, near);
+    if ((s = dev_get(ctx, (tag + "tables").c_str(), T.bytes, &dtables))) return s;
+    if (P.form == kCells || P.form == kPathCells) {
+        // long lists are rare (under one bin in a hundred): a quarter word per bin
+        cb.pool_words = (uint32_t)std::min<long long>(1ll << 30, P.cell_entries / 4 + 65536);
+        if ((s = dev_get(ctx, (tag + "cell_tab").c_str(), (size_t)P.cell_entries * 8, &cb.tab)) ||
+            (s = dev_get(ctx, (tag + "cell_rec").c_str(), (size_t)P.cell_floats * 4, &cb.rec)) ||
+            (s = dev_get(ctx, (tag + "cell_pool").c_str(), (size_t)cb.pool_words * 2, &cb.pool)))
+            return s;
+    } else if (P.form != kPlainF64) {
         if ((s = dev_get(ctx, (tag + "rec32").c_str(), (size_t)P.total_recs * P.rec_floats * 4, &drec32))) return s;
     } else {
         if ((s = dev_get(ctx, (tag + "rec64").c_str(), (size_t)P.total_recs * P.rec64 * 8, &drec64))) return s;
     }
-    if ((s = dev_get(ctx, (tag + "status").c_str(), sizeof(DevStatus), &dstatus))) return s;
     void* dtiles = nullptr;
     void* dtcitems = nullptr;
     if (P.form == kTcRecheck &&
@@ -840,33 +1057,11 @@ qt_status run_plan(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long M, uns
          (!P.tc_draw_in &&
           (s = dev_get(ctx, (tag + "tcitems").c_str(), (size_t)P.tc_chunk_items * P.tc_item_bytes, &dtcitems)))))
         return s;
-    void *hlayers, *hgrids, *hpf, *hpd;
-    if ((s = host_get(ctx, (tag + "layers").c_str(), sizeof(LayerDesc) * P.layers.size(), &hlayers))) return s;
-    if ((s = host_get(ctx, (tag + "grids").c_str(), sizeof(GridInfo) * P.grids.size(), &hgrids))) return s;
-    if ((s = host_get(ctx, (tag + "params_f").c_str(), pbytes * 4, &hpf))) return s;
-    if ((s = host_get(ctx, (tag + "params_d").c_str(), pbytes * 8, &hpd))) return s;
-    // the previous replay may still read the pinned tables
-    QT_CUDA(cudaEventSynchronize(ctx->ev_tables));
-    memcpy(hlayers, P.layers.data(), sizeof(LayerDesc) * P.layers.size());
-    memcpy(hgrids, P.grids.data(), sizeof(GridInfo) * P.grids.size());
-    float* pf = (float*)hpf;
-    double* pd = (double*)hpd;
-    memset(pf, 0, pbytes * 4);
-    memset(pd, 0, pbytes * 8);
-    if (params_d_host) {
-        for (long long e = 0; e < (long long)n * P.pstride; ++e) {
-            pd[e] = params_d_host[e];
-            pf[e] = (float)params_d_host[e];
-        }
-    }
-    ctx->status_buf = dstatus;
-    if (!use_graph) {
-        s = enqueue_forward(ctx, P, io, M, seed, o, source, dpf, dpd, hpf, hpd, pbytes, dlayers, dgrids, hlayers,
-                            hgrids, drec32, drec64, (DevStatus*)dstatus, st, dtiles, dtcitems);
-        if (s) return s;
-    } else {
-        // graph key: everything the enqueued work depends on
-        std::vector<unsigned char> key;
+    ctx->status_buf = (unsigned char*)dtables + T.status;
+
+    // everything the enqueued work depends on
+    std::vector<unsigned char> key;
+    if (use_graph) {
         key_append(key, &P.form, sizeof P.form);
         key_append(key, &P.S, sizeof P.S);
         key_append(key, &P.streamed, sizeof P.streamed);
@@ -880,17 +1075,54 @@ qt_status run_plan(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long M, uns
         if (io.dump) key_append(key, io.dump, sizeof *io.dump);
         key_append(key, P.layers.data(), sizeof(LayerDesc) * P.layers.size());
         key_append(key, P.grids.data(), sizeof(GridInfo) * P.grids.size());
-        key_append(key, pd, pbytes * 8);
-        if (!ctx->gexec || key != ctx->gkey) {
+        if (params_d_host) key_append(key, params_d_host, (size_t)n * P.pstride * 8);
+    }
+    const bool replay = use_graph && ctx->gexec && key == ctx->gkey;
+    const bool capturing = stream_is_capturing(st);
+    // the workspace is the last step's until that has ended (on whatever stream)
+    if (capturing) QT_CUDA(cudaEventSynchronize(ctx->ev_tables));
+    else QT_CUDA(cudaStreamWaitEvent(st, ctx->ev_tables, 0));
+    if (!replay) {
+        // A step is launched directly the first time and captured when the same call
+        // comes again: instantiating a graph costs 60 us, more than it saves a caller
+        // whose inputs change.  Direct launches alternate between two pinned blocks,
+        // each free again as soon as its upload is done; the graph has its own.
+        const bool capture = use_graph && key == ctx->seen;
+        const std::string block = capture ? "graph_tables" : capturing ? "cap_tables" : ctx->up ? "tables1" : "tables0";
+        void* ht;
+        if ((s = host_get(ctx, (tag + block).c_str(), T.bytes, &ht))) return s;
+        if (capture) QT_CUDA(cudaEventSynchronize(ctx->ev_tables));
+        else if (!capturing) QT_CUDA(cudaEventSynchronize(ctx->ev_up[ctx->up]));
+        unsigned char* hb = (unsigned char*)ht;
+        memset(hb, 0, T.bytes);
+        memcpy(hb + T.layers, P.layers.data(), sizeof(LayerDesc) * P.layers.size());
+        memcpy(hb + T.grids, P.grids.data(), sizeof(GridInfo) * P.grids.size());
+        if (params_d_host) {
+            float* pf = (float*)(hb + T.pf);
+            double* pd = (double*)(hb + T.pd);
+            for (long long e = 0; e < (long long)n * P.pstride; ++e) {
+                pd[e] = params_d_host[e];
+                pf[e] = (float)params_d_host[e];
+            }
+        }
+        CellGrid* hc = (CellGrid*)(hb + T.cells);
+        if (!P.cells.empty()) memcpy(hc, P.cells.data(), sizeof(CellGrid) * P.cells.size());
+        if (near) combine_near(P, params_d_host, (float*)(hb + T.near), hc);
+        if (!capture) {
+            s = enqueue_forward(ctx, P, io, M, seed, o, source, T, ht, dtables, drec32, drec64, st, dtiles, dtcitems,
+                                cb, capturing ? nullptr : ctx->ev_up[ctx->up]);
+            if (!capturing) ctx->up ^= 1;
+            if (s) return s;
+            if (use_graph) ctx->seen = key;
+        } else {
             if (ctx->gexec) {
                 cudaGraphExecDestroy(ctx->gexec);
                 ctx->gexec = nullptr;
             }
             cudaGraph_t graph = nullptr;
             QT_CUDA(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
-            qt_status es = enqueue_forward(ctx, P, io, M, seed, o, source, dpf, dpd, hpf, hpd, pbytes, dlayers,
-                                           dgrids, hlayers, hgrids, drec32, drec64, (DevStatus*)dstatus,
-                                           ctx->cap_stream, dtiles, dtcitems);
+            qt_status es = enqueue_forward(ctx, P, io, M, seed, o, source, T, ht, dtables, drec32, drec64,
+                                           ctx->cap_stream, dtiles, dtcitems, cb, nullptr);
             cudaError_t ee = cudaStreamEndCapture(ctx->cap_stream, &graph);
             if (es != QT_OK || ee != cudaSuccess) {
                 if (graph) cudaGraphDestroy(graph);
@@ -906,8 +1138,8 @@ qt_status run_plan(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long M, uns
             }
             ctx->gkey = key;
         }
-        QT_CUDA(cudaGraphLaunch(ctx->gexec, st));
     }
+    if (use_graph && ctx->gexec && key == ctx->gkey) QT_CUDA(cudaGraphLaunch(ctx->gexec, st));
     QT_CUDA(cudaEventRecord(ctx->ev_tables, st));
     return QT_OK;
 }
@@ -1085,7 +1317,8 @@ qt_status forward_common(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
         P2.euler = euler;
         P = P2;
     }
-    if (P.form != kTcRecheck && P.form != kRouterCert && P.form != kPathwise && o->tile_samples_per_thread <= 0 &&
+    if (P.form != kTcRecheck && P.form != kRouterCert && P.form != kPathwise && P.form != kCells &&
+        P.form != kPathCells && o->tile_samples_per_thread <= 0 &&
         !(o->flags & QT_FLAG_NO_TUNE) && !capturing && o->spin_budget >= 0) {
         const TuneKey key = tune_key(P, source == kArrays ? 0 : o->sample_prec, Ns, n);
         if (!ctx->tune.count(key)) {
@@ -1266,6 +1499,17 @@ extern "C" qt_status qt_transitions_workspace(const qt_model* model, const qt_op
     for (int k = 0; k <= n; ++k) recs += round_up(model->N[k], kChunk);
     const long long pstride = param_stride(d);
     size_t b = sizeof(LayerDesc) * n + sizeof(GridInfo) * (n + 1) + (size_t)n * pstride * 12 + sizeof(DevStatus);
+    if (cells_apply(227 * 1024, d, n, model->N, &o)) {
+        size_t entries = 0;
+        for (int k = 0; k <= n; ++k) {
+            int x = 0, y = 0;
+            if (model->N[k] > 1) cell_bins(d, model->N[k], &x, &y);
+            entries += (size_t)x * y;
+            b += cell_bytes(d, model->N[k]);
+        }
+        *bytes = b + sizeof(CellGrid) * (n + 1) + (size_t)n * kCellNearStride * 4 + (entries / 4 + 65536) * 2;
+        return QT_OK;
+    }
     b += o.form == QT_FORM_PLAIN_F64 ? (size_t)recs * rec64_for(dm) * 8 : (size_t)recs * rec_floats_for(dm) * 4;
     *bytes = b;
     return QT_OK;

@@ -1,0 +1,266 @@
+// qt_cells.cuh -- located nearest-cell search for d <= 2: a table of small boxes
+// ("bins") over each grid, every bin holding the few grid points whose Voronoi
+// cell can meet it, so that a search evaluates one to four distances instead of
+// all N_k (Sec. 3.2 of Pages & Wilbertz, arXiv:1101.3228, searches by brute
+// force; its kd-tree attempt is the prior art for a located search).
+//
+// Table of a grid (built per call by build_cells_kernel, one 64-bit entry per
+// bin): up to six 10-bit point indices in increasing order and their number in
+// the top four bits; kCellPool = a longer list in the pool (offset in bits 0-31,
+// length in bits 32-47); kCellScan = every point of the grid.  A point j is left
+// out of a bin only if one other point is nearer by more than every rounding
+// below, everywhere in the bin enlarged by a sixteenth of its width, so that the
+// exact FP64 argmin and everything tied with it is always in the list.
+//
+// Certificate: with a = x - mu in FP32 and g = fl32(c - mu), D~ = sum (a - g)^2
+// satisfies |D~ - D| <= err(D) = sqrt(d) (kappa D + e^2 / kappa) + d e^2 +
+// (d + 6) 2^-24 D, e the sum of both coordinates' errors, for any kappa > 0
+// (2 sqrt(D) e <= kappa D + e^2 / kappa).  The best candidate is the exact argmin
+// when second - best > 2 err(second); otherwise the exact FP64 distances of the
+// bin's candidates decide.  A sample whose e is f <= 1 times the grid's bound takes
+// f kappa: 2 err(D) = f (c1 D + c2) + c3 D.
+//
+// Why bins: brute force spends 2 d flops on each of N_k + N_{k+1} candidates (1000
+// on the 2-factor workload), and only the few points around a sample can be its
+// cell.  About 20 bins per point (104 x 104 at most: two tables fit one CTA's
+// shared memory) leave 2.6 candidates per search on average and 4 for the slowest
+// lane of a warp on the 2-factor grids; 64 x 64 bins leave 4.3 and 6.6.
+#pragma once
+#include "qt_forward.cuh"
+
+namespace qt {
+
+constexpr int kCellInline = 6;         // indices held in an entry
+constexpr int kCellPool = 15;          // entry refers to the pool
+constexpr int kCellScan = 14;          // entry stands for the whole grid
+constexpr uint64_t kCellScanEntry = (uint64_t)kCellScan << 60;
+
+__device__ __forceinline__ float cell_dist(const float* __restrict__ rec, int j, const float (&a)[1])
+{
+    const float dx = a[0] - rec[j];
+    return dx * dx;
+}
+__device__ __forceinline__ float cell_dist(const float* __restrict__ rec, int j, const float (&a)[2])
+{
+    const float2 g = reinterpret_cast<const float2*>(rec)[j];
+    const float dx = a[0] - g.x, dy = a[1] - g.y;
+    return __fmaf_rn(dy, dy, dx * dx);
+}
+
+// Lists longer than an entry: the pool's, or the whole grid (records in shared
+// memory).  The whole grid also serves samples outside the box, whose error grows
+// with their distance: e is scaled by (|a| + R) / S <= 1 + |a| / S there.
+// Returns the index, with the top bit set when the distances do not certify it.
+template <int DM>
+__device__ __noinline__ uint32_t cell_long_list(const float* __restrict__ rec, int N, const uint16_t* __restrict__ pool,
+                                                uint64_t e, float a0, float a1, float f, float c1, float c2, float c3,
+                                                float inv_span)
+{
+    const bool scan = (int)(e >> 60) == kCellScan;
+    const uint16_t* lst = pool + (uint32_t)e;
+    const int cnt = scan ? N : (int)((e >> 32) & 0xFFFFu);
+    float a[DM];
+    a[0] = a0;
+    if constexpr (DM == 2) a[1] = a1;
+    float best = __int_as_float(0x7F800000), second = best;
+    uint32_t bi = 0;
+    for (int q = 0; q < cnt; ++q) {
+        const int j = scan ? q : (int)lst[q];
+        const float D = cell_dist(rec, j, a);
+        second = fminf(second, fmaxf(D, best));
+        bi = D < best ? (uint32_t)j : bi;
+        best = fminf(best, D);
+    }
+    if (scan) {
+        const float g = 1.0f + (fabsf(a0) + fabsf(a1)) * inv_span;
+        f *= g * g;
+    }
+    const bool need = !(second - best > __fmaf_rn(f, __fmaf_rn(c1, second, c2), c3 * second));
+    return bi | (need ? 0x80000000u : 0u);
+}
+
+// Number of the bin of coordinate a along one axis: the FMA rounds a / h + origin to
+// the nearest integer in the low bits of a float near 2^23; whatever lies outside
+// the axis (or is not finite) gives a number outside [0, nb).
+__device__ __forceinline__ uint32_t cell_bin(float a, float inv_h, float org)
+{
+    return (uint32_t)__float_as_int(__fmaf_rn(a, inv_h, org)) - 0x4B000000u;
+}
+
+// Nearest candidate of the centred sample `a` in the grid G (shared memory: G, and
+// its table and records at `sm`); f: the sample's error as a share of the grid's
+// bound.  `entry` is its bin's list, `need` is set when the FP32 distances do not
+// certify the pick.
+template <int DM>
+__device__ __forceinline__ int cell_search(const CellGrid& G, const unsigned char* sm, const uint16_t* __restrict__ pool,
+                                           const float (&a)[DM], float f, uint64_t& entry, bool& need)
+{
+    const float4 axes = *reinterpret_cast<const float4*>(G.inv_h);
+    uint32_t b = cell_bin(a[0], axes.x, axes.z);
+    bool in = b < (uint32_t)G.nb0;
+    if constexpr (DM == 2) {
+        const uint32_t b1 = cell_bin(a[1], axes.y, axes.w);
+        in = in && b1 < (uint32_t)G.nb1;
+        b += b1 * (uint32_t)G.nb0;
+    }
+    uint64_t e = kCellScanEntry;
+    if (in) e = reinterpret_cast<const uint64_t*>(sm)[b];
+    entry = e;
+    const int cnt = (int)(e >> 60);
+    int idx = (int)(e & 1023u);
+    need = false;
+    const float* rec = reinterpret_cast<const float*>(sm + (size_t)((uint32_t)G.nb0 * (uint32_t)G.nb1 * 8u));
+    if (cnt > kCellInline) {
+        const uint32_t r = cell_long_list<DM>(rec, G.N, pool, e, a[0], DM == 2 ? a[DM - 1] : 0.0f, f, G.c1, G.c2, G.c3,
+                                              G.inv_span);
+        idx = (int)(r & 0x7FFFFFFFu);
+        need = (r >> 31) != 0;
+    } else if (cnt > 1) {
+        float best = cell_dist(rec, idx, a), second = __int_as_float(0x7F800000);
+        uint64_t r = e;
+        for (int q = 1; q < cnt; ++q) {
+            r >>= 10;
+            const int j = (int)(r & 1023u);
+            const float D = cell_dist(rec, j, a);
+            second = fminf(second, fmaxf(D, best));
+            idx = D < best ? j : idx;
+            best = fminf(best, D);
+        }
+        need = !(second - best > __fmaf_rn(f, __fmaf_rn(G.c1, second, G.c2), G.c3 * second));
+    }
+    return idx;
+}
+
+// Exact FP64 argmin over a bin's candidates (lowest index among equal distances).
+template <int DM>
+__device__ __noinline__ int cell_exact(const double (&z)[DM], uint64_t e, const uint16_t* __restrict__ pool,
+                                       const double* __restrict__ g64, int N, int d)
+{
+    const int kind = (int)(e >> 60);
+    const int cnt = kind == kCellScan ? N : (kind == kCellPool ? (int)((e >> 32) & 0xFFFFu) : kind);
+    double best = __longlong_as_double(0x7FF0000000000000LL);
+    int bi = 0;
+    for (int q = 0; q < cnt; ++q) {
+        const int j = kind == kCellScan ? q
+                                        : (kind == kCellPool ? (int)pool[(uint32_t)e + q] : (int)((e >> (10 * q)) & 1023u));
+        const double dj = dist64<DM>(z, g64 + (long long)j * d, d);
+        if (dj < best) {
+            best = dj;
+            bi = j;
+        }
+    }
+    return bi;
+}
+
+// Bulk copies of a grid's table and records into `dst` (one thread); returns the bytes.
+template <int DM>
+__device__ __forceinline__ uint32_t cell_stage_bytes(const CellGrid& G)
+{
+    return G.N > 1 ? (uint32_t)G.nb0 * G.nb1 * 8u + (uint32_t)((G.N * DM + 3) / 4 * 4) * 4u : 0u;
+}
+template <int DM>
+__device__ __forceinline__ void cell_stage(const ForwardParams& p, const CellGrid& G, uint32_t dst, uint32_t bar)
+{
+    if (G.N <= 1) return;
+    const uint32_t tb = (uint32_t)G.nb0 * G.nb1 * 8u;
+    bulk_g2s(dst, p.cell_tab + G.toff, tb, bar);
+    bulk_g2s(dst + tb, p.cell_rec + G.roff, (uint32_t)((G.N * DM + 3) / 4 * 4) * 4u, bar);
+}
+
+// ------------------------------------------------------------------ FP32 stand-in of the FP64 pair draw
+//
+// FP64 samples cost the FP64 pipe about 250 operations a pair, at 1/64 of the
+// FP32 rate: 3.0 ms for the 10^7 pairs of the 1-d workload.  The cells of nearly
+// all of them need far fewer digits: the pair is drawn from the same Philox words
+// with FP32 logarithm, square root, sine and cosine (each normal within
+// 2^-20 times its radius, radius <= 8.6), mapped by matrices already combined and
+// centred in FP64 on the host, and the certificate carries that error; the
+// uncertified few are drawn again in FP64.
+
+__device__ __forceinline__ float box_muller_near(const Philox4& w, float& g0, float& g1)
+{
+    const unsigned long long n0 = 2ull * (((unsigned long long)(w.v[0] >> 6) << 26) | (w.v[1] >> 6)) + 1ull;
+    const float u = __ull2float_rn(n0) * 0x1p-53f;
+    // ln u = e ln 2 + 2 atanh((f - 1)/(f + 1)); near 1 the difference 1 - u is
+    // taken from the integer, so that nothing cancels
+    float fm1, el2;
+    if (u > 0.70710678f) {
+        fm1 = -(__ull2float_rn((1ull << 53) - n0) * 0x1p-53f);
+        el2 = 0.0f;
+    } else {
+        const uint32_t bits = __float_as_uint(u);
+        int e = (int)(bits >> 23) - 127;
+        float f = __uint_as_float((bits & 0x007FFFFFu) | 0x3F800000u);
+        if (f > 1.41421354f) {
+            f *= 0.5f;
+            e += 1;
+        }
+        fm1 = f - 1.0f;
+        el2 = (float)e * 0.693147182f;
+    }
+    const float s = __fdividef(fm1, fm1 + 2.0f);
+    const float z = s * s;
+    float q = __fmaf_rn(z, 1.0f / 11.0f, 1.0f / 9.0f);
+    q = __fmaf_rn(q, z, 1.0f / 7.0f);
+    q = __fmaf_rn(q, z, 1.0f / 5.0f);
+    q = __fmaf_rn(q, z, 1.0f / 3.0f);
+    const float lnf = 2.0f * __fmaf_rn(s * z, q, s);
+    const float rad = __fsqrt_rn(-2.0f * (el2 + lnf));
+    // angle 2 pi u1: the quarter is the top two bits, x the next 32 of u1's 52 bits
+    const uint32_t quarter = w.v[2] >> 30;
+    const uint32_t x = ((w.v[2] << 2) & 0xFFFFFF00u) | (w.v[3] >> 24);
+    const float f = (float)x * 0x1p-32f;
+    const bool fold = f > 0.5f;
+    const float th = (fold ? 1.0f - f : f) * 1.57079633f;
+    const float t2 = th * th;
+    float ps = __fmaf_rn(t2, 1.0f / 362880.0f, -1.0f / 5040.0f);
+    ps = __fmaf_rn(ps, t2, 1.0f / 120.0f);
+    ps = __fmaf_rn(ps, t2, -1.0f / 6.0f);
+    const float st = __fmaf_rn(th * t2, ps, th);
+    float pc = __fmaf_rn(t2, -1.0f / 3628800.0f, 1.0f / 40320.0f);
+    pc = __fmaf_rn(pc, t2, -1.0f / 720.0f);
+    pc = __fmaf_rn(pc, t2, 1.0f / 24.0f);
+    pc = __fmaf_rn(pc, t2, -0.5f);
+    const float ct = __fmaf_rn(t2, pc, 1.0f);
+    const float s0 = fold ? ct : st, c0 = fold ? st : ct;
+    const float sa = (quarter & 1u) ? c0 : s0, ca = (quarter & 1u) ? s0 : c0;
+    const float sn = (quarter & 2u) ? -sa : sa;
+    const float cs = (quarter == 1u || quarter == 2u) ? -ca : ca;
+    g0 = rad * cs;
+    g1 = rad * sn;
+    return rad;
+}
+
+// Centred pair (X - mu_A, Y - mu_B) of an FP64 layer within its dA, dB: block P =
+// [cA (DM), L (DM^2), cB (DM), A L (DM^2), T (DM^2)].  Returns the largest radius as
+// a share of the 8.6 that dA and dB allow for.
+template <int DM>
+__device__ __forceinline__ float pair_near(const float* __restrict__ P, uint64_t seed, int k, uint64_t m,
+                                          float (&a)[DM], float (&b)[DM])
+{
+    float g[2 * DM], rad = 0.0f;
+#pragma unroll
+    for (int r = 0; r < DM; ++r) {
+        const Philox4 w = philox4x32_10((uint32_t)m, (uint32_t)(m >> 32), (uint32_t)k, (uint32_t)r, (uint32_t)seed,
+                                        (uint32_t)(seed >> 32));
+        rad = fmaxf(rad, box_muller_near(w, g[2 * r], g[2 * r + 1]));
+    }
+    const float* pL = P + DM;
+    const float* pc = pL + DM * DM;
+    const float* pAL = pc + DM;
+    const float* pT = pAL + DM * DM;
+#pragma unroll
+    for (int l = 0; l < DM; ++l) {
+        a[l] = P[l];
+        b[l] = pc[l];
+#pragma unroll
+        for (int q = 0; q < DM; ++q) {
+            a[l] = __fmaf_rn(pL[l * DM + q], g[q], a[l]);
+            b[l] = __fmaf_rn(pAL[l * DM + q], g[q], b[l]);
+            b[l] = __fmaf_rn(pT[l * DM + q], g[DM + q], b[l]);
+        }
+    }
+    return rad * (1.0001f / 8.6f);
+}
+
+}  // namespace qt

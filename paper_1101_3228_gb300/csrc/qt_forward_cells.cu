@@ -1,0 +1,442 @@
+// qt_forward_cells.cu -- located search (qt_cells.cuh) for d <= 2: the tables of
+// every grid, and Algorithm III (Pages & Wilbertz, arXiv:1101.3228, Sec. 4) or
+// the counting of given samples on them.
+#include "qt_cells.cuh"
+#include "qt_launch.h"
+
+namespace qt {
+
+namespace {
+
+constexpr int kBuildThreads = 256;
+constexpr int kBuildWarps = kBuildThreads / 32;
+constexpr int kPatchX = 8, kPatchY = 4;   // bins of a patch, one per lane (d = 1: 32 x 1)
+
+__device__ __forceinline__ float warp_min(float v)
+{
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) v = fminf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    return v;
+}
+__device__ __forceinline__ float warp_max(float v)
+{
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    return v;
+}
+
+}  // namespace
+
+// Table of grid p.cell_g0 + blockIdx.x (patches blockIdx.y, blockIdx.y + gridDim.y, ...).
+// A warp takes a patch of 32 bins: it finds the points that can be nearest
+// somewhere in the patch (about 25 of 500), then every lane tests those against
+// its own bin.  Point j is dropped from a box with centre c and half-widths h when,
+// against the point i nearest to c (for a bin also against the second nearest),
+//   D_j(x) - D_i(x) = |g_j - c|^2 - |g_i - c|^2 - 2 (x - c).(g_j - g_i)
+// is positive on the whole box by more than `marg`, which covers the FP32
+// rounding of the points and of this test.
+template <int DM>
+__global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const ForwardParams p)
+{
+    __shared__ float s_g[kCellMaxN * DM];
+    __shared__ uint16_t s_surv[kBuildWarps][kCellMaxN];
+    __shared__ float s_red[kBuildWarps][2 * DM + 1];
+    CellGrid& G = p.cells[p.cell_g0 + blockIdx.x];
+    const int N = G.N;
+    if (N <= 1) return;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const double* g64 = p.g64 + G.goff * DM;
+    float mn[DM], mx[DM], r2 = 0.0f;
+#pragma unroll
+    for (int l = 0; l < DM; ++l) {
+        mn[l] = __int_as_float(0x7F800000);
+        mx[l] = -__int_as_float(0x7F800000);
+    }
+    for (int j = tid; j < N; j += kBuildThreads) {
+        float n2 = 0.0f;
+#pragma unroll
+        for (int l = 0; l < DM; ++l) {
+            const float v = __double2float_rn(__dsub_rn(g64[(long long)j * DM + l], (double)G.mu[l]));
+            s_g[j * DM + l] = v;
+            mn[l] = fminf(mn[l], v);
+            mx[l] = fmaxf(mx[l], v);
+            n2 = __fmaf_rn(v, v, n2);
+            if (blockIdx.y == 0) p.cell_rec[G.roff + (long long)j * DM + l] = v;
+        }
+        r2 = fmaxf(r2, n2);
+    }
+#pragma unroll
+    for (int l = 0; l < DM; ++l) {
+        mn[l] = warp_min(mn[l]);
+        mx[l] = warp_max(mx[l]);
+        if (lane == 0) {
+            s_red[warp][2 * l] = mn[l];
+            s_red[warp][2 * l + 1] = mx[l];
+        }
+    }
+    r2 = warp_max(r2);
+    if (lane == 0) s_red[warp][2 * DM] = r2;
+    __syncthreads();
+    for (int w = 0; w < kBuildWarps; ++w) {
+#pragma unroll
+        for (int l = 0; l < DM; ++l) {
+            mn[l] = fminf(mn[l], s_red[w][2 * l]);
+            mx[l] = fmaxf(mx[l], s_red[w][2 * l + 1]);
+        }
+        r2 = fmaxf(r2, s_red[w][2 * DM]);
+    }
+    // the box: the grid's own, a quarter of its width wider on every side (quantizers
+    // reach about 3 standard deviations, so the box reaches 4.5); bin b of an axis is
+    // centred on (b - K) h, K an integer
+    const float R = __fsqrt_rn(r2) * 1.0001f;
+    const int nb[2] = {G.nb0, G.nb1};
+    float K[DM], h[DM], hmin = __int_as_float(0x7F800000), A2 = 0.0f;
+#pragma unroll
+    for (int l = 0; l < DM; ++l) {
+        const float ext = fmaxf(mx[l] - mn[l], fmaxf(0x1p-16f * R, 1e-30f));
+        h[l] = 1.5f * ext / (float)nb[l];
+        // a grid far from its centre has no bins here: `usable` is false for it
+        K[l] = fminf(fmaxf(rintf((0.25f * ext - mn[l]) / h[l]), -4194304.0f), 4194304.0f);
+        const float far_ = fmaxf(fabsf(mn[l]), fabsf(mx[l])) + 0.25f * ext + 2.0f * h[l];
+        A2 = __fmaf_rn(far_, far_, A2);
+        hmin = fminf(hmin, h[l]);
+    }
+    const float S = (__fsqrt_rn(A2) + R) * 1.0001f;
+    const float er = 0x1p-24f * 1.01f * S, e = er + G.err;
+    // the enlarged bins must cover the error of the centred sample and of its bin number
+    const bool usable = 32.0f * (G.err + 0x1p-21f * S) <= hmin;
+    const float marg = 0x1p-18f * S * S;
+    if (blockIdx.y == 0 && tid == 0) {
+        const float sq = DM == 1 ? 1.0f : 1.41421357f;
+        const float kappa = fmaxf(0x1p-22f, e / (2.0f * hmin));
+#pragma unroll
+        for (int l = 0; l < DM; ++l) {
+            G.inv_h[l] = 1.0f / h[l];
+            G.org[l] = 8388608.0f + K[l];
+        }
+        G.c1 = 2.02f * sq * kappa;
+        G.inv_span = 1.0f / S;
+        G.c2 = 2.02f * (sq * (e / kappa) * e + (float)DM * e * e);
+        G.c3 = 2.02f * (float)(DM + 6) * 0x1p-24f;
+        G.f0 = er / e;
+    }
+    const int pnx = DM == 1 ? nb[0] / 32 : nb[0] / kPatchX, pny = DM == 1 ? 1 : nb[1] / kPatchY;
+    unsigned long long* tab = p.cell_tab + G.toff;
+    uint16_t* surv = s_surv[warp];
+    for (int pt = blockIdx.y * kBuildWarps + warp; pt < pnx * pny; pt += gridDim.y * kBuildWarps) {
+        const int px = pt % pnx, py = pt / pnx;
+        // this lane's bin
+        const int x = DM == 1 ? px * 32 + lane : px * kPatchX + (lane & 7), y = DM == 1 ? 0 : py * kPatchY + (lane >> 3);
+        unsigned long long* out = tab + (long long)y * nb[0] + x;
+        if (!usable) {
+            *out = kCellScanEntry;
+            continue;
+        }
+        // ---- points that can win somewhere in the patch
+        float c[DM], hw[DM];
+        c[0] = ((DM == 1 ? (float)(px * 32) + 15.5f : (float)(px * kPatchX) + 3.5f) - K[0]) * h[0];
+        hw[0] = h[0] * (DM == 1 ? 16.1f : 4.1f);
+        if constexpr (DM == 2) {
+            c[1] = ((float)(py * kPatchY) + 1.5f - K[1]) * h[1];
+            hw[1] = h[1] * 2.1f;
+        }
+        float bD = __int_as_float(0x7F800000);
+        int bi = 0x7FFFFFFF;
+        for (int j = lane; j < N; j += 32) {
+            float D = 0.0f;
+#pragma unroll
+            for (int l = 0; l < DM; ++l) {
+                const float t = s_g[j * DM + l] - c[l];
+                D = __fmaf_rn(t, t, D);
+            }
+            if (D < bD) {
+                bD = D;
+                bi = j;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) {
+            const float od = __shfl_xor_sync(0xFFFFFFFFu, bD, o);
+            const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
+            if (od < bD || (od == bD && oi < bi)) {
+                bD = od;
+                bi = oi;
+            }
+        }
+        if (bi >= N) bi = 0;                        // non-finite points: nothing is dropped below
+        int ns = 0;
+        for (int j0 = 0; j0 < N; j0 += 32) {
+            const int j = j0 + lane;
+            bool keep = false;
+            if (j < N) {
+                float D = 0.0f, slack = 0.0f;
+#pragma unroll
+                for (int l = 0; l < DM; ++l) {
+                    const float t = s_g[j * DM + l] - c[l];
+                    D = __fmaf_rn(t, t, D);
+                    slack = __fmaf_rn(fabsf(s_g[j * DM + l] - s_g[bi * DM + l]), hw[l], slack);
+                }
+                keep = !(D - bD - 2.0f * slack > marg);
+            }
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, keep);
+            if (keep) surv[ns + __popc(m & ((1u << lane) - 1u))] = (uint16_t)j;
+            ns += __popc(m);
+        }
+        __syncwarp();
+        // ---- this lane's bin
+        c[0] = ((float)x - K[0]) * h[0];
+        hw[0] = 0.5f * 1.125f * h[0];
+        if constexpr (DM == 2) {
+            c[1] = ((float)y - K[1]) * h[1];
+            hw[1] = 0.5f * 1.125f * h[1];
+        }
+        float D0 = __int_as_float(0x7F800000), D1 = D0;
+        int i0 = surv[0], i1 = surv[0];
+        for (int t = 0; t < ns; ++t) {
+            const int j = surv[t];
+            float D = 0.0f;
+#pragma unroll
+            for (int l = 0; l < DM; ++l) {
+                const float v = s_g[j * DM + l] - c[l];
+                D = __fmaf_rn(v, v, D);
+            }
+            if (D < D0) {
+                D1 = D0;
+                i1 = i0;
+                D0 = D;
+                i0 = j;
+            } else if (D < D1) {
+                D1 = D;
+                i1 = j;
+            }
+        }
+        auto keeps = [&](int j) {
+            float D = 0.0f, sl0 = 0.0f, sl1 = 0.0f;
+#pragma unroll
+            for (int l = 0; l < DM; ++l) {
+                const float gj = s_g[j * DM + l], v = gj - c[l];
+                D = __fmaf_rn(v, v, D);
+                sl0 = __fmaf_rn(fabsf(gj - s_g[i0 * DM + l]), hw[l], sl0);
+                sl1 = __fmaf_rn(fabsf(gj - s_g[i1 * DM + l]), hw[l], sl1);
+            }
+            return !(D - D0 - 2.0f * sl0 > marg) && !(D - D1 - 2.0f * sl1 > marg);
+        };
+        uint64_t ent = 0;
+        int cnt = 0;
+        for (int t = 0; t < ns; ++t) {
+            const int j = surv[t];
+            if (!keeps(j)) continue;
+            if (cnt < kCellInline) ent |= (uint64_t)j << (10 * cnt);
+            ++cnt;
+        }
+        if (cnt <= kCellInline) {
+            ent |= (uint64_t)cnt << 60;
+        } else {
+            const uint32_t off = atomicAdd(p.cell_cursor, (uint32_t)cnt);
+            if (off + (uint32_t)cnt <= p.cell_pool_cap && off + (uint32_t)cnt >= off) {
+                int w = 0;
+                for (int t = 0; t < ns; ++t) {
+                    const int j = surv[t];
+                    if (keeps(j)) p.cell_pool[off + w++] = (uint16_t)j;
+                }
+                ent = (uint64_t)off | ((uint64_t)cnt << 32) | ((uint64_t)kCellPool << 60);
+            } else {
+                ent = kCellScanEntry;
+            }
+        }
+        *out = ent;
+        __syncwarp();
+    }
+}
+
+// Exact FP64 cell of sample m (X or Y) among the candidates of its bin.
+template <int DM>
+static __device__ __noinline__ int cell_recheck(const ForwardParams& p, const float* spf, const double* spd, int k,
+                                                unsigned long long m, bool wantY, uint64_t e, const CellGrid& G)
+{
+    double z[DM];
+    exact_sample<DM>(p, spf, spd, k, m, wantY, z);
+    atomicAdd(&p.status->rechecks, 1ull);
+    return cell_exact<DM>(z, e, p.cell_pool, p.g64 + G.goff * DM, G.N, DM);
+}
+
+// The forward step.  MODE 0: FP32 samples, 1: FP64 samples (drawn in FP32 first,
+// qt_cells.cuh), 2: given samples.  A work item is (layer, blockDim.x samples), one
+// sample per thread; a CTA takes a contiguous run of items, so that it loads the
+// two tables of a layer (170 KB at most) once or twice per launch instead of once
+// per item and layer.  What bounds it: issue slots (87% busy, 640 instructions a
+// pair at d = 2, most of them the draw).  2-factor workload, 10^9 pairs: 19.5 ms,
+// against 142.9 ms for brute force over 1000 candidates a pair.
+template <int DM, int MODE>
+__global__ void __launch_bounds__(kCellThreads, 1) forward_cells_kernel(const ForwardParams p)
+{
+    extern __shared__ __align__(128) unsigned char dsm_c[];
+    __shared__ __align__(8) unsigned long long s_bar;
+    __shared__ LayerDesc s_L;
+    __shared__ CellGrid s_GA, s_GB;
+    __shared__ __align__(16) float s_pf[param_count(DM)];
+    __shared__ __align__(16) double s_pd[param_count(DM)];
+    __shared__ float s_near[kCellNearStride];
+    __shared__ int s_abort;
+    const int tid = threadIdx.x;
+    const uint32_t bar = smem_u32(&s_bar);
+    uint32_t* hist = reinterpret_cast<uint32_t*>(dsm_c + p.smem_grid_bytes);
+    if (tid == 0) {
+        mbar_init(bar, 1);
+        fence_proxy_async();
+        s_abort = 0;
+    }
+    __syncthreads();
+    const long long lo = p.total_items * blockIdx.x / gridDim.x, hi = p.total_items * (blockIdx.x + 1) / gridDim.x;
+    uint32_t phase = 0;
+    int k = -1;
+    long long ibeg = 0, iend = 0;
+    bool hist_live = false;
+    const unsigned char* smB = dsm_c;
+    auto flush = [&]() {
+        const int ent = s_L.NA * s_L.NB;
+        for (int e = tid; e < ent; e += (int)blockDim.x) {
+            const uint32_t v = hist[e];
+            if (v) count_add(p.counts, p.counts_u32, s_L.coff + e, v);
+        }
+    };
+    for (long long item = lo; item < hi; ++item) {
+        if (k < 0 || item >= iend) {
+            __syncthreads();
+            if (hist_live) flush();
+            // the layer, then its descriptors, word by word (one round trip to L2)
+            if (p.cell_ipl > 0) k = (int)(item / p.cell_ipl);
+            else k = p.cell_g0;
+            __syncthreads();
+            for (int e = tid; e < (int)(sizeof(LayerDesc) / 4); e += (int)blockDim.x)
+                reinterpret_cast<int*>(&s_L)[e] = reinterpret_cast<const int*>(p.layers + k)[e];
+            for (int e = tid; e < (int)(sizeof(CellGrid) / 4); e += (int)blockDim.x) {
+                reinterpret_cast<int*>(&s_GA)[e] = reinterpret_cast<const int*>(p.cells + k)[e];
+                reinterpret_cast<int*>(&s_GB)[e] = reinterpret_cast<const int*>(p.cells + k + 1)[e];
+            }
+            if (p.source == kSampler) {
+                for (int e = tid; e < param_count(DM); e += (int)blockDim.x) {
+                    s_pf[e] = p.params_f[(long long)k * p.params_stride + e];
+                    s_pd[e] = p.params_d[(long long)k * p.params_stride + e];
+                }
+                if (MODE == 1 && tid < kCellNearStride) s_near[tid] = p.cell_near[k * kCellNearStride + tid];
+            }
+            __syncthreads();
+            if (tid == 0) {
+                const uint32_t ba = cell_stage_bytes<DM>(s_GA), bb = cell_stage_bytes<DM>(s_GB);
+                fence_proxy_async();
+                mbar_arrive_expect_tx(bar, ba + bb);
+                cell_stage<DM>(p, s_GA, smem_u32(dsm_c), bar);
+                cell_stage<DM>(p, s_GB, smem_u32(dsm_c) + ba, bar);
+            }
+            ibeg = s_L.item_begin;
+            iend = ibeg + s_L.items;
+            hist_live = s_L.hist_smem != 0;
+            if (hist_live)
+                for (int e = tid; e < s_L.NA * s_L.NB; e += (int)blockDim.x) hist[e] = 0;
+            if (!mbar_wait_bounded(bar, phase, p.spin_budget)) {
+                record_error(p.status, 4 /* QT_ETIMEOUT */, 50);
+                s_abort = 1;
+                mbar_wait_bounded(bar, phase, kDrainUs);
+            }
+            phase ^= 1u;
+            __syncthreads();
+            if (s_abort) return;
+            smB = dsm_c + cell_stage_bytes<DM>(s_GA);
+        }
+        const unsigned long long m = (unsigned long long)(item - ibeg) * blockDim.x + (unsigned long long)tid;
+        if (m >= p.M) continue;
+        // ---- the centred pair
+        float a[DM], b[DM], f = 1.0f;
+        if constexpr (MODE == 0) {
+            float X[DM], Y[DM];
+            pair_f32<DM>(s_pf, DM, p.seed, k, m, X, Y);
+#pragma unroll
+            for (int l = 0; l < DM; ++l) {
+                a[l] = __fsub_rn(X[l], s_GA.mu[l]);
+                b[l] = __fsub_rn(Y[l], s_GB.mu[l]);
+            }
+        } else if constexpr (MODE == 1) {
+            f = pair_near<DM>(s_near, p.seed, k, m, a, b);
+        } else {
+#pragma unroll
+            for (int l = 0; l < DM; ++l) {
+                a[l] = __double2float_rn(__dsub_rn(p.srcX[m * DM + l], (double)s_GA.mu[l]));
+                b[l] = __double2float_rn(__dsub_rn(p.srcY[m * DM + l], (double)s_GB.mu[l]));
+            }
+        }
+        // ---- both cells
+        int i = 0, j = 0;
+        uint64_t eA, eB;
+        bool needA = false, needB = false;
+        if (s_L.NA > 1)
+            i = cell_search<DM>(s_GA, dsm_c, p.cell_pool, a, MODE == 1 ? __fmaf_rn(f, 1.0f - s_GA.f0, s_GA.f0) : 1.0f, eA,
+                                needA);
+        if (s_L.NB > 1)
+            j = cell_search<DM>(s_GB, smB, p.cell_pool, b, MODE == 1 ? __fmaf_rn(f, 1.0f - s_GB.f0, s_GB.f0) : 1.0f, eB,
+                                needB);
+        if (needA) i = cell_recheck<DM>(p, s_pf, s_pd, k, m, false, eA, s_GA);
+        if (needB) j = cell_recheck<DM>(p, s_pf, s_pd, k, m, true, eB, s_GB);
+        // ---- counters p^k_ij (Sec. 3.3), per-sample cells, dumps
+        if (hist_live) atomicAdd(&hist[i * s_L.NB + j], 1u);
+        else count_add(p.counts, p.counts_u32, s_L.coff + (long long)i * s_L.NB + j, 1u);
+        if (MODE == 2 && p.cellsA) {
+            p.cellsA[m] = i;
+            p.cellsB[m] = j;
+        }
+        if (p.dump_count > 0 && (m % (unsigned long long)p.dump_stride) == 0ull) {
+            const unsigned long long t = m / (unsigned long long)p.dump_stride;
+            if (t < (unsigned long long)p.dump_count) {
+                const long long row = (long long)k * p.dump_count + (long long)t;
+                double z[DM];
+                exact_sample<DM>(p, s_pf, s_pd, k, m, false, z);
+                for (int l = 0; l < DM; ++l) p.dumpX[row * DM + l] = z[l];
+                exact_sample<DM>(p, s_pf, s_pd, k, m, true, z);
+                for (int l = 0; l < DM; ++l) p.dumpY[row * DM + l] = z[l];
+                p.dumpI[row] = i;
+                p.dumpJ[row] = j;
+            }
+        }
+    }
+    __syncthreads();
+    if (hist_live) flush();
+}
+
+cudaError_t launch_build_cells(int dm, const ForwardParams& p, int num_sms, cudaStream_t st)
+{
+    const int ng = p.cell_g1 - p.cell_g0;
+    // one patch per warp where there are few grids, about eight CTAs of eight warps
+    // per SM where there are many
+    const int most = dm == 1 ? 8192 / 32 / kBuildWarps : 104 * 104 / 32 / kBuildWarps + 1;
+    const int slices = (8 * num_sms + ng - 1) / ng;
+    dim3 grid((unsigned)ng, (unsigned)(slices < 1 ? 1 : (slices > most ? most : slices)));
+    if (dm == 1) build_cells_kernel<1><<<grid, kBuildThreads, 0, st>>>(p);
+    else build_cells_kernel<2><<<grid, kBuildThreads, 0, st>>>(p);
+    return cudaGetLastError();
+}
+
+template <int DM, int MODE>
+static cudaError_t launch_fc(const ForwardParams& p, int dyn, int num_sms, int* bps, cudaStream_t st)
+{
+    auto kern = forward_cells_kernel<DM, MODE>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    if (e != cudaSuccess) return e;
+    *bps = 1;
+    long long grid = num_sms;
+    if (grid > p.total_items) grid = p.total_items;
+    if (grid < 1) grid = 1;
+    kern<<<(unsigned)grid, (unsigned)p.tile, dyn, st>>>(p);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_forward_cells(int dm, const ForwardParams& p, int dyn, int num_sms, int* bps, cudaStream_t st)
+{
+    const int mode = p.source == kArrays ? 2 : (p.prec == 1 ? 0 : 1);
+#define QT_CASE(D, M) \
+    if (dm == D && mode == M) return launch_fc<D, M>(p, dyn, num_sms, bps, st);
+    QT_CASE(1, 0) QT_CASE(1, 1) QT_CASE(1, 2) QT_CASE(2, 0) QT_CASE(2, 1) QT_CASE(2, 2)
+#undef QT_CASE
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace qt

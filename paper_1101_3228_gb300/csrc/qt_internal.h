@@ -8,7 +8,11 @@ constexpr int kDMax = 16;          // largest state dimension
 constexpr int kChunk = 16;         // candidates per min-tracking chunk of the FP32 screen
 constexpr int kSlots = 2;          // ring slots of the streamed-grid mode
 
-enum Form : int32_t { kPlainF64 = 1, kF32Recheck = 2, kTcRecheck = 3, kRouterCert = 4, kPathwise = 5 };
+enum Form : int32_t {
+    kPlainF64 = 1, kF32Recheck = 2, kTcRecheck = 3, kRouterCert = 4, kPathwise = 5,
+    kCells = 6,                    // located search (d <= 2), Algorithm III and given samples
+    kPathCells = 7                 // located search, Algorithm II
+};
 enum Source : int32_t { kSampler = 0, kArrays = 1 };
 
 // Per-layer sampler parameters packed by the host: m[d], b[d], L[d*d], A[d*d],
@@ -25,6 +29,8 @@ struct DevStatus {
     unsigned long long candidates; // candidate distances (router form)
     unsigned long long done_items; // work items finished
     unsigned long long spare[4];   // [0]: router grid checksum; [1..3]: diagnostics
+    uint32_t cell_cursor;          // located search: pool words taken by the tables
+    uint32_t pad;
 };
 
 // One layer pair (k, k+1) of the forward step.
@@ -51,6 +57,27 @@ struct GridInfo {
     int32_t tc_tiles;              // tensor-core form: 256-point operand tiles of this grid
     long long tc_toff;             // tensor-core form: first tile of this grid
 };
+
+// One grid of the located search (d <= 2): sizes and places from the host, the
+// box, scales and certificate constants from build_cells_kernel.
+struct alignas(16) CellGrid {
+    float inv_h[2];                // bins per unit length
+    float org[2];                  // 2^23 + number of the bin centred on 0
+    float mu[2];                   // centre (FP32)
+    float c1, c2, c3;              // certificate: 2 err(D) = f (c1 D + c2) + c3 D, 0 < f <= 1
+    float f0;                      // the part of f that is the FP32 rounding of the points
+    float inv_span;                // 1 / S, S = |farthest corner of the box| + R
+    float err;                     // bound of the centred samples' error per coordinate beyond FP32 rounding
+    int32_t N, nb0, nb1;           // points, bins along each axis (nb1 = 1 for d = 1)
+    int32_t pad;
+    long long goff;                // first point in the FP64 grids
+    long long toff;                // first entry of the table
+    long long roff;                // first float of the FP32 records
+};
+
+constexpr int kCellMaxN = 1024;    // points of a grid: ten bits per index
+constexpr int kCellThreads = 1024; // most threads of the located-search kernels
+constexpr int kCellNearStride = 20;// floats of a layer's combined FP32 parameters (d <= 2)
 
 constexpr int kTcTileN = 256;      // grid points per tensor-core operand tile (MMA N)
 constexpr int kTcTileM = 128;      // samples per tensor-core work item (MMA M)
@@ -122,6 +149,17 @@ struct ForwardParams {
     long long item_lo, item_hi;    // tensor-core form: work items [item_lo, item_hi) of this launch
     int32_t tc_draw_in;            // tensor-core form: 1 = the screen kernel draws its samples
     unsigned char* tc_items;       // tensor-core form, draw pass: samples of the launch's items
+    // located search (d <= 2)
+    CellGrid* cells;               // [n+1]
+    unsigned long long* cell_tab;  // bin entries of every grid
+    float* cell_rec;               // centred FP32 points of every grid
+    uint16_t* cell_pool;           // candidate lists longer than an entry
+    uint32_t* cell_cursor;         // pool words taken
+    uint32_t cell_pool_cap;        // pool words
+    int32_t cell_g0, cell_g1;      // grids [g0, g1) to build
+    const float* cell_near;        // [n][kCellNearStride] combined FP32 parameters of FP64 layers
+    long long cell_tile;           // path-wise form: paths per work item
+    long long cell_ipl;            // work items of every layer (0: only one layer has any)
     // learned router + Elkan certificate
     const float* rt_params;        // MLP parameters, packed W1, b1, W2, b2, W3, b3
     const float* rt_linv;          // [n+1][d][d] FP32 inverse Cholesky factors (whitening)

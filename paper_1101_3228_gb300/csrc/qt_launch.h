@@ -30,6 +30,10 @@ bool pathwise_variant_exists(int dm, int S, bool f32, bool streamed);
 int pathwise_default_spt(int dm, bool f32, bool streamed, long long M, long long ctas);
 cudaError_t launch_pathwise(int dm, int S, bool f32, bool streamed, const ForwardParams& p, int dyn, int num_sms,
                             int* bps, cudaStream_t st);
+// located search (d <= 2): table building, then Algorithm III / given samples or Algorithm II
+cudaError_t launch_build_cells(int dm, const ForwardParams& p, int num_sms, cudaStream_t st);
+cudaError_t launch_forward_cells(int dm, const ForwardParams& p, int dyn, int num_sms, int* bps, cudaStream_t st);
+cudaError_t launch_path_cells(int dm, int S, const ForwardParams& p, int dyn, int num_sms, int* bps, cudaStream_t st);
 cudaError_t launch_f32_streamed(int dm, int S, const ForwardParams& p, int block, int dyn, int num_sms, int* bps,
                                 cudaStream_t st);
 

@@ -1,0 +1,172 @@
+"""The located search of d <= 2 (the automatic form's tables of candidate points)
+against the oracle, at the sizes where a table or a launch can go wrong: one-point
+and two-point grids, patches and inline lists filled and overflowing, ties, samples
+outside the tables' box, grids with no usable table, ragged tiles, both sample
+precisions, Algorithm II.  Counts and cells are compared bit for bit.
+"""
+import os
+import subprocess
+import tempfile
+
+import numpy as np
+import pytest
+
+import oracle
+import qt_workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def B(gpu_lib):
+    from paper_1101_3228_gb300 import binding
+    return binding
+
+
+@pytest.fixture(scope="module")
+def ctx(B):
+    c = B.Context(0)
+    yield c
+    c.close()
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def _run_program(name, *flags):
+    from paper_1101_3228_gb300.build import CSRC, _nvcc
+    with tempfile.TemporaryDirectory() as tmp:
+        exe = os.path.join(tmp, name)
+        subprocess.run([_nvcc(), "-gencode", "arch=compute_103a,code=sm_103a", "-O2", "-std=c++17",
+                        "--expt-relaxed-constexpr", "-I", CSRC, os.path.join(HERE, "cuda", name + ".cu"), "-o", exe],
+                       check=True)
+        return subprocess.run([exe], check=True, capture_output=True, text=True, timeout=120).stdout.split()
+
+
+def test_near_normals_within_their_bound():
+    """The certificate allows 1.375 2^-20 of the radius, and radii up to 8.6."""
+    out = _run_program("near_normals")
+    val = {out[i]: float(out[i + 1]) for i in range(1, len(out), 2)}
+    assert 0.0 < val["max_error"] < 1.0 and val["max_radius"] < 8.6 and val["max_radius_error"] < 1.0, val
+
+
+def _chain(d, n, Ns, M, scale=1.0, shift=0.0, seed=5):
+    rng = np.random.default_rng(seed)
+    A = np.repeat((0.9 * np.eye(d) + 0.05 * np.tri(d, k=-1).T)[None], n, 0)
+    T = np.repeat((scale * 0.3 * (np.eye(d) + 0.2 * np.tri(d, k=-1)))[None], n, 0)
+    L = np.concatenate([np.zeros((1, d, d)), np.repeat((scale * (np.eye(d) - 0.4 * np.tri(d, k=-1)))[None], n, 0)])
+    m = np.full((n + 1, d), shift)
+    b = np.repeat((shift - A[0] @ np.full(d, shift))[None], n, 0)
+    N = np.array([1] + list(Ns), dtype=np.int64)
+    g = np.concatenate([m[:1]] + [shift + scale * rng.standard_normal((k, d)) * 1.2 for k in Ns])
+    return W.Model("chain", d, n, N, A, b, T, m, L, np.arange(n + 1.0), 0.0, "put_exp1d", 1.0, None, M, 99,
+                   W.PREC_F32, "kmeans"), g
+
+
+@pytest.mark.parametrize("d", [1, 2])
+@pytest.mark.parametrize("prec", [W.PREC_F32, W.PREC_F64])
+@pytest.mark.parametrize("Ns,M", [((2, 3, 1, 64), 257), ((100, 101), 1025), ((500, 37), 20011), ((1023, 1024), 3001),
+                                  ((1024, 1025), 777)])
+def test_located_counts_bit_exact(ctx, B, d, prec, Ns, M):
+    model, g = _chain(d, len(Ns), Ns, M)
+    ref = oracle.transitions(model, g, M, model.seed, prec)
+    for ct in (B.COUNTS_I64, B.COUNTS_U32):
+        counts, st, dump = ctx.transitions(model, _dev(g), M, model.seed, B.options(prec=prec, counts_type=ct),
+                                           dump_count=50, dump_stride=7)
+        got = B.split_counts(model.N, counts.cpu().numpy().astype(np.int64))
+        for k in range(model.n):
+            np.testing.assert_array_equal(got[k], ref[k], err_msg=f"layer {k}")
+        assert st.form_used == B.FORM_F32_RECHECK and st.device_status == 0
+    off = model.offsets()
+    ok = dump["i"][-1].cpu().numpy() >= 0
+    X, Y = (dump[v][-1].cpu().numpy()[ok] for v in "XY")
+    np.testing.assert_array_equal(dump["i"][-1].cpu().numpy()[ok], oracle.nearest(g[off[-3]:off[-2]], X))
+    np.testing.assert_array_equal(dump["j"][-1].cpu().numpy()[ok], oracle.nearest(g[off[-2]:off[-1]], Y))
+
+
+@pytest.mark.parametrize("prec", [W.PREC_F32, W.PREC_F64])
+@pytest.mark.parametrize("scale,shift", [(1e-3, 5.0), (1e3, 0.0), (1e-6, 100.0)])
+def test_located_counts_over_scales(ctx, B, prec, scale, shift):
+    """Grids far from the origin: the last one leaves no usable table for FP32 samples
+    (their spacing there is coarser than the bins)."""
+    for d in (1, 2):
+        model, g = _chain(d, 2, (150, 90), 4001, scale, shift)
+        ref = oracle.transitions(model, g, model.M, model.seed, prec)
+        counts, _, _ = ctx.transitions(model, _dev(g), model.M, model.seed, B.options(prec=prec))
+        got = B.split_counts(model.N, counts.cpu().numpy())
+        for k in range(model.n):
+            np.testing.assert_array_equal(got[k], ref[k], err_msg=f"d {d} layer {k}")
+
+
+@pytest.mark.parametrize("d", [1, 2])
+@pytest.mark.parametrize("kind", ["ties", "cluster", "line", "same", "outside"])
+def test_located_cells_of_given_samples(ctx, B, d, kind):
+    rng = np.random.default_rng(3)
+    gA = rng.standard_normal((300, d))
+    gB = 1.2 * rng.standard_normal((317, d))
+    X, Y = rng.standard_normal((4001, d)), rng.standard_normal((4001, d))
+    if kind == "ties":
+        gA = np.round(gA * 8) / 8                    # dyadic: exact ties and duplicates
+        X = np.round(X * 16) / 16
+        Y[:2000] = W.boundary_samples(gB, 2000, seed=4, jitter=1e-9)
+    elif kind == "cluster":
+        gA[10:] = 1e-4 * gA[10:]                     # hundreds of points in one bin
+        X[::2] *= 1e-4
+        gB[5:] = gB[5] + 1e-9 * rng.standard_normal((312, d))
+    elif kind == "line":
+        gA[:, -1] = 0.25                             # no extent along the last axis
+        X[::3, -1] = 0.25
+    elif kind == "same":
+        gA[:] = gA[0]
+    else:
+        X *= 50.0
+        Y[7] = 1e30
+        X[5] = -1e18
+    for ct in (B.COUNTS_I64, B.COUNTS_U32):
+        counts, st, ii, jj = ctx.counts_from_samples(_dev(gA), _dev(gB), _dev(X), _dev(Y), B.options(counts_type=ct),
+                                                     want_cells=True)
+        np.testing.assert_array_equal(ii.cpu().numpy(), oracle.nearest(gA, X))
+        np.testing.assert_array_equal(jj.cpu().numpy(), oracle.nearest(gB, Y))
+        np.testing.assert_array_equal(counts.cpu().numpy(), oracle.counts_from_samples(gA, gB, X, Y))
+    if kind == "ties":
+        assert st.rechecks > 100
+
+
+@pytest.mark.parametrize("prec", [W.PREC_F32, W.PREC_F64])
+@pytest.mark.parametrize("M", [1, 33, 20011, 300007])
+def test_located_paths_bit_exact(ctx, B, prec, M):
+    """Algorithm II: few paths (one per thread), several per thread, the Euler chain."""
+    n = 3 if M > 10**5 else 5
+    for d in (1, 2):
+        model, g = _chain(d, n, [60, 1, 200, 33, 90][:n], M)
+        for euler in (None, (np.full((n, d), 0.5), np.full((n, d), 0.3))):
+            ref = oracle.pathwise(model, g, M, model.seed, prec, euler=euler)
+            ref = ref[0] if isinstance(ref, tuple) else ref
+            counts, _, _ = ctx.transitions_pathwise(model, _dev(g), M, model.seed, B.options(prec=prec), euler=euler)
+            got = B.split_counts(model.N, counts.cpu().numpy())
+            for k in range(n):
+                np.testing.assert_array_equal(got[k], ref[k], err_msg=f"d {d} layer {k}")
+
+
+def test_located_fused_price_and_timeouts(ctx, B):
+    """One layer at a time (the fused price), a wait that gives up in either kernel, and
+    alternating calls on one context (direct launches, then a captured step)."""
+    model, g = _chain(2, 3, (80, 120, 60), 5003)
+    phi = np.maximum(1.0 - np.exp(g.sum(1)), 0.0)
+    ref = oracle.price(model.N, oracle.transitions(model, g, model.M, model.seed, W.PREC_F32), phi)
+    other, g2 = _chain(1, 2, (70, 50), 3001, seed=8)
+    phi2 = np.maximum(1.0 - np.exp(g2[:, 0]), 0.0)
+    ref2 = oracle.price(other.N, oracle.transitions(other, g2, other.M, other.seed, W.PREC_F32), phi2)
+    for flags in (0, B.FLAG_FUSED_BACKWARD, B.FLAG_NO_GRAPH, 0, 0, 0):
+        for mdl, gr, ph, want in ((model, g, phi, ref), (other, g2, phi2, ref2)):
+            for _ in range(3 if flags == 0 else 1):
+                price, st = ctx.price(mdl, gr, mdl.M, mdl.seed, ph, B.options(flags=flags))
+                assert abs(price - want) <= 1e-12 * max(abs(want), 1e-300)
+    for call in (ctx.transitions, ctx.transitions_pathwise):
+        with pytest.raises(B.QtError) as e:
+            call(model, _dev(g), model.M, model.seed, B.options(spin_budget=-1))
+        assert e.value.status == B.QT_ETIMEOUT
+        call(model, _dev(g), model.M, model.seed)
