@@ -23,11 +23,9 @@ __device__ __forceinline__ void normals_range_f32(uint64_t seed, int k, uint64_t
             for (int pair = 0; pair < 2; ++pair) {
                 const int q = 4 * r + 2 * pair;
                 if (q + 2 > lo && q < hi) {
-                    const float u0 = uniform_f32(w.v[2 * pair]);
-                    const float u1 = uniform_f32(w.v[2 * pair + 1]);
-                    const float rad = __fsqrt_rn(__fmul_rn(-2.0f, ln_f32(u0)));
+                    const float rad = sqrt_mid(__fmul_rn(-2.0f, ln_f32(uniform_f32(w.v[2 * pair]))));
                     float sn, cs;
-                    sincos2pi_f32(u1, sn, cs);
+                    sincos2pi_word(w.v[2 * pair + 1], sn, cs);
                     if (q < CNT) g[q] = __fmul_rn(rad, cs);
                     if (q + 1 < CNT) g[q + 1] = __fmul_rn(rad, sn);
                 }

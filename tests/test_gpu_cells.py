@@ -53,6 +53,12 @@ def test_near_normals_within_their_bound():
     assert 0.0 < val["max_error"] < 1.0 and val["max_radius"] < 8.6 and val["max_radius_error"] < 1.0, val
 
 
+def test_sampler_operations_are_the_ieee_ones():
+    """Uniform, logarithm, radius, sine and cosine for all 2^23 FP32 uniforms, bit for bit."""
+    out = _run_program("sampler_exact")
+    assert [int(v) for v in out[3::2]] == [0] * 5, out
+
+
 def _chain(d, n, Ns, M, scale=1.0, shift=0.0, seed=5):
     rng = np.random.default_rng(seed)
     A = np.repeat((0.9 * np.eye(d) + 0.05 * np.tri(d, k=-1).T)[None], n, 0)
