@@ -31,7 +31,7 @@ __global__ void kmeans_assign_kernel(int, long long, const float*, int, const fl
                                      unsigned long long*, int);
 __global__ void kmeans_update_kernel(int, int, const unsigned long long*, const unsigned long long*, float*);
 __global__ void map_grid_kernel(int, int, const double*, const double*, const double*, double*);
-__global__ void prep_tc_tiles_kernel(const float*, GridInfo*, int, int, int, int, int, long long, __half*);
+__global__ void prep_tc_tiles_kernel(const float*, GridInfo*, int, int, int, int, int, long long, __half*, float*);
 cudaError_t launch_router_forward(int dm, const ForwardParams& p, int num_sms, int* bps, cudaStream_t st);
 cudaError_t launch_grid_checksum(const double* grids, long long count, unsigned long long* out, cudaStream_t st);
 void router_fill_params(const qt_router* r, ForwardParams& fp);
@@ -319,16 +319,16 @@ struct Plan {
     int form = 0, dm = 0, S = 0, block = 256;
     bool streamed = false;
     int seg_records = 0;
-    int tc_k = 0, tc_slots = 0, tc_resident = 0;
+    int tc_k = 0, tc_slots = 0;
     long long tc_total_tiles = 0;
     long long tc_chunk_items = 0;      // tensor-core form: work items per launch
-    int tc_draw_in = 0;                // tensor-core form: 1 = the screen kernel draws its samples
-    size_t tc_item_bytes = 0;          // tensor-core form: drawn-sample bytes per work item
+    size_t tc_item_bytes = 0;          // tensor-core form: record bytes per work item
     int d = 0, n = 0, ngrids = 0;
     int euler = 0;                     // path-wise form: Euler-scheme chain
     long long total_recs = 0;
     size_t grid_bytes = 0, hist_bytes = 0, dyn_smem = 0;
     long long total_items = 0;
+    int only_layer = -1;               // the one layer with work items, or -1
     int tile = 0;
     int rec_floats = 0, rec64 = 0, pstride = 0;
     std::vector<LayerDesc> layers;
@@ -426,13 +426,15 @@ bool cells_apply(size_t smem, int d, int n, const int64_t* Ns, const qt_options*
     return total <= (1ull << 30) && pair + 16 * 1024 <= smem;
 }
 
-// Work items per launch of the tensor-core form: all of them when the screen
-// kernel draws its own samples, as many as 2 GiB of drawn samples hold with the
-// draw pass, or fewer when the caller caps it.
+// Tensor-core form: the FP16 operand tiles, then the chunk-major FP32 records.
+size_t tc_tile_bytes(const Plan& P) { return (size_t)P.tc_total_tiles * kTcTileN * P.tc_k * 2; }
+float* tc_rows_of(const Plan& P, void* tiles) { return (float*)((unsigned char*)tiles + tc_tile_bytes(P)); }
+
+// Work items per window of the tensor-core form: as many as 1 GiB of records holds,
+// or fewer when the caller caps it.
 long long tc_chunk(const Plan& P, const qt_options* o)
 {
-    long long c = P.total_items;
-    if (!P.tc_draw_in) c = std::min<long long>(c, (2ll << 30) / (long long)P.tc_item_bytes);
+    long long c = std::min<long long>(P.total_items, (1ll << 30) / (long long)P.tc_item_bytes);
     if (o->tc_chunk_items > 0) c = std::min<long long>(c, o->tc_chunk_items);
     return std::max<long long>(1, c);
 }
@@ -448,6 +450,7 @@ qt_status make_plan(qt_ctx* ctx, int d, int n, const int64_t* Ns, const double* 
     if (!s && algo == 2 && only_layer >= 0) return fail(ctx, QT_EUNSUPPORTED, "the path-wise form runs every layer");
     if (s || only_layer < 0) return s;
     if (only_layer >= n) return fail(ctx, QT_EINVAL, "layer %d of %d", only_layer, n);
+    P.only_layer = only_layer;
     const int items = P.layers[only_layer].items;
     for (int k = 0; k < n; ++k) {
         P.layers[k].item_begin = k <= only_layer ? 0 : items;
@@ -678,29 +681,20 @@ qt_status make_plan_full(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
         return QT_OK;
     }
     if (P.form == kTcRecheck) {
-        // one CTA of 16 warps per SM owns the 512 TMEM columns (four 128-column
-        // accumulators); the operand tiles take what the pipeline's buffers
-        // leave of the shared memory, at most 16 tiles
+        // four CTAs share an SM, each a quarter of its shared memory at most: the
+        // operand tiles take what the samples leave, up to kTcMaxSlots
         P.tc_k = P.dm <= 4 ? 16 : 32;
         const size_t tile_bytes = (size_t)kTcTileN * P.tc_k * 2;
         const long long fixed = tc_fixed_smem(P.dm, P.tc_k);
-        const long long room = (long long)ctx->smem_optin - fixed - 2048;
+        const long long room = ((long long)ctx->smem_optin + 1024) / kTcCtas - 2048 - fixed;
         P.tc_slots = (int)std::min<long long>(kTcMaxSlots, room > 0 ? room / (long long)tile_bytes : 0);
         if (P.tc_slots < 2) return fail(ctx, QT_EUNSUPPORTED, "too little shared memory for the tensor-core form");
-        int tmax = 0;
-        for (int k = 0; k < n; ++k) tmax = std::max(tmax, P.grids[k].tc_tiles + P.grids[k + 1].tc_tiles);
-        P.tc_resident = tmax <= P.tc_slots;
-        // resident tiles take only the slots they need: the rest of the unified
-        // L1/shared memory caches the FP32 records that the certifiers re-score
-        if (P.tc_resident) P.tc_slots = std::max(2, tmax);
         P.S = 1;
         P.block = kTcThreads;
         P.tile = kTcTileM;
-        // where the samples are drawn: the caller's choice, else the autotuned
-        // one (the caller passes it through tc_draw), else in the screen kernel
-        P.tc_draw_in = o->tc_draw != 1;
-        P.tc_item_bytes = (size_t)(tc_item_op_bytes(P.tc_k) + tc_item_cert_bytes(P.dm));
-        P.grid_bytes = (size_t)fixed + (size_t)P.tc_slots * tile_bytes;
+        P.tc_item_bytes = (size_t)tc_item_bytes(P.dm);
+        // more than a fifth, so that a fifth CTA never waits for tensor memory
+        P.grid_bytes = std::max((size_t)fixed + (size_t)P.tc_slots * tile_bytes, (ctx->smem_optin + 1024) / 5);
         P.hist_bytes = 0;
         P.dyn_smem = P.grid_bytes;
         P.layers.resize(n);
@@ -844,15 +838,16 @@ qt_status enqueue_forward(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long
     if (P.form == kTcRecheck) {
         const long long rows = P.tc_total_tiles * kTcTileN;
         prep_tc_tiles_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(
-            (const float*)drec32, (GridInfo*)dgrids, P.ngrids, P.d, P.dm, P.rec_floats, P.tc_k, rows, (__half*)dtiles);
+            (const float*)drec32, (GridInfo*)dgrids, P.ngrids, P.d, P.dm, P.rec_floats, P.tc_k, rows, (__half*)dtiles,
+            tc_rows_of(P, dtiles));
         QT_CUDA(cudaGetLastError());
     }
     ForwardParams fp;
     memset(&fp, 0, sizeof fp);
     fp.tc_tiles = dtiles;
+    fp.tc_rows = P.form == kTcRecheck ? tc_rows_of(P, dtiles) : nullptr;
     fp.tc_k = P.tc_k;
     fp.tc_slots = P.tc_slots;
-    fp.tc_resident = P.tc_resident;
     fp.d = P.d;
     fp.n = P.n;
     fp.form = P.form;
@@ -921,21 +916,15 @@ qt_status enqueue_forward(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long
     const unsigned evflags = stream_is_capturing(st) ? cudaEventRecordExternal : cudaEventRecordDefault;
     QT_CUDA(cudaEventRecordWithFlags(ctx->ev_k0, st, evflags));
     if (P.form == kTcRecheck) {
-        // one launch over every work item (or one per window when capped); with
-        // the draw-pass layout each window's samples are drawn first
-        fp.tc_draw_in = P.tc_draw_in;
+        // draw, screen and certificate, window by window
         fp.tc_items = (unsigned char*)dtcitems;
+        fp.tc_ipl = P.only_layer < 0 ? P.layers[0].items : 0;
         for (long long lo = 0; lo < P.total_items; lo += P.tc_chunk_items) {
             fp.item_lo = lo;
             fp.item_hi = std::min(P.total_items, lo + P.tc_chunk_items);
-            cudaError_t e = cudaSuccess;
-            if (!P.tc_draw_in) {
-                e = launch_tc_draw(P.dm, fp, st);
-                if (e != cudaSuccess) return fail(ctx, QT_ECUDA, "draw pass launch: %s", cudaGetErrorString(e));
-            }
-            e = forward_launch(P.form, P.dm, P.S, P.streamed, fp, P.block, (int)P.dyn_smem, ctx->num_sms,
-                               &blocks_per_sm, st);
-            launches += P.tc_draw_in ? 1 : 2;
+            cudaError_t e = forward_launch(P.form, P.dm, P.S, P.streamed, fp, P.block, (int)P.dyn_smem, ctx->num_sms,
+                                           &blocks_per_sm, st);
+            launches += 3;
             if (e != cudaSuccess) return fail(ctx, QT_ECUDA, "forward kernel launch: %s", cudaGetErrorString(e));
         }
     } else {
@@ -947,7 +936,7 @@ qt_status enqueue_forward(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long
     QT_CUDA(cudaEventRecordWithFlags(ctx->ev_k1, st, evflags));
     ctx->timed = true;
     ctx->last_launches = launches;
-    ctx->last_tc_draw = P.form == kTcRecheck ? (P.tc_draw_in ? 2 : 1) : 0;
+    ctx->last_tc_draw = P.form == kTcRecheck ? 1 : 0;
     return QT_OK;
 }
 
@@ -1053,9 +1042,8 @@ qt_status run_plan(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long M, uns
     void* dtiles = nullptr;
     void* dtcitems = nullptr;
     if (P.form == kTcRecheck &&
-        ((s = dev_get(ctx, (tag + "tctiles").c_str(), (size_t)P.tc_total_tiles * kTcTileN * P.tc_k * 2, &dtiles)) ||
-         (!P.tc_draw_in &&
-          (s = dev_get(ctx, (tag + "tcitems").c_str(), (size_t)P.tc_chunk_items * P.tc_item_bytes, &dtcitems)))))
+        ((s = dev_get(ctx, (tag + "tctiles").c_str(), tc_tile_bytes(P) + (size_t)P.tc_total_tiles * kTcTileN * (P.dm + 1) * 4, &dtiles)) ||
+         (s = dev_get(ctx, (tag + "tcitems").c_str(), (size_t)P.tc_chunk_items * P.tc_item_bytes, &dtcitems))))
         return s;
     ctx->status_buf = (unsigned char*)dtables + T.status;
 
@@ -1206,76 +1194,6 @@ qt_status autotune(qt_ctx* ctx, int d, int n, const int64_t* Ns, const double* m
     return QT_OK;
 }
 
-// Autotuner of the tensor-core form: time both sample-draw layouts (a separate
-// draw pass, or the screen kernel drawing its own samples) on the widest window
-// of up to four consecutive layer pairs with up to 2^20 samples each (best of
-// three runs), keep the faster for the key.
-qt_status autotune_tc(qt_ctx* ctx, int d, int n, const int64_t* Ns, const double* mus, const double* params_d_host,
-                      long long M, unsigned long long seed, const qt_options* o, int source, const FwdIO& io,
-                      const Plan& base, const TuneKey& key, cudaStream_t st)
-{
-    const int n2 = std::min(n, 4);
-    int k0 = 0;
-    long long wbest = -1;
-    for (int k = 0; k + n2 <= n; ++k) {
-        long long w = 0;
-        for (int q = k; q < k + n2; ++q) w += Ns[q] + Ns[q + 1];
-        if (w > wbest) {
-            wbest = w;
-            k0 = k;
-        }
-    }
-    Ns += k0;
-    mus += (long long)k0 * d;
-    if (params_d_host) params_d_host += (long long)k0 * base.pstride;
-    const long long M2 = std::min<long long>(M, 1ll << 20);
-    long long ent = 0;
-    for (int k = 0; k < n2; ++k) ent += Ns[k] * Ns[k + 1];
-    void* tcounts;
-    qt_status s = dev_get(ctx, "tune.counts", (size_t)ent * 8, &tcounts);
-    if (s) return s;
-    FwdIO tio = io;
-    tio.counts = tcounts;
-    tio.dump = nullptr;
-    tio.cellsA = tio.cellsB = nullptr;
-    cudaEvent_t e0, e1;
-    QT_CUDA(cudaEventCreate(&e0));
-    QT_CUDA(cudaEventCreate(&e1));
-    float best = 1e30f;
-    int bestv = 2;
-    for (int v = 1; v <= 2; ++v) {
-        qt_options to = *o;
-        to.tc_draw = v;
-        to.tc_chunk_items = 0;
-        to.counts_type = QT_COUNTS_I64;
-        to.flags |= QT_FLAG_NO_TUNE;
-        Plan P;
-        if (make_plan(ctx, d, n2, Ns, mus, M2, &to, source == kArrays, P) != QT_OK) continue;
-        float fastest = 1e30f;
-        for (int rep = 0; rep < 4; ++rep) {
-            QT_CUDA(cudaEventRecord(e0, st));
-            if ((s = run_plan(ctx, P, tio, M2, seed, &to, source, params_d_host, st, false, "tune."))) {
-                cudaEventDestroy(e0);
-                cudaEventDestroy(e1);
-                return s;
-            }
-            QT_CUDA(cudaEventRecord(e1, st));
-            QT_CUDA(cudaEventSynchronize(e1));
-            float ms = 0.f;
-            QT_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-            if (rep > 0) fastest = std::min(fastest, ms);     // the first run warms up
-        }
-        if (fastest < best) {
-            best = fastest;
-            bestv = v;
-        }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    ctx->tune[key] = bestv;
-    return QT_OK;
-}
-
 TuneKey tune_key(const Plan& P, int prec, const int64_t* Ns, int n)
 {
     long long mx = 1;
@@ -1301,22 +1219,6 @@ qt_status forward_common(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
     if (s) return s;
     P.euler = euler;
     const bool capturing = stream_is_capturing(st);
-    if (P.form == kTcRecheck && o->tc_draw == 0 && !(o->flags & QT_FLAG_NO_TUNE) && !capturing &&
-        o->spin_budget >= 0 && source == kSampler) {
-        const TuneKey key = tune_key(P, o->sample_prec, Ns, n);
-        if (!ctx->tune.count(key)) {
-            if ((s = autotune_tc(ctx, d, n, Ns, mus, params_d_host, M, seed, o, source, io, P, key, st))) return s;
-        }
-        if (o != &oi) {
-            oi = *o;
-            o = &oi;
-        }
-        oi.tc_draw = ctx->tune[key];
-        Plan P2;
-        if ((s = make_plan(ctx, d, n, Ns, mus, M, o, source == kArrays, P2, only_layer, algo))) return s;
-        P2.euler = euler;
-        P = P2;
-    }
     if (P.form != kTcRecheck && P.form != kRouterCert && P.form != kPathwise && P.form != kCells &&
         P.form != kPathCells && o->tile_samples_per_thread <= 0 &&
         !(o->flags & QT_FLAG_NO_TUNE) && !capturing && o->spin_budget >= 0) {

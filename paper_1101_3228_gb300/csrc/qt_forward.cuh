@@ -100,7 +100,10 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
     const unsigned long long t0 = global_ns();
     const unsigned long long lim = (unsigned long long)budget_us * 1000ull;
     while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
+        // several tries to a reading of the timer (eight instructions)
+#pragma unroll 1
+        for (int r = 0; r < 8; ++r)
+            if (mbar_try_wait(bar, parity)) return true;
         if (global_ns() - t0 > lim) return false;
     }
 }

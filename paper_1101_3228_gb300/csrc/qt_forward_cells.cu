@@ -36,7 +36,7 @@ __device__ __forceinline__ float warp_max(float v)
 // is positive on the whole box by more than `marg`, which covers the FP32
 // rounding of the points and of this test.
 template <int DM>
-__global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const ForwardParams p)
+__global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid_constant__ ForwardParams p)
 {
     __shared__ float s_g[kCellMaxN * DM];
     __shared__ uint16_t s_surv[kBuildWarps][kCellMaxN];
@@ -268,7 +268,7 @@ static __device__ __noinline__ int cell_recheck(const ForwardParams& p, const fl
 // pair at d = 2, most of them the draw).  2-factor workload, 10^9 pairs: 19.5 ms,
 // against 142.9 ms for brute force over 1000 candidates a pair.
 template <int DM, int MODE>
-__global__ void __launch_bounds__(kCellThreads, 1) forward_cells_kernel(const ForwardParams p)
+__global__ void __launch_bounds__(kCellThreads, 1) forward_cells_kernel(const __grid_constant__ ForwardParams p)
 {
     extern __shared__ __align__(128) unsigned char dsm_c[];
     __shared__ __align__(8) unsigned long long s_bar;

@@ -54,7 +54,7 @@ struct GridInfo {
     int32_t N, Npad;
     long long goff, roff;
     int32_t tc_exp;                // tensor-core form: operands scaled by 2^tc_exp
-    int32_t tc_tiles;              // tensor-core form: 256-point operand tiles of this grid
+    int32_t tc_tiles;              // tensor-core form: 128-point operand tiles of this grid
     long long tc_toff;             // tensor-core form: first tile of this grid
 };
 
@@ -79,26 +79,24 @@ constexpr int kCellMaxN = 1024;    // points of a grid: ten bits per index
 constexpr int kCellThreads = 1024; // most threads of the located-search kernels
 constexpr int kCellNearStride = 20;// floats of a layer's combined FP32 parameters (d <= 2)
 
-constexpr int kTcTileN = 256;      // grid points per tensor-core operand tile (MMA N)
-constexpr int kTcTileM = 128;      // samples per tensor-core work item (MMA M)
-constexpr int kTcThreads = 512;    // tensor-core form: 16 warps (8 epilogue, 2 MMA, tile loader, draw, 4 certifier)
-constexpr int kTcMaxSlots = 16;    // tensor-core form: most operand tiles held in shared memory
+constexpr int kTcTileN = 128;      // grid points per tensor-core operand tile (MMA N)
+constexpr int kTcTileM = 128;      // samples of a tensor-core work item (MMA M)
+constexpr int kTcThreads = 128;    // tensor-core form: one warpgroup per CTA,
+constexpr int kTcCtas = 4;         // four CTAs per SM
+constexpr int kTcMaxSlots = 6;     // tensor-core form: most operand tiles in flight in shared memory
 
-// Bytes of one work item's drawn samples in the tensor-core form, as the
-// certifier warps draw them into an item slot in shared memory, or the draw
-// pass writes them to device memory: the FP16 operand rows of both grids
-// (128 x K each, core-matrix layout), then the centred FP32 coordinates and
-// norms ([grid][dm + 1][128]).
-__host__ __device__ constexpr long long tc_item_op_bytes(int K) { return 2ll * kTcTileM * K * 2; }
+// Bytes of one work item's record between the kernels of the tensor-core form: the
+// centred FP32 coordinates and norms ([grid][dm + 1][128]) and the chunk states
+// ([grid][4][128]).
 __host__ __device__ constexpr long long tc_item_cert_bytes(int dm) { return 2ll * (dm + 1) * kTcTileM * 4; }
+__host__ __device__ constexpr long long tc_item_bytes(int dm) { return tc_item_cert_bytes(dm) + 2ll * 4 * kTcTileM * 4; }
 
-// Dynamic shared memory of the tensor-core form besides its ring of operand
-// tiles (dimension class dm, K columns per operand row).
+// Dynamic shared memory of the tensor-core screen besides its ring of operand tiles
+// (dimension class dm, K columns per operand row): the operand rows of one grid
+// and the centred samples of two items.
 __host__ __device__ constexpr long long tc_fixed_smem(int dm, int K)
 {
-    return 2 * tc_item_op_bytes(K)                           // sample operands: 2 items
-           + 2ll * 2 * 2 * 5 * kTcTileM * 4                  // chunk states: 2 items x 2 grids x 2 warpgroups x 5
-           + 2 * tc_item_cert_bytes(dm);                     // centred samples: 2 items
+    return (long long)kTcTileM * K * 2 + 2 * tc_item_cert_bytes(dm);
 }
 
 struct ForwardParams {
@@ -142,13 +140,13 @@ struct ForwardParams {
     int32_t* dumpJ;
     DevStatus* status;
     // tensor-core form
-    const void* tc_tiles;          // FP16 operand tiles [tiles][256][K] in the canonical K-major layout
+    const void* tc_tiles;          // FP16 operand tiles [tiles][128][K] in the canonical K-major layout
+    const float* tc_rows;          // chunk-major FP32 records [tiles * 8][dm + 1][16]
     int32_t tc_k;                  // 16 or 32
     int32_t tc_slots;              // ring slots of operand tiles in shared memory
-    int32_t tc_resident;           // 1: both grids' tiles stay in shared memory for the layer
     long long item_lo, item_hi;    // tensor-core form: work items [item_lo, item_hi) of this launch
-    int32_t tc_draw_in;            // tensor-core form: 1 = the screen kernel draws its samples
-    unsigned char* tc_items;       // tensor-core form, draw pass: samples of the launch's items
+    long long tc_ipl;              // tensor-core form: work items of every layer (0: one layer has them all)
+    unsigned char* tc_items;       // tensor-core form: records of the window's items
     // located search (d <= 2)
     CellGrid* cells;               // [n+1]
     unsigned long long* cell_tab;  // bin entries of every grid

@@ -16,7 +16,7 @@
 namespace qt {
 
 template <int DM, int S, bool F32>
-__global__ void __launch_bounds__(kCellThreads, 1) path_cells_kernel(const ForwardParams p)
+__global__ void __launch_bounds__(kCellThreads, 1) path_cells_kernel(const __grid_constant__ ForwardParams p)
 {
     using T = typename SampleType<F32>::T;
     extern __shared__ __align__(128) unsigned char dsm_pc[];

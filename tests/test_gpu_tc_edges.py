@@ -1,0 +1,79 @@
+"""The tensor-core form at the sizes where its tiles, items and windows end, against
+the oracle: grids of one point, one chunk, one operand tile and one point either side
+of a tile, more tiles than the ring holds, samples either side of an item of 128, and
+samples that tie within a chunk (exact distances to the chunk alone) or across chunks
+(window search).  Counts and cells are compared bit for bit.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import qt_workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def B(gpu_lib):
+    from paper_1101_3228_gb300 import binding
+    return binding
+
+
+@pytest.fixture(scope="module")
+def ctx(B):
+    c = B.Context(0)
+    yield c
+    c.close()
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+@pytest.mark.parametrize("d", [3, 4, 6, 8, 10])
+@pytest.mark.parametrize("NA,NB,M", [(1, 16, 1), (17, 127, 127), (128, 129, 128), (1, 1, 129), (255, 2, 300),
+                                     (1500, 1, 513), (900, 1700, 1000)])
+def test_cells_at_tile_edges(ctx, B, d, NA, NB, M):
+    rng = np.random.default_rng(NA + 7 * NB + d)
+    gA, gB = rng.standard_normal((NA, d)), 0.7 * rng.standard_normal((NB, d)) + 0.2
+    X, Y = rng.standard_normal((M, d)), rng.standard_normal((M, d))
+    # last points of the last chunk, and exact ties: duplicated points near and far in the grid
+    if NA > 16:
+        gA[-1] = gA[3]
+        gA[5] = gA[4]
+        X[::5] = gA[rng.integers(0, NA, len(X[::5]))]
+    if NB > 16:
+        gB[NB // 2] = gB[NB // 2 - 1]
+        Y[::4] = gB[rng.integers(0, NB, len(Y[::4]))] + 1e-9 * rng.standard_normal((len(Y[::4]), d))
+    for ct in (B.COUNTS_I64, B.COUNTS_U32):
+        counts, st, ii, jj = ctx.counts_from_samples(_dev(gA), _dev(gB), _dev(X), _dev(Y),
+                                                     B.options(form=B.FORM_TC_RECHECK, counts_type=ct), want_cells=True)
+        np.testing.assert_array_equal(ii.cpu().numpy(), oracle.nearest(gA, X))
+        np.testing.assert_array_equal(jj.cpu().numpy(), oracle.nearest(gB, Y))
+        np.testing.assert_array_equal(counts.cpu().numpy(), oracle.counts_from_samples(gA, gB, X, Y))
+        assert st.form_used == B.FORM_TC_RECHECK and st.device_status == 0
+
+
+@pytest.mark.parametrize("chunk", [1, 3, 0])
+def test_uneven_layers_over_windows(ctx, B, chunk):
+    """Layers of very different grid sizes, a one-point grid in the middle, windows that
+    end inside a layer; given draws of either layout option are the same step."""
+    d, Ns = 4, [1, 300, 20, 1, 700, 129]
+    rng = np.random.default_rng(2)
+    n = len(Ns) - 1
+    L = np.concatenate([np.zeros((1, d, d)), np.repeat((np.eye(d) - 0.3 * np.tri(d, k=-1))[None], n, 0)])
+    A = np.repeat(0.9 * np.eye(d)[None], n, 0)
+    T = np.repeat(0.4 * np.eye(d)[None], n, 0)
+    model = W.Model("edge", d, n, np.array(Ns, dtype=np.int64), A, np.zeros((n, d)), T, np.zeros((n + 1, d)), L,
+                    np.arange(n + 1.0), 0.0, "basket_put", 1.0, None, 700, 31, W.PREC_F32, "kmeans")
+    g = np.concatenate([rng.standard_normal((k, d)) for k in Ns])
+    for prec in (W.PREC_F32, W.PREC_F64):
+        ref = oracle.transitions(model, g, model.M, model.seed, prec)
+        for draw in (0, 1, 2):
+            counts, st, _ = ctx.transitions(model, _dev(g), model.M, model.seed,
+                                            B.options(prec=prec, tc_chunk_items=chunk, tc_draw=draw))
+            got = B.split_counts(model.N, counts.cpu().numpy())
+            for k in range(n):
+                np.testing.assert_array_equal(got[k], ref[k], err_msg=f"layer {k}")
+            assert st.device_status == 0
