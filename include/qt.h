@@ -242,7 +242,8 @@ QT_API qt_status qt_counts_from_samples(qt_ctx* ctx, int32_t d, const double* gA
  * V_k(i) = max(phi_k(i), sum_j pi^k_ij V_{k+1}(j)) with pi^k_ij = p^k_ij / p^k_i
  * (Algorithm III's normalisation).  A row with p^k_i = 0 has no continuation:
  * V_k(i) = phi_k(i).  The continuation is evaluated as
- * (sum_j p^k_ij V_{k+1}(j)) / p^k_i in FP64, j summed in lanes j mod 32 and
+ * (sum_j p^k_ij V_{k+1}(j)) / p^k_i in FP64, j summed (one fused multiply-add
+ * each) in lanes j mod 32 and
  * combined by a fixed butterfly, so results are bitwise reproducible.
  *   N      host int64 [n+1]
  *   counts dev, counts_type elements, concatenated as in qt_transitions

@@ -20,12 +20,18 @@
 
 namespace qt {
 __global__ void prep_records_kernel(const double*, GridInfo*, int, int, int, int, long long, float*, double*);
-__global__ void backward_layer_kernel(const void*, int, long long, int, int, const double*, const double*, double*);
+cudaError_t launch_backward_layer(const void* counts, int u32, long long coff, int Nk, int Nk1, const double* phik,
+                                  const double* Vnext, double* Vk, int num_sms, cudaStream_t st);
+bool backward_tree_fits(int n, const int64_t* N, int num_sms);
+cudaError_t launch_backward_tree(const void* counts, int u32, int n, int maxN, const void* layers, const double* phi,
+                                 double* V, double* X, int num_sms, cudaStream_t st);
+int backward_tree_blocks(int maxN, int num_sms);
 __global__ void root_price_kernel(const void*, int, int, int, const double*, double*);
 __global__ void fold_status_kernel(const DevStatus*, DevStatus*);
 __global__ void swing_terminal_kernel(int, int, int, int, double*);
-__global__ void swing_layer_kernel(const void*, int, long long, int, int, const double*, const double*, double*, int,
-                                   int, int, int);
+cudaError_t launch_swing_layer(const void* counts, int u32, long long coff, int Nk, int Nk1, const double* vk,
+                               const double* Pnext, double* Pk, int n, int k, int Qmin, int Qmax, int num_sms,
+                               cudaStream_t st);
 __global__ void kmeans_draw_kernel(int, unsigned long long, long long, float*);
 __global__ void kmeans_assign_kernel(int, long long, const float*, int, const float*, unsigned long long*,
                                      unsigned long long*, int);
@@ -75,6 +81,9 @@ struct qt_ctx {
     cudaEvent_t ev_tables = nullptr;   // end of the last forward step (workspace and tables in use until then)
     cudaEvent_t ev_up[2] = {nullptr, nullptr};   // last upload from each of the two pinned table blocks
     int up = 0;
+    cudaEvent_t ev_tree = nullptr;     // end of the last one-launch backward induction
+    cudaEvent_t ev_up_tree[2] = {nullptr, nullptr};   // last upload from each of its pinned tables
+    int up_tree = 0;
     cudaEvent_t ev_k0 = nullptr, ev_k1 = nullptr;   // around the forward kernel (stats.ms)
     bool timed = false;
     // cached graph of the last forward call
@@ -258,6 +267,9 @@ extern "C" qt_status qt_create(qt_ctx** out, int32_t device)
         cudaEventCreateWithFlags(&ctx->ev_tables, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_up[0], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_up[1], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_tree, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_up_tree[0], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&ctx->ev_up_tree[1], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreate(&ctx->ev_k0) != cudaSuccess || cudaEventCreate(&ctx->ev_k1) != cudaSuccess) {
         delete ctx;
         return QT_ECUDA;
@@ -278,8 +290,11 @@ extern "C" qt_status qt_destroy(qt_ctx* ctx)
         if (kv.second.p) cudaFreeHost(kv.second.p);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->ev_tables) cudaEventDestroy(ctx->ev_tables);
-    for (int u = 0; u < 2; ++u)
+    if (ctx->ev_tree) cudaEventDestroy(ctx->ev_tree);
+    for (int u = 0; u < 2; ++u) {
         if (ctx->ev_up[u]) cudaEventDestroy(ctx->ev_up[u]);
+        if (ctx->ev_up_tree[u]) cudaEventDestroy(ctx->ev_up_tree[u]);
+    }
     if (ctx->ev_k0) cudaEventDestroy(ctx->ev_k0);
     if (ctx->ev_k1) cudaEventDestroy(ctx->ev_k1);
     delete ctx;
@@ -1433,15 +1448,46 @@ extern "C" qt_status qt_backward(qt_ctx* ctx, int32_t n, const int64_t* N, const
     std::vector<long long> goff(n + 2, 0), coff(n + 1, 0);
     for (int k = 0; k <= n; ++k) goff[k + 1] = goff[k] + N[k];
     for (int k = 0; k < n; ++k) coff[k + 1] = coff[k] + N[k] * N[k + 1];
-    QT_CUDA(cudaMemcpyAsync(V + goff[n], phi + goff[n], sizeof(double) * N[n], cudaMemcpyDeviceToDevice, st));
     const int u32 = counts_type == QT_COUNTS_U32;
-    for (int k = n - 1; k >= 0; --k) {
-        const long long threads = (long long)N[k] * 32;
-        const int blk = 256;
-        backward_layer_kernel<<<(unsigned)((threads + blk - 1) / blk), blk, 0, st>>>(
-            counts, u32, coff[k], (int)N[k], (int)N[k + 1], phi + goff[k], V + goff[k + 1], V + goff[k]);
-        QT_CUDA(cudaGetLastError());
+    if (backward_tree_fits(n, N, ctx->num_sms) && !stream_is_capturing(st)) {
+        // a small tree in one launch.  Its layer table and the exchange of its CTAs are
+        // the context's: a call on another stream waits for the last one
+        const size_t bytes = sizeof(TreeLayer) * (size_t)(n + 1);
+        int maxN = 1;
+        for (int k = 0; k <= n; ++k) maxN = std::max(maxN, (int)N[k]);
+        const size_t xb = sizeof(double) * 8 * (size_t)n * backward_tree_blocks(maxN, ctx->num_sms);
+        void *dt, *dx, *ht;
+        qt_status s;
+        const std::string block = ctx->up_tree ? "tree1" : "tree0";
+        // a capture on another stream of this thread does not mind the allocations
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        QT_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+        if (!(s = dev_get(ctx, "tree", bytes, &dt)) && !(s = dev_get(ctx, "tree_x", xb, &dx)))
+            s = host_get(ctx, block.c_str(), bytes, &ht);
+        QT_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+        if (s == QT_OK) {
+            QT_CUDA(cudaEventSynchronize(ctx->ev_up_tree[ctx->up_tree]));
+            QT_CUDA(cudaStreamWaitEvent(st, ctx->ev_tree, 0));
+            TreeLayer* tl = (TreeLayer*)ht;
+            for (int k = 0; k <= n; ++k) tl[k] = TreeLayer{coff[k], goff[k], (int)N[k], 0};
+            QT_CUDA(cudaMemcpyAsync(dt, ht, bytes, cudaMemcpyHostToDevice, st));
+            QT_CUDA(cudaEventRecord(ctx->ev_up_tree[ctx->up_tree], st));
+            ctx->up_tree ^= 1;
+            const cudaError_t e =
+                launch_backward_tree(counts, u32, n, maxN, dt, phi, V, (double*)dx, ctx->num_sms, st);
+            QT_CUDA(cudaEventRecord(ctx->ev_tree, st));
+            if (e != cudaErrorCooperativeLaunchTooLarge) {
+                QT_CUDA(e);
+                return QT_OK;
+            }
+            cudaGetLastError();
+        }
+        // no memory for it, or a partition with fewer SMs than the device: layer by layer
     }
+    QT_CUDA(cudaMemcpyAsync(V + goff[n], phi + goff[n], sizeof(double) * N[n], cudaMemcpyDeviceToDevice, st));
+    for (int k = n - 1; k >= 0; --k)
+        QT_CUDA(launch_backward_layer(counts, u32, coff[k], (int)N[k], (int)N[k + 1], phi + goff[k], V + goff[k + 1],
+                                      V + goff[k], ctx->num_sms, st));
     return QT_OK;
 }
 
@@ -1470,18 +1516,14 @@ extern "C" qt_status qt_swing(qt_ctx* ctx, int32_t n, const int64_t* N, const vo
     for (int k = 0; k < n; ++k)
         if ((N[k] * qchunks * 32 + 255) / 256 > 0x7FFFFFFFll)
             return fail(ctx, QT_EINVAL, "N[%d] x (Qmax + 1) too large for one launch", k);
-    for (int k = n - 1; k >= 0; --k) {
-        const long long threads = (long long)N[k] * qchunks * 32;
-        swing_layer_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(
-            counts, u32, coff[k], (int)N[k], (int)N[k + 1], v + goff[k], P + nq * goff[k + 1], P + nq * goff[k], n,
-            k, Qmin, Qmax);
-        QT_CUDA(cudaGetLastError());
-    }
+    for (int k = n - 1; k >= 0; --k)
+        QT_CUDA(launch_swing_layer(counts, u32, coff[k], (int)N[k], (int)N[k + 1], v + goff[k], P + nq * goff[k + 1],
+                                   P + nq * goff[k], n, k, Qmin, Qmax, ctx->num_sms, st));
     if (price) {
         void* dout;
         qt_status s = dev_get(ctx, "swing_out", sizeof(double), &dout);
         if (s) return s;
-        root_price_kernel<<<1, 32, 0, st>>>(counts, u32, (int)N[0], (int)N[1], P, (double*)dout);
+        root_price_kernel<<<1, 1024, 0, st>>>(counts, u32, (int)N[0], (int)N[1], P, (double*)dout);
         QT_CUDA(cudaGetLastError());
         QT_CUDA(cudaMemcpyAsync(price, dout, sizeof(double), cudaMemcpyDeviceToHost, st));
         QT_CUDA(cudaStreamSynchronize(st));
@@ -1564,16 +1606,14 @@ extern "C" qt_status qt_price(qt_ctx* ctx, const qt_model* model, const double* 
                 return s;
             fold_status_kernel<<<1, 1, 0, st>>>((const DevStatus*)ctx->status_buf, (DevStatus*)dacc);
             QT_CUDA(cudaGetLastError());
-            const long long threads = model->N[k] * 32;
-            backward_layer_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(
-                dcounts, o.counts_type == QT_COUNTS_U32, 0, (int)model->N[k], (int)model->N[k + 1], dphi + goff[k],
-                V + goff[k + 1], V + goff[k]);
-            QT_CUDA(cudaGetLastError());
+            QT_CUDA(launch_backward_layer(dcounts, o.counts_type == QT_COUNTS_U32, 0, (int)model->N[k],
+                                          (int)model->N[k + 1], dphi + goff[k], V + goff[k + 1], V + goff[k],
+                                          ctx->num_sms, st));
         }
         // the status the caller reads is the accumulated one
         QT_CUDA(cudaMemcpyAsync(ctx->status_buf, dacc, sizeof(DevStatus), cudaMemcpyDeviceToDevice, st));
     }
-    root_price_kernel<<<1, 32, 0, st>>>(dcounts, o.counts_type == QT_COUNTS_U32, (int)model->N[0], (int)model->N[1],
+    root_price_kernel<<<1, 1024, 0, st>>>(dcounts, o.counts_type == QT_COUNTS_U32, (int)model->N[0], (int)model->N[1],
                                         (const double*)dV, (double*)dout);
     QT_CUDA(cudaGetLastError());
     QT_CUDA(cudaMemcpyAsync(price, dout, sizeof(double), cudaMemcpyDeviceToHost, st));

@@ -170,6 +170,12 @@ struct ForwardParams {
     unsigned long long rt_checksum;// checksum of the grids the router was built for
 };
 
+// One layer of a tree whose backward induction runs in one launch.
+struct TreeLayer {
+    long long coff, goff;          // its counts and its points, from the first
+    int32_t N, pad;
+};
+
 constexpr int kSwingQ = 8;         // swing option: consumption states per warp
 
 constexpr int kRtHidden = 64;      // router MLP width
