@@ -32,11 +32,6 @@ __global__ void swing_terminal_kernel(int, int, int, int, double*);
 cudaError_t launch_swing_layer(const void* counts, int u32, long long coff, int Nk, int Nk1, const double* vk,
                                const double* Pnext, double* Pk, int n, int k, int Qmin, int Qmax, int num_sms,
                                cudaStream_t st);
-__global__ void kmeans_draw_kernel(int, unsigned long long, long long, float*);
-__global__ void kmeans_assign_kernel(int, long long, const float*, int, const float*, unsigned long long*,
-                                     unsigned long long*, int);
-__global__ void kmeans_update_kernel(int, int, const unsigned long long*, const unsigned long long*, float*);
-__global__ void map_grid_kernel(int, int, const double*, const double*, const double*, double*);
 __global__ void prep_tc_tiles_kernel(const float*, GridInfo*, int, int, int, int, int, long long, __half*, float*);
 cudaError_t launch_router_forward(int dm, const ForwardParams& p, int num_sms, int* bps, cudaStream_t st);
 cudaError_t launch_grid_checksum(const double* grids, long long count, unsigned long long* out, cudaStream_t st);
@@ -1733,16 +1728,19 @@ extern "C" qt_status qt_build_grids(qt_ctx* ctx, const qt_model* model, int32_t 
     if (tol <= 0) tol = 1e-14;
     DeviceGuard g(ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
-    std::map<long long, std::vector<double>> base;   // N -> base grid of N(0, I_d), [N][d]
+    // distinct sizes, each with its base grid of N(0, I_d): FP64 [N][d] in one block, or
+    // the centres of the sample Lloyd
+    std::map<long long, long long> at;   // N -> first double of the block, or float of the centres
+    std::vector<double> G;
+    long long maxN = 0;
     for (int k = 0; k <= n; ++k) {
         const long long Nk = model->N[k];
-        if (base.count(Nk)) continue;
-        std::vector<double> G((size_t)Nk * d, 0.0);
-        if (Nk == 1) {
-            // the single point is the mean
-        } else if (method == QT_GRID_LLOYD1D) {
-            std::vector<double> x = lloyd1d((int)Nk, tol);
-            for (long long j = 0; j < Nk; ++j) G[j] = x[j];
+        maxN = std::max(maxN, Nk);
+        if (Nk == 1 || at.count(Nk)) continue;   // the single point is the mean
+        at[Nk] = (long long)G.size();
+        if (method == QT_GRID_LLOYD1D) {
+            const std::vector<double> x = lloyd1d((int)Nk, tol);
+            G.insert(G.end(), x.begin(), x.end());
         } else if (method == QT_GRID_PRODUCT) {
             std::vector<int> best, cur;
             double score = 0;
@@ -1750,69 +1748,79 @@ extern "C" qt_status qt_build_grids(qt_ctx* ctx, const qt_model* model, int32_t 
             std::sort(best.begin(), best.end());
             std::vector<std::vector<double>> ax;
             for (int l = 0; l < d; ++l) ax.push_back(lloyd1d(best[l], tol));
+            const size_t at0 = G.size();
+            G.resize(at0 + (size_t)Nk * d);
             for (long long j = 0; j < Nk; ++j) {
                 long long r = j;
                 for (int l = d - 1; l >= 0; --l) {
-                    G[j * d + l] = ax[l][r % best[l]];
+                    G[at0 + j * d + l] = ax[l][r % best[l]];
                     r /= best[l];
                 }
             }
-        } else {
-            const long long S = samples > 0 ? samples : std::max<long long>(20 * Nk, 100000);
-            const int its = iters > 0 ? iters : 20;
-            if (S < Nk) return fail(ctx, QT_EINVAL, "k-means needs at least N training samples");
-            void *dZ, *dC, *dsum, *dcnt;
-            if ((s = dev_get(ctx, "km_Z", sizeof(float) * (size_t)S * d, &dZ))) return s;
-            if ((s = dev_get(ctx, "km_C", sizeof(float) * (size_t)Nk * d, &dC))) return s;
-            if ((s = dev_get(ctx, "km_sum", 8 * (size_t)Nk * d, &dsum))) return s;
-            if ((s = dev_get(ctx, "km_cnt", 8 * (size_t)Nk, &dcnt))) return s;
-            const unsigned long long kseed = seed ^ (0x9E3779B97F4A7C15ull * (unsigned long long)Nk);
-            kmeans_draw_kernel<<<(unsigned)((S + 255) / 256), 256, 0, st>>>(d, kseed, S, (float*)dZ);
-            QT_CUDA(cudaGetLastError());
-            QT_CUDA(cudaMemcpyAsync(dC, dZ, sizeof(float) * (size_t)Nk * d, cudaMemcpyDeviceToDevice, st));
-            const size_t csm = sizeof(float) * (size_t)Nk * d;
-            const int use_smem = csm <= 160 * 1024;
-            if (use_smem)
-                QT_CUDA(cudaFuncSetAttribute(kmeans_assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)csm));
-            for (int it = 0; it < its; ++it) {
-                QT_CUDA(cudaMemsetAsync(dsum, 0, 8 * (size_t)Nk * d, st));
-                QT_CUDA(cudaMemsetAsync(dcnt, 0, 8 * (size_t)Nk, st));
-                kmeans_assign_kernel<<<(unsigned)((S + 255) / 256), 256, use_smem ? csm : 0, st>>>(
-                    d, S, (const float*)dZ, (int)Nk, (const float*)dC, (unsigned long long*)dsum,
-                    (unsigned long long*)dcnt, use_smem);
-                QT_CUDA(cudaGetLastError());
-                kmeans_update_kernel<<<(unsigned)((Nk + 255) / 256), 256, 0, st>>>(
-                    d, (int)Nk, (const unsigned long long*)dsum, (const unsigned long long*)dcnt, (float*)dC);
-                QT_CUDA(cudaGetLastError());
-            }
-            std::vector<float> Gf((size_t)Nk * d);
-            QT_CUDA(cudaMemcpyAsync(Gf.data(), dC, csm, cudaMemcpyDeviceToHost, st));
-            QT_CUDA(cudaStreamSynchronize(st));
-            for (size_t e = 0; e < Gf.size(); ++e) G[e] = (double)Gf[e];
         }
-        base[Nk] = std::move(G);
     }
-    // map every layer: x = m_k + L_k g
+    void *dG = nullptr, *dC = nullptr, *dtab;
+    if (method == QT_GRID_KMEANS && !at.empty()) {
+        const int dm = kmeans_dim_class(d), its = iters > 0 ? iters : 20;
+        auto draws = [&](long long Nk) { return samples > 0 ? (long long)samples : std::max<long long>(20 * Nk, 100000); };
+        long long centres = 0;
+        for (auto& kv : at) {
+            if (draws(kv.first) < kv.first) return fail(ctx, QT_EINVAL, "k-means needs at least N training samples");
+            kv.second = centres;
+            centres += (kv.first + 15) / 16 * 16 * dm;
+        }
+        if ((s = dev_get(ctx, "km_C", sizeof(float) * (size_t)centres, &dC))) return s;
+        // as many sizes in each launch as keep their draws within 1 GiB (one at least),
+        // the largest first
+        for (auto it = at.rbegin(); it != at.rend();) {
+            KmJobs jobs;
+            int nj = 0;
+            size_t zf = 0, sw = 0;
+            auto end = it;
+            for (; end != at.rend() && nj < kKmJobs; ++end, ++nj) {
+                const size_t z = (size_t)draws(end->first) * d;
+                if (nj > 0 && (zf + z) * sizeof(float) > ((size_t)1 << 30)) break;
+                zf += z;
+                sw += (size_t)end->first * (d + 1);
+            }
+            void *dZ, *dsum;
+            if ((s = dev_get(ctx, "km_Z", sizeof(float) * zf, &dZ))) return s;
+            if ((s = dev_get(ctx, "km_sum", sizeof(unsigned long long) * sw, &dsum))) return s;
+            zf = sw = 0;
+            for (int i = 0; i < nj; ++i, ++it) {
+                const long long Nk = it->first;
+                jobs.j[i] = KmJob{(float*)dZ + zf, (float*)dC + it->second, (unsigned long long*)dsum + sw,
+                                  seed ^ (0x9E3779B97F4A7C15ull * (unsigned long long)Nk), draws(Nk), (int)Nk,
+                                  (int)((Nk + 15) / 16 * 16)};
+                zf += (size_t)draws(Nk) * d;
+                sw += (size_t)Nk * (d + 1);
+            }
+            QT_CUDA(launch_kmeans(jobs, nj, d, its, ctx->num_sms, st));
+        }
+    } else if (!G.empty()) {
+        if ((s = dev_get(ctx, "bg_G", sizeof(double) * G.size(), &dG))) return s;
+        QT_CUDA(cudaMemcpyAsync(dG, G.data(), sizeof(double) * G.size(), cudaMemcpyHostToDevice, st));
+    }
+    // map every layer in one launch: x = m_k + L_k g
+    const size_t mb = sizeof(double) * (size_t)(n + 1) * d, lb = mb * d, tb = sizeof(MapLayer) * (size_t)(n + 1);
+    std::vector<unsigned char> tab(tb + mb + lb);
     long long off = 0;
-    void *dG, *dm, *dL;
-    long long maxN = 0;
-    for (int k = 0; k <= n; ++k) maxN = std::max<long long>(maxN, model->N[k]);
-    if ((s = dev_get(ctx, "bg_G", sizeof(double) * (size_t)maxN * d, &dG))) return s;
-    if ((s = dev_get(ctx, "bg_m", sizeof(double) * d, &dm))) return s;
-    if ((s = dev_get(ctx, "bg_L", sizeof(double) * d * d, &dL))) return s;
     for (int k = 0; k <= n; ++k) {
         const long long Nk = model->N[k];
-        const std::vector<double>& G = base[Nk];
-        QT_CUDA(cudaMemcpyAsync(dG, G.data(), sizeof(double) * (size_t)Nk * d, cudaMemcpyHostToDevice, st));
-        QT_CUDA(cudaMemcpyAsync(dm, model->m + (long long)k * d, sizeof(double) * d, cudaMemcpyHostToDevice, st));
-        QT_CUDA(cudaMemcpyAsync(dL, model->L + (long long)k * d * d, sizeof(double) * d * d, cudaMemcpyHostToDevice, st));
-        map_grid_kernel<<<(unsigned)((Nk + 255) / 256), 256, 0, st>>>(d, (int)Nk, (const double*)dG,
-                                                                    (const double*)dm, (const double*)dL,
-                                                                    grids + off * d);
-        QT_CUDA(cudaGetLastError());
-        QT_CUDA(cudaStreamSynchronize(st));  // the staging buffers are reused next layer
+        MapLayer T{nullptr, nullptr, off * d, (int)Nk, 0};
+        if (Nk > 1) {
+            if (dG) T.f64 = (const double*)dG + at[Nk];
+            else T.f32 = (const float*)dC + at[Nk];
+        }
+        memcpy(tab.data() + sizeof(MapLayer) * (size_t)k, &T, sizeof(MapLayer));
         off += Nk;
     }
+    memcpy(tab.data() + tb, model->m, mb);
+    memcpy(tab.data() + tb + mb, model->L, lb);
+    if ((s = dev_get(ctx, "bg_tab", tab.size(), &dtab))) return s;
+    QT_CUDA(cudaMemcpyAsync(dtab, tab.data(), tab.size(), cudaMemcpyHostToDevice, st));
+    QT_CUDA(launch_map_grids(d, n + 1, maxN, (const MapLayer*)dtab, (const double*)((unsigned char*)dtab + tb),
+                             (const double*)((unsigned char*)dtab + tb + mb), grids, st));
+    QT_CUDA(cudaStreamSynchronize(st));   // the uploads' host memory and the workspace are free again
     return QT_OK;
 }

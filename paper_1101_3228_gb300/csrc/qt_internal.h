@@ -170,6 +170,28 @@ struct ForwardParams {
     unsigned long long rt_checksum;// checksum of the grids the router was built for
 };
 
+// Sample Lloyd: one grid size of a launch (qt_kmeans.cu).
+struct KmJob {
+    float* Z;                      // training draws [d][S]
+    float* C;                      // centres, pairs [Npad/2][dim class][2]
+    unsigned long long* sums;      // [N][d + 1]: fixed-point sums, count
+    unsigned long long seed;
+    long long S;
+    int32_t N, Npad;
+};
+constexpr int kKmJobs = 32;        // grid sizes per launch
+struct KmJobs {
+    KmJob j[kKmJobs];
+};
+
+// A layer of the grids built: its base grid (neither: the origin) and first output.
+struct MapLayer {
+    const double* f64;             // [N][d]
+    const float* f32;              // k-means centres
+    long long off;
+    int32_t N, pad;
+};
+
 // One layer of a tree whose backward induction runs in one launch.
 struct TreeLayer {
     long long coff, goff;          // its counts and its points, from the first

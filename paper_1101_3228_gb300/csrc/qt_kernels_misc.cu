@@ -686,80 +686,4 @@ __global__ void __launch_bounds__(1024) root_price_kernel(const void* __restrict
     if (lane == 0) *out = tot > 0 ? __ddiv_rn(acc, (double)tot) : 0.0;
 }
 
-// ------------------------------------------------------------------ sample Lloyd (grid builder)
-
-// Seeded N(0, I_d) training draws from the same Philox/Box-Muller sampler
-// (layer index 0xFFFF separates this stream from the forward step's).
-__global__ void kmeans_draw_kernel(int d, unsigned long long seed, long long S, float* Z)
-{
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= S) return;
-    float g[kDMax];
-    normals_f32<kDMax>(seed, 0xFFFF, (unsigned long long)t, d, g);
-    for (int l = 0; l < d; ++l) Z[t * d + l] = g[l];
-}
-
-// Nearest centre in FP32 (training assignment; exactness is not needed here)
-// and fixed-point sums (scale 2^36) so that the centroids do not depend on the
-// order of the atomics.
-__global__ void kmeans_assign_kernel(int d, long long S, const float* __restrict__ Z, int N,
-                                     const float* __restrict__ C, unsigned long long* sums,
-                                     unsigned long long* cnt, int use_smem)
-{
-    extern __shared__ float sC_dyn[];
-    if (use_smem) {
-        for (int e = threadIdx.x; e < N * d; e += blockDim.x) sC_dyn[e] = C[e];
-        __syncthreads();
-    }
-    const float* sC = use_smem ? sC_dyn : C;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= S) return;
-    float z[kDMax];
-    for (int l = 0; l < d; ++l) z[l] = Z[t * d + l];
-    float best = __int_as_float(0x7F800000);
-    int bi = 0;
-    for (int j = 0; j < N; ++j) {
-        float acc = 0.f;
-        for (int l = 0; l < d; ++l) {
-            const float df = z[l] - sC[j * d + l];
-            acc = fmaf(df, df, acc);
-        }
-        if (acc < best) {
-            best = acc;
-            bi = j;
-        }
-    }
-    atomicAdd(&cnt[bi], 1ull);
-    for (int l = 0; l < d; ++l) {
-        const long long q = __double2ll_rn((double)z[l] * 68719476736.0);
-        atomicAdd(&sums[(long long)bi * d + l], (unsigned long long)q);
-    }
-}
-
-__global__ void kmeans_update_kernel(int d, int N, const unsigned long long* sums, const unsigned long long* cnt,
-                                     float* C)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= N) return;
-    const unsigned long long c = cnt[j];
-    if (c == 0) return;  // empty cell keeps its centre
-    for (int l = 0; l < d; ++l) {
-        const long long s = (long long)sums[(long long)j * d + l];
-        C[j * d + l] = (float)(((double)s / 68719476736.0) / (double)c);
-    }
-}
-
-// Layer grids from a base grid: x = m_k + L_k g.
-__global__ void map_grid_kernel(int d, int N, const double* __restrict__ G, const double* __restrict__ mk,
-                                const double* __restrict__ Lk, double* out)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= N) return;
-    for (int l = 0; l < d; ++l) {
-        double acc = mk[l];
-        for (int q = 0; q <= l; ++q) acc += Lk[l * d + q] * G[j * d + q];
-        out[(long long)j * d + l] = acc;
-    }
-}
-
 }  // namespace qt

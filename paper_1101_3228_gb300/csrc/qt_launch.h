@@ -32,6 +32,11 @@ cudaError_t launch_pathwise(int dm, int S, bool f32, bool streamed, const Forwar
 cudaError_t launch_build_cells(int dm, const ForwardParams& p, int num_sms, cudaStream_t st);
 cudaError_t launch_forward_cells(int dm, const ForwardParams& p, int dyn, int num_sms, int* bps, cudaStream_t st);
 cudaError_t launch_path_cells(int dm, int S, const ForwardParams& p, int dyn, int num_sms, int* bps, cudaStream_t st);
+// grid builder: sample Lloyd of n <= kKmJobs sizes, and the layer grids
+int kmeans_dim_class(int d);
+cudaError_t launch_kmeans(const KmJobs& jobs, int n, int d, int iters, int num_sms, cudaStream_t st);
+cudaError_t launch_map_grids(int d, int layers, long long maxN, const MapLayer* tab, const double* m, const double* L,
+                             double* out, cudaStream_t st);
 cudaError_t launch_f32_streamed(int dm, int S, const ForwardParams& p, int block, int dyn, int num_sms, int* bps,
                                 cudaStream_t st);
 
