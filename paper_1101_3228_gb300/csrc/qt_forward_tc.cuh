@@ -36,9 +36,9 @@
 // issue slots of the chunk tracking (about 50 half-rate instructions per thread and
 // tile); what is left is the round trip of the 512 columns of tensor memory (issue,
 // MMA, arrival, read, hand-over: about 1700 cycles for the SM's four tiles, 420 a tile).
-// 8-d tree, 12 dates of 4000 points, 2e6 paths: 21.3 -> 19.5 ms; 4-d, 50 dates of
-// 2000 points on average, 1e6 paths: 19.1 -> 14.0 ms (draw 1.35, screen 9.7, certify
-// 3.1 ms of it); 10-d, 6 dates of 8000 points, 1e6 paths: 9.7 -> 8.8 ms; 3-d given
+// 8-d tree, 12 dates of 4000 points, 2e6 paths: 21.3 -> 19.3 ms; 4-d, 50 dates of
+// 2000 points on average, 1e6 paths: 19.1 -> 13.8 ms (draw 1.35, screen 9.7, certify
+// 2.9 ms of it); 10-d, 6 dates of 8000 points, 1e6 paths: 9.7 -> 8.7 ms; 3-d given
 // samples: 0.55 -> 0.38 ms.
 // The hand-over costs 2 (8 DM + 40) bytes of traffic per pair and reads of
 // them, 0.3 KB at d = 8, and buys kernels that each fit their registers: one kernel
@@ -111,10 +111,10 @@ __device__ __forceinline__ void tc_chunk_min4(uint32_t taddr, float& m0, float& 
 // plus 32 FP32 additions of the MMA (2^-23 each, counted as truncations), the
 // dropped tail product and the head/tail representation (3 * 2^-22), and the
 // absolute floor of the FP16 tails (2^-25 each) divided by sigma^2.
-__device__ __forceinline__ float tc_bound(int d, float A, float r, float inv_sigma)
+__device__ __forceinline__ float tc_bound(float sqrt_d, float A, float r, float sigma, float inv_sigma)
 {
     const float rel = 1.5f * 0x1p-18f;
-    const float absf = (0x1p-23f * sqrtf((float)d) * (A + r) * (1.0f / inv_sigma) + 0x1p-24f) * inv_sigma * inv_sigma;
+    const float absf = (0x1p-23f * sqrt_d * (A + r) * sigma + 0x1p-24f) * inv_sigma * inv_sigma;
     return rel * (r * r + 2.0f * A * r) + absf;
 }
 
@@ -123,55 +123,96 @@ __device__ __forceinline__ float cc_bound(int d, float A, float r)
     return (float)(d + 2) * 0x1p-24f * (1.0f + 0x1p-10f) * (r * r + 2.0f * A * r);
 }
 
-// FP32 re-score of every lane's chunk of 16 points by its quad of lanes: for each of
-// the quad's four samples in turn, lane q scores points 4q .. 4q+3 (one 16-byte load
-// per coordinate; the quad's loads cover 64 consecutive bytes of the chunk's
-// coordinate row) and two exchanges combine the quad.  A lane that fetched its own
-// chunk record by record touched 32 lines with every warp load, 1536 L1 wavefronts
-// per warp and search; this takes 288.  rows: the chunk-major records [chunk][DM + 1]
-// [16] (cc first), cert: the warp's centred samples [DM][128], lane's at `lane`.
-// Whole warp; lanes with chunk < 0 have nothing to score.
+// FP32 re-score of chunk ch of 16 points for the sample of lane src by a quad of
+// lanes: lane q of it scores points 4q .. 4q+3 (one 16-byte load per coordinate; the
+// quad's loads cover 64 consecutive bytes of the chunk's coordinate row) and two
+// exchanges combine the quad: smallest score, second smallest, first point of the
+// smallest.  rows: the chunk-major records [chunk][DM + 1][16] (cc first), cert: the
+// warp's centred samples [DM][128].
+template <int DM>
+__device__ __forceinline__ void quad_score(const float* __restrict__ rows, const float* cert, int q, int src, int ch,
+                                           float& best, float& second, int& idx)
+{
+    const float4* c4 = reinterpret_cast<const float4*>(rows) + (long long)ch * ((DM + 1) * 4) + q;
+    float4 g[DM + 1];
+#pragma unroll
+    for (int l = 0; l <= DM; ++l) g[l] = c4[l * 4];
+    float4 sc = g[0];
+#pragma unroll
+    for (int l = 0; l < DM; ++l) {
+        const float x = cert[l * kTcTileM + src];
+        sc.x = __fmaf_rn(x, g[1 + l].x, sc.x);
+        sc.y = __fmaf_rn(x, g[1 + l].y, sc.y);
+        sc.z = __fmaf_rn(x, g[1 + l].z, sc.z);
+        sc.w = __fmaf_rn(x, g[1 + l].w, sc.w);
+    }
+    // smallest (lowest point first) and second smallest of the lane's four
+    const bool xy = sc.y < sc.x, zw = sc.w < sc.z;
+    const float m0 = fminf(sc.x, sc.y), m1 = fminf(sc.z, sc.w);
+    const bool hi = m1 < m0;
+    best = fminf(m0, m1);
+    idx = hi ? (zw ? 3 : 2) : (xy ? 1 : 0);
+    second = fminf(fmaxf(m0, m1), hi ? fmaxf(sc.z, sc.w) : fmaxf(sc.x, sc.y));
+    idx += ch * kChunk + 4 * q;
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1) {
+        const float ob = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+        const float o2 = __shfl_xor_sync(0xFFFFFFFFu, second, o);
+        const int oi = __shfl_xor_sync(0xFFFFFFFFu, idx, o);
+        second = fminf(fminf(second, o2), fmaxf(best, ob));
+        const bool take = ob < best || (ob == best && oi < idx);
+        best = take ? ob : best;
+        idx = take ? oi : idx;
+    }
+}
+
+// Every lane's chunk, the quad's four samples in turn.  A lane that fetched its own
+// chunk record by record touched 32 lines with every warp load, 1536 L1 wavefronts per
+// warp and search; this takes 288.  Whole warp.
 template <int DM>
 __device__ __forceinline__ void quad_rescore(const float* __restrict__ rows, const float* cert, int lane, int chunk,
                                              float& best, float& second, int& idx)
 {
-    const int q = lane & 3;
-#pragma unroll 1
+    constexpr int kUnroll = DM <= 4 ? 2 : 1;   // two chunks' loads in flight where the registers allow it
+#pragma unroll kUnroll
     for (int s = 0; s < 4; ++s) {
         const int src = (lane & ~3) | s;
         const int ch = __shfl_sync(0xFFFFFFFFu, chunk, src);
-        const float4* c4 = reinterpret_cast<const float4*>(rows) + (long long)max(ch, 0) * ((DM + 1) * 4) + q;
-        float4 g[DM + 1];
-#pragma unroll
-        for (int l = 0; l <= DM; ++l) g[l] = c4[l * 4];
-        float4 sc = g[0];
-#pragma unroll
-        for (int l = 0; l < DM; ++l) {
-            const float x = cert[l * kTcTileM + src];
-            sc.x = __fmaf_rn(x, g[1 + l].x, sc.x);
-            sc.y = __fmaf_rn(x, g[1 + l].y, sc.y);
-            sc.z = __fmaf_rn(x, g[1 + l].z, sc.z);
-            sc.w = __fmaf_rn(x, g[1 + l].w, sc.w);
+        float b, s2;
+        int bi;
+        quad_score<DM>(rows, cert, lane & 3, src, max(ch, 0), b, s2, bi);
+        if ((lane & 3) == s) {
+            best = b;
+            second = s2;
+            idx = bi;
         }
-        // smallest (lowest point first) and second smallest of the lane's four
-        const bool xy = sc.y < sc.x, zw = sc.w < sc.z;
-        const float m0 = fminf(sc.x, sc.y), m1 = fminf(sc.z, sc.w);
-        const bool hi = m1 < m0;
-        float b = fminf(m0, m1);
-        int bi = hi ? (zw ? 3 : 2) : (xy ? 1 : 0);
-        float s2 = fminf(fmaxf(m0, m1), hi ? fmaxf(sc.z, sc.w) : fmaxf(sc.x, sc.y));
-        bi += ch * kChunk + 4 * q;
-#pragma unroll
-        for (int o = 1; o <= 2; o <<= 1) {
-            const float ob = __shfl_xor_sync(0xFFFFFFFFu, b, o);
-            const float o2 = __shfl_xor_sync(0xFFFFFFFFu, s2, o);
-            const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
-            s2 = fminf(fminf(s2, o2), fmaxf(b, ob));
-            const bool take = ob < b || (ob == b && oi < bi);
-            b = take ? ob : b;
-            bi = take ? oi : bi;
-        }
-        if (q == s) {
+    }
+}
+
+// The chunks of the lanes that want it only, a quad for each, eight at a time: 9% of
+// the searches at d = 8 need a second chunk, so some lane of nearly every warp does,
+// and with all four samples of every quad in turn the kernel took 631 against 582 us for
+// the 1e7 pairs of 50 dates at d = 4.
+template <int DM>
+__device__ __forceinline__ void quad_rescore_some(const float* __restrict__ rows, const float* cert, int lane, bool want,
+                                                  int chunk, float& best, float& second, int& idx)
+{
+    unsigned todo = __ballot_sync(0xFFFFFFFFu, want);
+    const int rank = __popc(todo & ((1u << lane) - 1u));
+    for (int r0 = 0; todo; r0 += 8) {
+        int src = __ffs(todo) - 1;                     // quads without a sample repeat the first
+#pragma unroll 1
+        for (int i = 0; i < 8 && todo; ++i, todo &= todo - 1)
+            if (i == lane >> 2) src = __ffs(todo) - 1;
+        const int ch = __shfl_sync(0xFFFFFFFFu, chunk, src);
+        float b, s2;
+        int bi;
+        quad_score<DM>(rows, cert, lane & 3, src, ch, b, s2, bi);
+        const int from = ((rank - r0) & 7) * 4;
+        b = __shfl_sync(0xFFFFFFFFu, b, from);
+        s2 = __shfl_sync(0xFFFFFFFFu, s2, from);
+        bi = __shfl_sync(0xFFFFFFFFu, bi, from);
+        if (want && rank >= r0 && rank < r0 + 8) {
             best = b;
             second = s2;
             idx = bi;
@@ -185,7 +226,7 @@ __device__ __forceinline__ void quad_rescore(const float* __restrict__ rows, con
 // Bit 0 of the result: the FP32 scores inside do not single out the best; bit 1: a
 // point outside may be nearer.
 __device__ __forceinline__ int tc_uncertified(int d, float A, float best, float S1, float B2tc, float R,
-                                              float inv_sigma)
+                                              float sqrt_d, float sigma, float inv_sigma)
 {
     const float Ap = A * (1.0f + 0x1p-18f);
     const float E1 = cc_bound(d, Ap, R * (1.0f + 0x1p-18f));
@@ -195,7 +236,7 @@ __device__ __forceinline__ int tc_uncertified(int d, float A, float best, float 
     const float rad = fmaxf(A2 + U + 0x1p-18f * (A2 + fabsf(U)) + eta, 0.0f);
     const float rho = Ap + __fsqrt_rn(rad);
     const float lo_in = S1 - cc_bound(d, Ap, rho);
-    const float lo_out = B2tc - tc_bound(d, Ap, rho, inv_sigma);
+    const float lo_out = B2tc - tc_bound(sqrt_d, Ap, rho, sigma, inv_sigma);
     const float rhs = U + eta;
     // additive slack for the FP32 evaluation of both sides
     const bool ok_in = lo_in - rhs > 0x1p-20f * (fabsf(lo_in) + fabsf(rhs)) + eta || lo_in == __int_as_float(0x7F800000);
@@ -647,6 +688,7 @@ __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(cons
     extern __shared__ __align__(128) float dsm_cf[];   // two records
     __shared__ __align__(8) unsigned long long s_full[2];
     __shared__ GridInfo s_G[2];
+    __shared__ float s_sigma[2][2];                    // 2^tc_exp and its inverse
     const int t = threadIdx.x, lane = t & 31;
     const int d = p.d;
     // the screen gave up: its states are not valid
@@ -669,6 +711,7 @@ __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(cons
     __syncthreads();
     int k = -1;
     LayerDesc L;
+    const float sqrt_d = sqrtf((float)d);
     for (long long n = 0;; ++n) {
         const long long item = p.item_lo + blockIdx.x + n * (long long)gridDim.x;
         if (item >= p.item_hi) break;
@@ -679,6 +722,10 @@ __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(cons
             for (int e = t; e < (int)(sizeof(GridInfo) / 4); e += kTcTileM) {
                 reinterpret_cast<int*>(&s_G[0])[e] = reinterpret_cast<const int*>(p.grids + L.gridA)[e];
                 reinterpret_cast<int*>(&s_G[1])[e] = reinterpret_cast<const int*>(p.grids + L.gridB)[e];
+            }
+            if (t < 4) {
+                const int e = p.grids[t < 2 ? L.gridA : L.gridB].tc_exp;
+                s_sigma[t >> 1][t & 1] = ldexpf(1.0f, (t & 1) ? -e : e);
             }
             __syncthreads();
         }
@@ -704,19 +751,19 @@ __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(cons
             const float Araw = cert[DM * kTcTileM + lane];
             const bool big = (__float_as_int(Araw) & (int)0x80000000) != 0;
             const float A = fabsf(Araw);
-            const float inv_sg = ldexpf(1.0f, -Gi.tc_exp), inv2 = inv_sg * inv_sg;
+            const float sg = s_sigma[gr][0], inv_sg = s_sigma[gr][1], inv2 = inv_sg * inv_sg;
             const float second = st[2 * kTcTileM] * inv2, rest = st[3 * kTcTileM] * inv2;
             float best, in2;
             int idx;
             quad_rescore<DM>(rows, cert, lane, c0, best, in2, idx);
             // FP32 inside the best chunk, tensor-core scores outside it
-            int why = tc_uncertified(d, A, best, in2, fminf(second, rest), Gi.R, inv_sg);
+            int why = tc_uncertified(d, A, best, in2, fminf(second, rest), Gi.R, sqrt_d, sg, inv_sg);
             // the second chunk competes: FP32 inside both, tensor-core scores outside
             const bool two = valid && (why & 2) != 0 && c1 != c0;
             if (__any_sync(0xFFFFFFFFu, two)) {
-                float best2, S12;
-                int idx2;
-                quad_rescore<DM>(rows, cert, lane, two ? c1 : c0, best2, S12, idx2);
+                float best2 = 0.0f, S12 = 0.0f;
+                int idx2 = 0;
+                quad_rescore_some<DM>(rows, cert, lane, two, c1, best2, S12, idx2);
                 if (two) {
                     if (best2 < best || (best2 == best && idx2 < idx)) {
                         in2 = fminf(S12, best);
@@ -725,7 +772,7 @@ __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(cons
                     } else {
                         in2 = fminf(in2, best2);
                     }
-                    why = tc_uncertified(d, A, best, in2, rest, Gi.R, inv_sg);
+                    why = tc_uncertified(d, A, best, in2, rest, Gi.R, sqrt_d, sg, inv_sg);
                 }
             }
             const bool rng_ok = idx < Gi.N && !big;
@@ -734,18 +781,19 @@ __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(cons
             // exact FP64 distances for the lanes in `need`, the whole warp for one sample: to
             // the points of the re-scored chunks where no other can be nearer (nearly always:
             // two points tie within the FP32 bound), by the window search of the whole grid
-            // otherwise (100 us of latency for 4000 points)
+            // otherwise (its latency, 32 rounds of loads for 4000 points, ends the kernel)
             unsigned mask = __ballot_sync(0xFFFFFFFFu, need);
             if (mask) {
                 const float* gpf = p.params_f ? p.params_f + (long long)k * p.params_stride : nullptr;
                 const double* gpd = p.params_d ? p.params_d + (long long)k * p.params_stride : nullptr;
                 const double* g64 = p.g64 + Gi.goff * d;
                 const bool inside = (why & 2) == 0 && rng_ok;
+                // an FP64 operation takes a warp as long for one lane as for all that need it
+                double z[DM];
+                if (need) exact_sample<DM>(p, gpf, gpd, k, ms, gr == 1, z);
                 while (mask) {
                     const int src = __ffs(mask) - 1;
                     mask &= mask - 1;
-                    double z[DM];
-                    if (lane == src) exact_sample<DM>(p, gpf, gpd, k, ms, gr == 1, z);
                     int r;
                     if (__shfl_sync(0xFFFFFFFFu, (int)inside, src)) {
                         const int a = __shfl_sync(0xFFFFFFFFu, c0, src), b = __shfl_sync(0xFFFFFFFFu, two ? c1 : c0, src);
