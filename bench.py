@@ -291,14 +291,17 @@ def tensor_roofline(model, units, kern_ms, peaks):
             if "bf16_tflops_sustained" in peaks else "fallback 1.7 PFLOP/s sustained (of fallback)"}
 
 
-def alu_roofline(model, units, kern_ms, peaks, n_sm, pathwise=False):
+def alu_roofline(model, units, kern_ms, peaks, n_sm, pathwise=False, automatic=False):
     """FP32 screen against the FP32 FMA lanes (SMs x 128 lanes x 2 flops x max clock)."""
     sm_max = peaks.get("sm_max_mhz", 2070.0)
     peak = 2.0 * FP32_LANES_PER_SM * n_sm * sm_max * 1e6 / 1e12
     work = flops_per_sample_layer(model, pathwise)
     ach = work * units / (kern_ms / 1e3) / 1e12
+    # the located search (automatic form, d <= 2, at most 1024 points) evaluates one to
+    # four of the candidates: there the figure is a rate of answers, not the pipe's share
+    located = automatic and model.d <= 2 and int(max(model.N)) <= 1024
     return {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-            "kernel_ms": kern_ms,
+            "kernel_ms": kern_ms, "basis": "brute-force candidates" if located else "candidates evaluated",
             "work": f"{work:.0f} flops per sample.layer (2d per candidate, "
                     f"{candidates_per_sample_layer(model, pathwise):.0f} candidates)",
             "peak_basis": f"FP32 FMA lanes: {n_sm} SMs x {FP32_LANES_PER_SM} x 2 flops x {sm_max:.0f} MHz"}
@@ -361,7 +364,7 @@ def extra_workloads(ctx, B, dev, stream, flush, peaks, n_sm):
             r["tc_draw"] = {1: "draw pass", 2: "in the screen kernel"}.get(st.tc_draw)
             r["roofline"] = tensor_roofline(model, units, kmean, peaks)
         else:
-            r["roofline"] = alu_roofline(model, units, kmean, peaks, n_sm, pathwise)
+            r["roofline"] = alu_roofline(model, units, kmean, peaks, n_sm, pathwise, o.form == B.FORM_AUTO)
         del counts
         torch.cuda.empty_cache()
         return r, g
