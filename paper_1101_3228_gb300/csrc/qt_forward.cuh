@@ -612,8 +612,9 @@ __device__ __noinline__ int warp_window_nn(const float (&xs)[DM], float A, const
             i1 = oi;
         }
     }
-    // window bound (same bounds as the certificate, with slack)
-    const float* r = recs + (long long)i1 * F;
+    // window bound (same bounds as the certificate, with slack); i1 is no record when every
+    // score overflows or is undefined
+    const float* r = recs + (long long)min(i1, N - 1) * F;
     float n2 = 0.0f;
 #pragma unroll
     for (int l = 0; l < DM; ++l) n2 = __fmaf_rn(r[1 + l], r[1 + l], n2);
@@ -628,21 +629,27 @@ __device__ __noinline__ int warp_window_nn(const float (&xs)[DM], float A, const
     const float rho = Ap + __fsqrt_rn(rad);
     const float Erho = cd * (rho * rho + 2.0f * Ap * rho);
     const float lim = b1 + (E1 + Erho + eta) * 1.25f + 0x1p-20f * fabsf(b1) + 0x1p-100f;
-    // exact distances on the window only
+    // exact distances on the window only; on every record where the scores bound nothing (a
+    // sample so far out that they overflow).  A sample with no finite distance has no cell:
+    // the index returned is out of range, and the callers refuse it
+    constexpr int kNone = 0x7FFFFFFF;
+    const bool all = i1 >= N || !(lim < __int_as_float(0x7F800000));
     double best = __longlong_as_double(0x7FF0000000000000LL);
-    int bi = 0x7FFFFFFF;
+    int bi = kNone;
     double zz[DM];
 #pragma unroll
     for (int l = 0; l < DM; ++l) zz[l] = __shfl_sync(0xFFFFFFFFu, z[l], src);
     auto exact = [&](int j) {
         const double dj = dist64<DM>(zz, g64 + (long long)j * d, d);
-        if (dj < best || (dj == best && j < bi)) {
+        if (dj < best || (dj == best && j < bi && bi != kNone)) {
             best = dj;
             bi = j;
         }
     };
-    if (!__any_sync(0xFFFFFFFFu, l3 <= lim)) {
-        if (l1 <= lim) exact(k1);
+    if (all) {
+        for (int j = lane; j < N; j += 32) exact(j);
+    } else if (!__any_sync(0xFFFFFFFFu, l3 <= lim)) {
+        if (l1 <= lim) exact(k1);                      // lim is finite: a lane's own record
         if (l2 <= lim) exact(k2);
     } else {
         for (int j0 = lane; j0 < N; j0 += 32 * kU) {
