@@ -704,8 +704,9 @@ __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(cons
     __shared__ float s_sigma[2][2];                    // 2^tc_exp and its inverse
     const int t = threadIdx.x, lane = t & 31;
     const int d = p.d;
-    // the screen gave up: its states are not valid
-    if (*((volatile int32_t*)&p.status->code) != 0) return;
+    // the screen gave up: its states are not valid.  One answer for the whole CTA: another
+    // CTA may be recording an error while this one starts
+    if (__syncthreads_or(*((volatile int32_t*)&p.status->code) != 0)) return;
     const uint32_t full = smem_u32(&s_full[0]), buf = smem_u32(dsm_cf);
     auto load = [&](long long n) {
         const long long item = p.item_lo + blockIdx.x + n * (long long)gridDim.x;
@@ -742,10 +743,11 @@ __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(cons
             }
             __syncthreads();
         }
-        // the records were written by earlier kernels: the copy always lands
-        if (!mbar_wait_bounded(full + (uint32_t)(8 * (n & 1)), (uint32_t)((n >> 1) & 1), kDrainUs))
-        {
+        // the records were written by earlier kernels: the copy always lands (if it did not,
+        // the copy of the next item is waited for too before the CTA leaves)
+        if (!mbar_wait_bounded(full + (uint32_t)(8 * (n & 1)), (uint32_t)((n >> 1) & 1), kDrainUs)) {
             record_error(p.status, 4 /* QT_ETIMEOUT */, 27);
+            mbar_wait_bounded(full + (uint32_t)(8 * ((n + 1) & 1)), (uint32_t)(((n + 1) >> 1) & 1), 1000000);
             return;
         }
         const float* rec = dsm_cf + (n & 1) * TcItem<DM>::kFloats;

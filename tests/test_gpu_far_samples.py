@@ -65,3 +65,17 @@ def test_undefined_samples_are_refused(ctx, B, form, d, bad):
     # the context stays usable
     counts, _, _, _ = ctx.counts_from_samples(_dev(g), _dev(g), _dev(X), _dev(X), B.options(form=getattr(B, form)))
     np.testing.assert_array_equal(counts.cpu().numpy(), oracle.counts_from_samples(g, g, X, X))
+
+
+def test_refusal_while_other_blocks_start(ctx, B):
+    """Errors recorded by the first blocks of the tensor-core form's last kernel while others
+    begin: every block takes one decision, and the call ends with the refusal, not a timeout."""
+    d, M = 3, 400000
+    rng = np.random.default_rng(5)
+    g = rng.standard_normal((50, d))
+    X = rng.standard_normal((M, d))
+    X[::97, 0] = np.nan
+    for _ in range(20):
+        with pytest.raises(B.QtError) as e:
+            ctx.counts_from_samples(_dev(g), _dev(g), _dev(X), _dev(X), B.options(form=B.FORM_TC_RECHECK))
+        assert e.value.status == B.QT_EDEVICE
