@@ -232,14 +232,14 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         if (cnt <= kCellInline) {
             ent |= (uint64_t)cnt << 60;
         } else {
-            const uint32_t off = atomicAdd(p.cell_cursor, (uint32_t)cnt);
-            if (off + (uint32_t)cnt <= p.cell_pool_cap && off + (uint32_t)cnt >= off) {
+            const unsigned long long off = atomicAdd(p.cell_cursor, (unsigned long long)cnt);
+            if (pool_holds(off, (uint32_t)cnt, p.cell_pool_cap)) {
                 int w = 0;
                 for (int t = 0; t < ns; ++t) {
                     const int j = surv[t];
                     if (keeps(j)) p.cell_pool[off + w++] = (uint16_t)j;
                 }
-                ent = (uint64_t)off | ((uint64_t)cnt << 32) | ((uint64_t)kCellPool << 60);
+                ent = off | ((uint64_t)cnt << 32) | ((uint64_t)kCellPool << 60);
             } else {
                 ent = kCellScanEntry;
             }
@@ -378,6 +378,10 @@ __global__ void __launch_bounds__(kCellThreads, 1) forward_cells_kernel(const __
         if (needA) i = cell_recheck<DM>(p, s_pf, s_pd, k, m, false, eA, s_GA);
         if (needB) j = cell_recheck<DM>(p, s_pf, s_pd, k, m, true, eB, s_GB);
         // ---- counters p^k_ij (Sec. 3.3), per-sample cells, dumps
+        if ((unsigned)i >= (unsigned)s_L.NA || (unsigned)j >= (unsigned)s_L.NB) {
+            record_error(p.status, 6 /* QT_EDEVICE */, 52);
+            continue;
+        }
         if (hist_live) atomicAdd(&hist[i * s_L.NB + j], 1u);
         else count_add(p.counts, p.counts_u32, s_L.coff + (long long)i * s_L.NB + j, 1u);
         if (MODE == 2 && p.cellsA) {

@@ -29,9 +29,18 @@ struct DevStatus {
     unsigned long long candidates; // candidate distances (router form)
     unsigned long long done_items; // work items finished
     unsigned long long spare[4];   // [0]: router grid checksum; [1..3]: diagnostics
-    uint32_t cell_cursor;          // located search: pool words taken by the tables
-    uint32_t pad;
+    unsigned long long cell_cursor;// located search: pool words that the tables asked for
 };
+
+// Whether a list of cnt words at offset off, both as taken from the cursor, lies in a
+// pool of cap words.  The cursor counts on after the pool is full; 64 bits, because the
+// words asked for can pass 2^32 (a bin whose candidates are all of 1024 points, 10816
+// bins a grid: about 400 grids), and a cursor that starts again at 0 would hand out words
+// that other bins refer to.
+__host__ __device__ constexpr bool pool_holds(unsigned long long off, uint32_t cnt, uint32_t cap)
+{
+    return off + cnt <= cap;
+}
 
 // One layer pair (k, k+1) of the forward step.
 struct LayerDesc {
@@ -152,7 +161,7 @@ struct ForwardParams {
     unsigned long long* cell_tab;  // bin entries of every grid
     float* cell_rec;               // centred FP32 points of every grid
     uint16_t* cell_pool;           // candidate lists longer than an entry
-    uint32_t* cell_cursor;         // pool words taken
+    unsigned long long* cell_cursor; // pool words asked for
     uint32_t cell_pool_cap;        // pool words
     int32_t cell_g0, cell_g1;      // grids [g0, g1) to build
     const float* cell_near;        // [n][kCellNearStride] combined FP32 parameters of FP64 layers

@@ -125,6 +125,11 @@ __global__ void __launch_bounds__(kCellThreads, 1) path_cells_kernel(const __gri
                         j = cell_exact<DM>(z, e, p.cell_pool, p.g64 + G.goff * DM, N, DM);
                     }
                 }
+                if ((unsigned)j >= (unsigned)N) {
+                    record_error(p.status, 6 /* QT_EDEVICE */, 53);
+                    cell[s] = 0;
+                    continue;
+                }
                 if (k >= 0) count_add(p.counts, p.counts_u32, coff + (long long)cell[s] * N + j, 1u);
                 if (row >= 0) {
                     for (int l = 0; l < DM; ++l) p.dumpY[row * DM + l] = (double)x[s][l];

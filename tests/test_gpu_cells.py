@@ -176,3 +176,19 @@ def test_located_fused_price_and_timeouts(ctx, B):
             call(model, _dev(g), model.M, model.seed, B.options(spin_budget=-1))
         assert e.value.status == B.QT_ETIMEOUT
         call(model, _dev(g), model.M, model.seed)
+
+
+def test_located_full_pool(ctx, B):
+    """More long candidate lists than the pool holds: nearly every point of 40 grids in one
+    bin's width, so that every bin of them keeps all of these points."""
+    n, N, M = 40, 1024, 501
+    rng = np.random.default_rng(9)
+    model, _ = _chain(2, n, [N] * n, M)
+    g = 1e-7 * rng.standard_normal((int(model.N.sum()), 2))
+    g[1::N] += 1.0
+    ref = oracle.transitions(model, g, M, model.seed, W.PREC_F32)
+    counts, st, _ = ctx.transitions(model, _dev(g), M, model.seed)
+    got = B.split_counts(model.N, counts.cpu().numpy())
+    for k in range(n):
+        np.testing.assert_array_equal(got[k], ref[k], err_msg=f"layer {k}")
+    assert st.device_status == 0
