@@ -131,7 +131,9 @@ __device__ __forceinline__ int cell_search(const CellGrid& G, const unsigned cha
     return idx;
 }
 
-// Exact FP64 argmin over a bin's candidates (lowest index among equal distances).
+// Exact FP64 argmin over a bin's candidates (lowest index among equal distances).  A
+// sample without a finite distance has no cell: the index is out of range, and the callers
+// refuse it, as in the other forms.
 template <int DM>
 __device__ __noinline__ int cell_exact(const double (&z)[DM], uint64_t e, const uint16_t* __restrict__ pool,
                                        const double* __restrict__ g64, int N, int d)
@@ -139,7 +141,7 @@ __device__ __noinline__ int cell_exact(const double (&z)[DM], uint64_t e, const 
     const int kind = (int)(e >> 60);
     const int cnt = kind == kCellScan ? N : (kind == kCellPool ? (int)((e >> 32) & 0xFFFFu) : kind);
     double best = __longlong_as_double(0x7FF0000000000000LL);
-    int bi = 0;
+    int bi = 0x7FFFFFFF;
     for (int q = 0; q < cnt; ++q) {
         const int j = kind == kCellScan ? q
                                         : (kind == kCellPool ? (int)pool[(uint32_t)e + q] : (int)((e >> (10 * q)) & 1023u));

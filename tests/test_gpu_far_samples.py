@@ -29,8 +29,8 @@ def _dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
-FORMS = [("FORM_F32_RECHECK", 1), ("FORM_F32_RECHECK", 2), ("FORM_F32_RECHECK", 12), ("FORM_TC_RECHECK", 3),
-         ("FORM_TC_RECHECK", 8)]
+FORMS = [("FORM_AUTO", 1), ("FORM_AUTO", 2), ("FORM_F32_RECHECK", 1), ("FORM_F32_RECHECK", 2),
+         ("FORM_F32_RECHECK", 12), ("FORM_TC_RECHECK", 3), ("FORM_TC_RECHECK", 8)]
 
 
 @pytest.mark.parametrize("form,d", FORMS)
