@@ -16,6 +16,7 @@
 
 #include "../../include/qt.h"
 #include "qt_internal.h"
+#include "qt_near.h"
 #include "qt_launch.h"
 
 namespace qt {
@@ -984,42 +985,18 @@ void key_append(std::vector<unsigned char>& k, const void* p, size_t n)
     k.insert(k.end(), b, b + n);
 }
 
-// FP64 layers of the located search: the pair (X - mu_A, Y - mu_B) as FP32 maps of
-// the normals, combined in FP64 (block layout: pair_near in qt_cells.cuh), and each
-// grid's bound on the resulting error: the normals' (2^-20 of their radius, at most
-// 8.6) through the maps, and a few FP32 roundings.
+// FP64 layers of the located search: the FP32 maps of every layer and each grid's error
+// bounds (qt_near.h).
 void combine_near(const Plan& P, const double* params, float* out, CellGrid* cells)
 {
-    const int d = P.d;
     for (int k = 0; k < P.n; ++k) {
-        const double* p = params + (long long)k * P.pstride;
-        const double *m = p, *b = p + d, *L = p + 2 * d, *A = L + d * d, *T = A + d * d;
-        float* o = out + (long long)k * kCellNearStride;
-        memset(o, 0, kCellNearStride * sizeof(float));
-        float *cA = o, *oL = o + d, *cB = oL + d * d, *oAL = cB + d, *oT = oAL + d * d;
-        const CellGrid& GA = P.cells[k];
-        const CellGrid& GB = P.cells[k + 1];
-        double errA = 0.0, errB = 0.0;
-        for (int l = 0; l < d; ++l) {
-            const double a = m[l] - (double)GA.mu[l];
-            double c = b[l] - (double)GB.mu[l], sa = 0.0, sb = 0.0;
-            for (int q = 0; q < d; ++q) {
-                c += A[l * d + q] * m[q];
-                double al = 0.0;
-                for (int r = 0; r < d; ++r) al += A[l * d + r] * L[r * d + q];
-                oL[l * d + q] = (float)L[l * d + q];
-                oAL[l * d + q] = (float)al;
-                oT[l * d + q] = (float)T[l * d + q];
-                sa += std::fabs(L[l * d + q]);
-                sb += std::fabs(al) + std::fabs(T[l * d + q]);
-            }
-            cA[l] = (float)a;
-            cB[l] = (float)c;
-            errA = std::max(errA, 8.6 * sa * 0x1.6p-20 + std::fabs(a) * 0x1p-22);
-            errB = std::max(errB, 8.6 * sb * 0x1.6p-20 + std::fabs(c) * 0x1p-22);
-        }
-        cells[k].err = std::max(cells[k].err, (float)(1.01 * errA));
-        cells[k + 1].err = std::max(cells[k + 1].err, (float)(1.01 * errB));
+        NearBound A, B;
+        near_layer(P.d, params + (long long)k * P.pstride, P.cells[k].mu, P.cells[k + 1].mu,
+                   out + (long long)k * kCellNearStride, A, B);
+        cells[k].err = std::max(cells[k].err, (float)A.grows);
+        cells[k].err0 = std::max(cells[k].err0, (float)A.fixed);
+        cells[k + 1].err = std::max(cells[k + 1].err, (float)B.grows);
+        cells[k + 1].err0 = std::max(cells[k + 1].err0, (float)B.fixed);
     }
 }
 

@@ -174,10 +174,17 @@ __device__ __forceinline__ void cell_stage(const ForwardParams& p, const CellGri
 // FP64 samples cost the FP64 pipe about 250 operations a pair, at 1/64 of the
 // FP32 rate: 3.0 ms for the 10^7 pairs of the 1-d workload.  The cells of nearly
 // all of them need far fewer digits: the pair is drawn from the same Philox words
-// with FP32 logarithm, square root, sine and cosine (each normal within
-// 2^-20 times its radius, radius <= 8.6), mapped by matrices already combined and
-// centred in FP64 on the host, and the certificate carries that error; the
-// uncertified few are drawn again in FP64.
+// with FP32 logarithm, square root, sine and cosine, mapped by matrices already
+// combined and centred in FP64 on the host, and the certificate carries the error
+// (qt_near.h); the uncertified few are drawn again in FP64.
+//
+// Each normal lies within 2^-20 of its radius, radius <= 8.6.  The logarithm: s has the
+// roundings of f - 1, f + 1 and the division (2 ulp), 1.5 2^-22 in all, so ln f is within
+// 1.75 2^-22 of itself, |ln f| < 0.35; where u <= 0.7071 (-ln u > 0.346) u's rounding and
+// e ln 2 add 2.1 2^-24: 3.2 2^-22 of -ln u at its smallest, half of that after the square
+// root, 0.47 2^-20 with its rounding.  The angle, truncated and rounded to FP32, is within
+// 1.6 2^-24 and the polynomials within 1.5 2^-24: 0.19 2^-20.  0.72 2^-20 with the last
+// product; 2^24 pairs and the extreme words stay below 2^-20 (tests/cuda/near_normals.cu).
 
 __device__ __forceinline__ float box_muller_near(const Philox4& w, float& g0, float& g1)
 {

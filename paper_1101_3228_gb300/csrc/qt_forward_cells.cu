@@ -102,10 +102,11 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         hmin = fminf(hmin, h[l]);
     }
     const float S = (__fsqrt_rn(A2) + R) * 1.0001f;
-    const float er = 0x1p-24f * 1.01f * S, e = er + G.err;
+    const float er = 0x1p-24f * 1.01f * S + G.err0, e = er + G.err;
     // the enlarged bins must cover the error of the centred sample and of its bin number
-    const bool usable = 32.0f * (G.err + 0x1p-21f * S) <= hmin;
-    const float marg = 0x1p-18f * S * S;
+    const bool usable = 32.0f * (G.err + G.err0 + 0x1p-21f * S) <= hmin;
+    // (floors here and in c2: products of the smallest grids fall out of FP32's range)
+    const float marg = 0x1p-18f * S * S + 0x1p-120f;
     if (blockIdx.y == 0 && tid == 0) {
         const float sq = DM == 1 ? 1.0f : 1.41421357f;
         const float kappa = fmaxf(0x1p-22f, e / (2.0f * hmin));
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         }
         G.c1 = 2.02f * sq * kappa;
         G.inv_span = 1.0f / S;
-        G.c2 = 2.02f * (sq * (e / kappa) * e + (float)DM * e * e);
+        G.c2 = 2.02f * (sq * (e / kappa) * e + (float)DM * e * e) + 0x1p-120f * (e / er);
         G.c3 = 2.02f * (float)(DM + 6) * 0x1p-24f;
         G.f0 = er / e;
     }

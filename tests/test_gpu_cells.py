@@ -192,3 +192,42 @@ def test_located_full_pool(ctx, B):
     for k in range(n):
         np.testing.assert_array_equal(got[k], ref[k], err_msg=f"layer {k}")
     assert st.device_status == 0
+
+
+@pytest.mark.parametrize("d", [1, 2])
+def test_located_fp64_pairs_at_the_draws_own_rounding(ctx, B, d):
+    """Scale 1e-9 about 100: the FP64 draw moves in steps of 1.4e-14, 10^-5 of the scale, so
+    that some samples tie between two points exactly; the FP32 stand-in must not decide them."""
+    M = 2 * 10**6
+    model, _ = _chain(d, 2, (2, 3), M, 1e-9, 100.0)
+    g = np.full((6, d), 100.0)
+    g[1, 0] -= 2.0**-30
+    g[2, 0] += 2.0**-30
+    g[3, 0] -= 2.0**-29
+    g[5, 0] += 2.0**-29
+    ref = oracle.transitions(model, g, M, model.seed, W.PREC_F64)
+    counts, st, _ = ctx.transitions(model, _dev(g), M, model.seed, B.options(prec=B.PREC_F64))
+    got = B.split_counts(model.N, counts.cpu().numpy())
+    for k in range(model.n):
+        np.testing.assert_array_equal(got[k], ref[k], err_msg=f"layer {k}")
+
+
+@pytest.mark.parametrize("d", [1, 2])
+@pytest.mark.parametrize("spread", [1.0, 1e-5])
+def test_located_fp64_pairs_off_the_next_mean(ctx, B, d, spread):
+    """Marginal means that do not follow from each other (m_{k+1} != A m_k + b): the constant
+    of the map is large against the normals' part, and its rounding does not shrink with
+    their radius.  The grid of the next layer lies where the samples go."""
+    M, n, N = 200003, 2, 60
+    rng = np.random.default_rng(11)
+    model, _ = _chain(d, n, (N, N), M, spread)
+    m = model.m + np.array([0.0, 1.0, -0.7])[:, None]
+    model = W.Model("off", d, n, model.N, model.A, model.b, model.T, m, model.L, model.t, 0.0, "put_exp1d", 1.0,
+                    None, M, 99, W.PREC_F64, "kmeans")
+    g = np.concatenate([m[:1], (model.A[0] @ m[0] + model.b[0]) + spread * 0.4 * rng.standard_normal((N, d)),
+                        (model.A[1] @ m[1] + model.b[1]) + spread * rng.standard_normal((N, d))])
+    ref = oracle.transitions(model, g, M, model.seed, W.PREC_F64)
+    counts, _, _ = ctx.transitions(model, _dev(g), M, model.seed, B.options(prec=B.PREC_F64))
+    got = B.split_counts(model.N, counts.cpu().numpy())
+    for k in range(n):
+        np.testing.assert_array_equal(got[k], ref[k], err_msg=f"layer {k}")
