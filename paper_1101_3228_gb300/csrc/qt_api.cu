@@ -819,6 +819,15 @@ bool stream_is_capturing(cudaStream_t st)
     return cs != cudaStreamCaptureStatusNone;
 }
 
+// The forward step's workspace is the last step's until that has ended, on whatever
+// stream: nothing that a step still running may read is written before this.
+qt_status workspace_wait(qt_ctx* ctx, cudaStream_t st, bool capturing)
+{
+    if (capturing) QT_CUDA(cudaEventSynchronize(ctx->ev_tables));
+    else QT_CUDA(cudaStreamWaitEvent(st, ctx->ev_tables, 0));
+    return QT_OK;
+}
+
 // Enqueue the whole forward step on `st`: table upload, zeroing, record
 // preparation, the persistent kernel.
 qt_status enqueue_forward(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long M, unsigned long long seed,
@@ -1054,9 +1063,7 @@ qt_status run_plan(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long M, uns
     }
     const bool replay = use_graph && ctx->gexec && key == ctx->gkey;
     const bool capturing = stream_is_capturing(st);
-    // the workspace is the last step's until that has ended (on whatever stream)
-    if (capturing) QT_CUDA(cudaEventSynchronize(ctx->ev_tables));
-    else QT_CUDA(cudaStreamWaitEvent(st, ctx->ev_tables, 0));
+    if ((s = workspace_wait(ctx, st, capturing))) return s;
     if (!replay) {
         // A step is launched directly the first time and captured when the same call
         // comes again: instantiating a graph costs 60 us, more than it saves a caller
@@ -1352,7 +1359,7 @@ extern "C" qt_status qt_counts_from_samples(qt_ctx* ctx, int32_t d, const double
     // both grids contiguous in one workspace buffer
     void* dg;
     qt_status s = dev_get(ctx, "pair_grids", sizeof(double) * (size_t)(NA + NB) * d, &dg);
-    if (s) return s;
+    if (s || (s = workspace_wait(ctx, st, stream_is_capturing(st)))) return s;
     QT_CUDA(cudaMemcpyAsync(dg, gA, sizeof(double) * NA * d, cudaMemcpyDeviceToDevice, st));
     QT_CUDA(cudaMemcpyAsync((double*)dg + NA * d, gB, sizeof(double) * NB * d, cudaMemcpyDeviceToDevice, st));
     // centres of the screen: zero (the bound uses the norms about this centre)
