@@ -245,6 +245,10 @@ QT_API qt_status qt_counts_from_samples(qt_ctx* ctx, int32_t d, const double* gA
  * (sum_j p^k_ij V_{k+1}(j)) / p^k_i in FP64, j summed (one fused multiply-add
  * each) in lanes j mod 32 and
  * combined by a fixed butterfly, so results are bitwise reproducible.
+ * A small tree (n >= 3, N_k <= 1024) runs in one launch whose blocks wait for
+ * one another's values, each wait bounded by 10 s (in qt_price by
+ * opts->spin_budget); one that runs out leaves NaN in the values that depend on
+ * it, and qt_get_status (qt_price itself) returns QT_ETIMEOUT.
  *   N      host int64 [n+1]
  *   counts dev, counts_type elements, concatenated as in qt_transitions
  *   phi, V dev FP64 [sum_k N_k] (V written)                                    */
@@ -282,7 +286,8 @@ QT_API qt_status qt_price(qt_ctx* ctx, const qt_model* model, const double* grid
                    qt_stats* stats, void* stream);
 
 /* Synchronise the stream and return the device status of the last forward
- * call on this context (QT_OK, QT_ETIMEOUT or QT_EDEVICE).                    */
+ * call on this context and of the qt_backward after it (QT_OK, QT_ETIMEOUT or
+ * QT_EDEVICE).                                                                */
 QT_API qt_status qt_get_status(qt_ctx* ctx, void* stream, qt_stats* stats);
 
 /* Device bytes the context will allocate for a qt_transitions call of this

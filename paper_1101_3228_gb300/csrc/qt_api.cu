@@ -25,7 +25,8 @@ cudaError_t launch_backward_layer(const void* counts, int u32, long long coff, i
                                   const double* Vnext, double* Vk, int num_sms, cudaStream_t st);
 bool backward_tree_fits(int n, const int64_t* N, int num_sms);
 cudaError_t launch_backward_tree(const void* counts, int u32, int n, int maxN, const void* layers, const double* phi,
-                                 double* V, double* X, int num_sms, cudaStream_t st);
+                                 double* V, double* X, DevStatus* status, long long budget_us, int num_sms,
+                                 cudaStream_t st);
 int backward_tree_blocks(int maxN, int num_sms);
 __global__ void root_price_kernel(const void*, int, int, int, const double*, double*);
 __global__ void fold_status_kernel(const DevStatus*, DevStatus*);
@@ -92,6 +93,8 @@ struct qt_ctx {
     int last_launches = 0;             // kernels enqueued by the last forward step
     int last_tc_draw = 0;              // sample-draw layout of the last tensor-core step
     void* status_buf = nullptr;   // status block of the last forward call
+    void* tree_status = nullptr;  // that of the one-launch backward induction after it, if any
+    DevStatus* status_host = nullptr;   // pinned: both as read
 };
 
 namespace {
@@ -149,6 +152,13 @@ int injected_timeout_layer()
     const char* f = getenv("QT_FAULT");
     if (!f || strncmp(f, "timeout_layer:", 14) != 0) return -1;
     return atoi(f + 14);
+}
+
+// QT_FAULT=timeout_tree gives the one-launch backward induction a negative wait budget.
+bool injected_timeout_tree()
+{
+    const char* f = getenv("QT_FAULT");
+    return f && strcmp(f, "timeout_tree") == 0;
 }
 
 qt_status dev_get(qt_ctx* ctx, const char* name, size_t bytes, void** out)
@@ -266,6 +276,7 @@ extern "C" qt_status qt_create(qt_ctx** out, int32_t device)
         cudaEventCreateWithFlags(&ctx->ev_tree, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_up_tree[0], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_up_tree[1], cudaEventDisableTiming) != cudaSuccess ||
+        cudaMallocHost(&ctx->status_host, 2 * sizeof(DevStatus)) != cudaSuccess ||
         cudaEventCreate(&ctx->ev_k0) != cudaSuccess || cudaEventCreate(&ctx->ev_k1) != cudaSuccess) {
         delete ctx;
         return QT_ECUDA;
@@ -284,6 +295,7 @@ extern "C" qt_status qt_destroy(qt_ctx* ctx)
         if (kv.second.p) cudaFree(kv.second.p);
     for (auto& kv : ctx->host)
         if (kv.second.p) cudaFreeHost(kv.second.p);
+    if (ctx->status_host) cudaFreeHost(ctx->status_host);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->ev_tables) cudaEventDestroy(ctx->ev_tables);
     if (ctx->ev_tree) cudaEventDestroy(ctx->ev_tree);
@@ -962,11 +974,16 @@ qt_status enqueue_forward(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long
 
 qt_status read_status(qt_ctx* ctx, cudaStream_t st, qt_stats* stats, long long samples, long long searches)
 {
-    void* dstatus = ctx->status_buf;
-    DevStatus hs;
-    memset(&hs, 0, sizeof hs);
+    DevStatus* const h = ctx->status_host;
+    memset(h, 0, 2 * sizeof *h);
+    if (ctx->status_buf) QT_CUDA(cudaMemcpyAsync(&h[0], ctx->status_buf, sizeof *h, cudaMemcpyDeviceToHost, st));
+    if (ctx->tree_status) QT_CUDA(cudaMemcpyAsync(&h[1], ctx->tree_status, sizeof *h, cudaMemcpyDeviceToHost, st));
     QT_CUDA(cudaStreamSynchronize(st));
-    if (dstatus) QT_CUDA(cudaMemcpy(&hs, dstatus, sizeof hs, cudaMemcpyDeviceToHost));
+    DevStatus hs = h[0];
+    if (hs.code == 0 && h[1].code != 0) {
+        hs.code = h[1].code;
+        hs.where = h[1].where;
+    }
     if (stats) {
         stats->samples = samples;
         stats->searches = searches;
@@ -1209,6 +1226,7 @@ qt_status forward_common(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
         o = &oi;
     }
     Plan P;
+    ctx->tree_status = nullptr;
     qt_status s = make_plan(ctx, d, n, Ns, mus, M, o, source == kArrays, P, only_layer, algo);
     if (s) return s;
     P.euler = euler;
@@ -1413,10 +1431,11 @@ extern "C" qt_status qt_transitions_workspace(const qt_model* model, const qt_op
 
 // ------------------------------------------------------------------ backward induction and price
 
-extern "C" qt_status qt_backward(qt_ctx* ctx, int32_t n, const int64_t* N, const void* counts, int32_t counts_type,
-                                 const double* phi, double* V, void* stream)
+namespace {
+// qt_backward with the bound of the waits inside its kernels (microseconds, 0 = 10 s)
+qt_status backward_impl(qt_ctx* ctx, int32_t n, const int64_t* N, const void* counts, int32_t counts_type,
+                        const double* phi, double* V, long long spin_budget, void* stream)
 {
-    if (!ctx) return QT_EINVAL;
     if (n < 1 || !N || !counts || !phi || !V) return fail(ctx, QT_EINVAL, "bad arguments to qt_backward");
     if (counts_type != QT_COUNTS_I64 && counts_type != QT_COUNTS_U32)
         return fail(ctx, QT_EINVAL, "counts_type %d", counts_type);
@@ -1428,10 +1447,14 @@ extern "C" qt_status qt_backward(qt_ctx* ctx, int32_t n, const int64_t* N, const
     for (int k = 0; k <= n; ++k) goff[k + 1] = goff[k] + N[k];
     for (int k = 0; k < n; ++k) coff[k + 1] = coff[k] + N[k] * N[k + 1];
     const int u32 = counts_type == QT_COUNTS_U32;
+    ctx->tree_status = nullptr;
     if (backward_tree_fits(n, N, ctx->num_sms) && !stream_is_capturing(st)) {
         // a small tree in one launch.  Its layer table and the exchange of its CTAs are
-        // the context's: a call on another stream waits for the last one
-        const size_t bytes = sizeof(TreeLayer) * (size_t)(n + 1);
+        // the context's: a call on another stream waits for the last one.  A zeroed status
+        // block goes up ahead of the table
+        constexpr size_t kHead = 128;
+        static_assert(sizeof(DevStatus) <= kHead, "status block");
+        const size_t bytes = kHead + sizeof(TreeLayer) * (size_t)(n + 1);
         int maxN = 1;
         for (int k = 0; k <= n; ++k) maxN = std::max(maxN, (int)N[k]);
         const size_t xb = sizeof(double) * 8 * (size_t)n * backward_tree_blocks(maxN, ctx->num_sms);
@@ -1447,14 +1470,18 @@ extern "C" qt_status qt_backward(qt_ctx* ctx, int32_t n, const int64_t* N, const
         if (s == QT_OK) {
             QT_CUDA(cudaEventSynchronize(ctx->ev_up_tree[ctx->up_tree]));
             QT_CUDA(cudaStreamWaitEvent(st, ctx->ev_tree, 0));
-            TreeLayer* tl = (TreeLayer*)ht;
+            memset(ht, 0, kHead);
+            TreeLayer* tl = (TreeLayer*)((unsigned char*)ht + kHead);
+            const long long budget = injected_timeout_tree() ? -1 : spin_budget == 0 ? 10000000ll : spin_budget;
             for (int k = 0; k <= n; ++k) tl[k] = TreeLayer{coff[k], goff[k], (int)N[k], 0};
             QT_CUDA(cudaMemcpyAsync(dt, ht, bytes, cudaMemcpyHostToDevice, st));
             QT_CUDA(cudaEventRecord(ctx->ev_up_tree[ctx->up_tree], st));
             ctx->up_tree ^= 1;
             const cudaError_t e =
-                launch_backward_tree(counts, u32, n, maxN, dt, phi, V, (double*)dx, ctx->num_sms, st);
+                launch_backward_tree(counts, u32, n, maxN, (unsigned char*)dt + kHead, phi, V, (double*)dx,
+                                     (DevStatus*)dt, budget, ctx->num_sms, st);
             QT_CUDA(cudaEventRecord(ctx->ev_tree, st));
+            ctx->tree_status = dt;
             if (e != cudaErrorCooperativeLaunchTooLarge) {
                 QT_CUDA(e);
                 return QT_OK;
@@ -1468,6 +1495,14 @@ extern "C" qt_status qt_backward(qt_ctx* ctx, int32_t n, const int64_t* N, const
         QT_CUDA(launch_backward_layer(counts, u32, coff[k], (int)N[k], (int)N[k + 1], phi + goff[k], V + goff[k + 1],
                                       V + goff[k], ctx->num_sms, st));
     return QT_OK;
+}
+}  // namespace
+
+extern "C" qt_status qt_backward(qt_ctx* ctx, int32_t n, const int64_t* N, const void* counts, int32_t counts_type,
+                                 const double* phi, double* V, void* stream)
+{
+    if (!ctx) return QT_EINVAL;
+    return backward_impl(ctx, n, N, counts, counts_type, phi, V, 0, stream);
 }
 
 extern "C" qt_status qt_swing(qt_ctx* ctx, int32_t n, const int64_t* N, const void* counts, int32_t counts_type,
@@ -1564,7 +1599,8 @@ extern "C" qt_status qt_price(qt_ctx* ctx, const qt_model* model, const double* 
     }
     if (!fused) {
         if ((s = qt_transitions(ctx, model, dgrids, M, seed, &o, dcounts, nullptr, nullptr, stream))) return s;
-        if ((s = qt_backward(ctx, n, model->N, dcounts, o.counts_type, dphi, (double*)dV, stream))) return s;
+        if ((s = backward_impl(ctx, n, model->N, dcounts, o.counts_type, dphi, (double*)dV, o.spin_budget, stream)))
+            return s;
     } else {
         // layers in reverse order: the counts of pair (k, k + 1), then V_k from
         // them and V_{k+1} at once (the same kernels and arithmetic as the

@@ -274,7 +274,8 @@ cudaError_t launch_backward_layer(const void* counts, int u32, long long coff, i
 //    every third layer, put the non-zero ones aside and prepare the reciprocal of the row
 //    sum, one to three layers ahead of the consumer warps, which only run through the
 //    lists.
-// Every wait is bounded; one that gives up leaves NaN in the values that depend on it.
+// Every wait is bounded; one that gives up records QT_ETIMEOUT (site 60) in the status block
+// ahead of the layer table and leaves NaN in the values that depend on it.
 constexpr int kBackRows = 2;           // rows of a warp, at most
 constexpr int kTreeWarps = 4;          // consumer warps, and warps of a producer group
 constexpr int kTreeGroups = 3;
@@ -324,7 +325,7 @@ template <typename C>
 __global__ void __launch_bounds__(kTreeThreads) backward_tree_kernel(const C* __restrict__ counts, int n, int rows,
                                                                      const TreeLayer* __restrict__ layers,
                                                                      const double* __restrict__ phi, double* V,
-                                                                     double* X)
+                                                                     double* X, DevStatus* status, long long budget_us)
 {
     extern __shared__ uint32_t s_dyn[];                 // lists [group][rows][warp][slot][lane]
     __shared__ double s_val[kBackRows * kTreeWarps];
@@ -377,6 +378,8 @@ __global__ void __launch_bounds__(kTreeThreads) backward_tree_kernel(const C* __
 #pragma unroll
         for (int q = 0; q < kTreeMaxN / kHalf; ++q) v[q] = t + q * kHalf < Ln.N ? kUnset : 0ull;
         unsigned long long t0 = 0;
+        // a negative budget gives up without waiting, as every bounded wait does
+        bool give_up = s > 0 && !gave_up && budget_us < 0;
         for (int polls = 0;; ++polls) {
 #pragma unroll
             for (int q = 0; q < kTreeMaxN / kHalf; ++q) {
@@ -388,12 +391,17 @@ __global__ void __launch_bounds__(kTreeThreads) backward_tree_kernel(const C* __
             bool missing = false;
 #pragma unroll
             for (int q = 0; q < kTreeMaxN / kHalf; ++q) missing |= v[q] == kUnset;
-            if (!missing || s == 0 || gave_up) break;
+            if ((!missing && !give_up) || s == 0 || gave_up) break;
             if ((polls & 255) == 255) {
                 unsigned long long now;
                 asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
                 if (t0 == 0) t0 = now;
-                gave_up = now - t0 > 2000000000ull && polls > 100000;
+                give_up = give_up || now - t0 > (unsigned long long)budget_us * 1000ull;
+            }
+            if (give_up) {
+                gave_up = true;
+                if (atomicCAS(&status->code, 0, 4 /* QT_ETIMEOUT */) == 0) status->where = 60;
+                break;
             }
         }
         bool odd = false;
@@ -462,7 +470,8 @@ bool backward_tree_fits(int n, const int64_t* N, int num_sms)
 int backward_tree_blocks(int maxN, int num_sms) { return std::min((maxN + kTreeWarps - 1) / kTreeWarps, num_sms); }
 
 cudaError_t launch_backward_tree(const void* counts, int u32, int n, int maxN, const void* layers, const double* phi,
-                                 double* V, double* X, int num_sms, cudaStream_t st)
+                                 double* V, double* X, DevStatus* status, long long budget_us, int num_sms,
+                                 cudaStream_t st)
 {
     const int blocks = backward_tree_blocks(maxN, num_sms), rows = maxN > blocks * kTreeWarps ? 2 : 1;
     cudaError_t e = cudaMemsetAsync(X, 0xFF, (size_t)n * blocks * 8 * sizeof(double), st);
@@ -471,7 +480,8 @@ cudaError_t launch_backward_tree(const void* counts, int u32, int n, int maxN, c
     const size_t dyn = sizeof(uint32_t) * kRowBatch * kTreeWarps * kTreeGroups * rows;
     e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     if (e != cudaSuccess) return e;
-    void* args[] = {(void*)&counts, (void*)&n, (void*)&rows, (void*)&layers, (void*)&phi, (void*)&V, (void*)&X};
+    void* args[] = {(void*)&counts, (void*)&n, (void*)&rows, (void*)&layers, (void*)&phi, (void*)&V, (void*)&X,
+                    (void*)&status, (void*)&budget_us};
     return cudaLaunchCooperativeKernel(f, dim3((unsigned)blocks), dim3(kTreeThreads), args, dyn, st);
 }
 
