@@ -193,8 +193,11 @@ qt_status host_get(qt_ctx* ctx, const char* name, size_t bytes, void** out)
     HostBuf& b = ctx->host[name];
     if (b.bytes < bytes) {
         if (b.p) {
-            // an upload may still read it
-            if (ctx->ev_tables) cudaEventSynchronize(ctx->ev_tables);
+            // an upload may still read it: a forward step's (ev_tables comes after all of
+            // its uploads) or a backward induction's
+            cudaEventSynchronize(ctx->ev_tables);
+            cudaEventSynchronize(ctx->ev_up_tree[0]);
+            cudaEventSynchronize(ctx->ev_up_tree[1]);
             cudaFreeHost(b.p);
         }
         b.p = nullptr;

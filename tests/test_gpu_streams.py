@@ -91,3 +91,33 @@ def test_trees_on_two_streams(ctx, B, d):
         torch.cuda.synchronize()
         for k, (_, _, counts, want) in enumerate(cases):
             np.testing.assert_array_equal(counts.cpu().numpy(), want, err_msg=f"case {k}, round {rep}")
+
+
+def test_backward_on_two_streams(ctx, B):
+    """One-launch inductions of growing depth alternate between two streams while a long
+    kernel holds the first: their layer tables are uploaded from pinned blocks that grow."""
+    rng = np.random.default_rng(1)
+    cases = []
+    for n in (3, 8, 20, 60, 150, 400):
+        N = np.array([1] + [40] * n, dtype=np.int64)
+        counts = rng.integers(0, 50, int(np.sum(N[:-1] * N[1:])))
+        phi = rng.random(int(N.sum()))
+        off, want = np.concatenate([[0], np.cumsum(N)]), phi.copy()
+        at = len(counts)
+        for k in range(n - 1, -1, -1):
+            c = counts[at - N[k] * N[k + 1]:at].reshape(N[k], N[k + 1]).astype(np.float64)
+            at -= N[k] * N[k + 1]
+            cont = c @ want[off[k + 1]:off[k + 2]] / c.sum(1)
+            want[off[k]:off[k + 1]] = np.maximum(phi[off[k]:off[k + 1]], cont)
+        cases.append((N, _dev(counts), _dev(phi), want))
+    s = [torch.cuda.Stream(), torch.cuda.Stream()]
+    busy = torch.empty(1 << 28, dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s[0]):
+        for _ in range(20):
+            busy.add_(1.0)
+    got = [ctx.backward(N, counts, phi, stream=s[k % 2]) for k, (N, counts, phi, _) in enumerate(cases)]
+    torch.cuda.synchronize()
+    for V, (_, _, _, want) in zip(got, cases):
+        # 40 terms a row in either order, non-negative: (40 + 3) 2^-53 a layer, no growth
+        np.testing.assert_allclose(V.cpu().numpy(), want, rtol=1e-13, atol=0)
