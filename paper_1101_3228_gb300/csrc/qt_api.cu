@@ -1463,7 +1463,7 @@ qt_status backward_impl(qt_ctx* ctx, int32_t n, const int64_t* N, const void* co
         const size_t xb = sizeof(double) * 8 * (size_t)n * backward_tree_blocks(maxN, ctx->num_sms);
         void *dt, *dx, *ht;
         qt_status s;
-        const std::string block = ctx->up_tree ? "tree1" : "tree0";
+        const std::string block = ctx->up_tree ? "tree1" : "tree0", err = ctx->err;
         // a capture on another stream of this thread does not mind the allocations
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
         QT_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
@@ -1491,7 +1491,9 @@ qt_status backward_impl(qt_ctx* ctx, int32_t n, const int64_t* N, const void* co
             }
             cudaGetLastError();
         }
-        // no memory for it, or a partition with fewer SMs than the device: layer by layer
+        // no memory for it, or a partition with fewer SMs than the device: layer by layer,
+        // and no message of an error that the caller does not see
+        ctx->err = err;
     }
     QT_CUDA(cudaMemcpyAsync(V + goff[n], phi + goff[n], sizeof(double) * N[n], cudaMemcpyDeviceToDevice, st));
     for (int k = n - 1; k >= 0; --k)

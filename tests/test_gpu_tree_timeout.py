@@ -58,3 +58,19 @@ def test_a_wait_that_runs_out_is_reported(B, monkeypatch, u32):
     monkeypatch.delenv("QT_FAULT")
     ctx.transitions(model, G, model.M, model.seed, opts)
     ctx.close()
+
+
+def test_without_workspace_layer_by_layer(B, monkeypatch):
+    """No memory for the one launch: the induction runs a launch per layer, succeeds, and
+    leaves no message of the allocation that failed."""
+    model, g, phi = _tree()
+    ref = oracle.transitions(model, g, model.M, model.seed, W.PREC_F32)
+    want = oracle.price(model.N, ref, phi)
+    counts = torch.from_numpy(np.concatenate([c.reshape(-1) for c in ref]).astype(np.int64)).cuda()
+    ctx = B.Context(0)
+    monkeypatch.setenv("QT_FAULT", "alloc")
+    V = ctx.backward(model.N, counts, torch.from_numpy(phi).cuda())
+    monkeypatch.delenv("QT_FAULT")
+    assert abs(float(V[0]) - want) <= 1e-12 * abs(want)
+    assert ctx.lib.qt_last_error(ctx.h) == b""
+    ctx.close()
