@@ -33,8 +33,14 @@ __device__ __forceinline__ float warp_max(float v)
 // its own bin.  Point j is dropped from a box with centre c and half-widths h when,
 // against the point i nearest to c (for a bin also against the second nearest),
 //   D_j(x) - D_i(x) = |g_j - c|^2 - |g_i - c|^2 - 2 (x - c).(g_j - g_i)
-// is positive on the whole box by more than `marg`, which covers the FP32
-// rounding of the points and of this test.
+// is positive on the whole box by more than the FP32 rounding of the points and of this
+// test, u = 2^-24: a point's coordinates are off by u R (R bounds |g|) and its differences
+// t from c by u |t|, so D is off by (DM + 4) u D + 2 u R sum |t| and, with sum |t| <=
+// sqrt(DM) (D / s + s) / 2 for any s > 0 (s = the widest half-width here),
+//   error <= u (DM + 4 + R sqrt(DM) / s) (D_j + D_i) + u R (2 sqrt(DM) s + 4 sum h)
+//            + 8 u slack.
+// Twice that is allowed for.  (A bound of 2^-18 S^2 for every bin, S the size of the box,
+// kept 16 points in every bin of a 1-d grid of 1000.)
 template <int DM>
 __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid_constant__ ForwardParams p)
 {
@@ -105,8 +111,19 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
     const float er = 0x1p-24f * 1.01f * S + G.err0, e = er + G.err;
     // the enlarged bins must cover the error of the centred sample and of its bin number
     const bool usable = 32.0f * (G.err + G.err0 + 0x1p-21f * S) <= hmin;
-    // (floors here and in c2: products of the smallest grids fall out of FP32's range)
-    const float marg = 0x1p-18f * S * S + 0x1p-120f;
+    // the test's error, as above: rel (D_j + D_i) + fix + slk slack.  (The floors here and in
+    // c2: products of the smallest grids fall out of FP32's range)
+    constexpr float u2 = 0x1p-23f, slk = 0x1p-20f, sqd = DM == 1 ? 1.0f : 1.41421357f;
+    float rel, fix;
+    auto margins = [&](const float (&hw)[DM]) {
+        float s = hw[0], sum = hw[0];
+        if constexpr (DM == 2) {
+            s = fmaxf(s, hw[1]);
+            sum += hw[1];
+        }
+        rel = u2 * ((float)(DM + 4) + R * sqd / s);
+        fix = u2 * R * (2.0f * sqd * s + 4.0f * sum) + 0x1p-120f;
+    };
     if (blockIdx.y == 0 && tid == 0) {
         const float sq = DM == 1 ? 1.0f : 1.41421357f;
         const float kappa = fmaxf(0x1p-22f, e / (2.0f * hmin));
@@ -141,6 +158,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
             c[1] = ((float)(py * kPatchY) + 1.5f - K[1]) * h[1];
             hw[1] = h[1] * 2.1f;
         }
+        margins(hw);
         float bD = __int_as_float(0x7F800000);
         int bi = 0x7FFFFFFF;
         for (int j = lane; j < N; j += 32) {
@@ -177,7 +195,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
                     D = __fmaf_rn(t, t, D);
                     slack = __fmaf_rn(fabsf(s_g[j * DM + l] - s_g[bi * DM + l]), hw[l], slack);
                 }
-                keep = !(D - bD - 2.0f * slack > marg);
+                keep = !(D - bD - 2.0f * slack > __fmaf_rn(rel, D + bD, __fmaf_rn(slk, slack, fix)));
             }
             const unsigned m = __ballot_sync(0xFFFFFFFFu, keep);
             if (keep) surv[ns + __popc(m & ((1u << lane) - 1u))] = (uint16_t)j;
@@ -191,6 +209,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
             c[1] = ((float)y - K[1]) * h[1];
             hw[1] = 0.5f * 1.125f * h[1];
         }
+        margins(hw);
         float D0 = __int_as_float(0x7F800000), D1 = D0;
         int i0 = surv[0], i1 = surv[0];
         for (int t = 0; t < ns; ++t) {
@@ -220,7 +239,8 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
                 sl0 = __fmaf_rn(fabsf(gj - s_g[i0 * DM + l]), hw[l], sl0);
                 sl1 = __fmaf_rn(fabsf(gj - s_g[i1 * DM + l]), hw[l], sl1);
             }
-            return !(D - D0 - 2.0f * sl0 > marg) && !(D - D1 - 2.0f * sl1 > marg);
+            return !(D - D0 - 2.0f * sl0 > __fmaf_rn(rel, D + D0, __fmaf_rn(slk, sl0, fix))) &&
+                   !(D - D1 - 2.0f * sl1 > __fmaf_rn(rel, D + D1, __fmaf_rn(slk, sl1, fix)));
         };
         uint64_t ent = 0;
         int cnt = 0;

@@ -231,3 +231,26 @@ def test_located_fp64_pairs_off_the_next_mean(ctx, B, d, spread):
     got = B.split_counts(model.N, counts.cpu().numpy())
     for k in range(n):
         np.testing.assert_array_equal(got[k], ref[k], err_msg=f"layer {k}")
+
+
+@pytest.mark.parametrize("d,N", [(1, 100), (1, 1000), (1, 1024), (2, 100), (2, 1000)])
+@pytest.mark.parametrize("scale,shift", [(1.0, 0.0), (1e-3, 1.0), (1e4, 3e5), (1e-18, 0.0)])
+@pytest.mark.parametrize("kind", ["normal", "cluster"])
+def test_located_cells_at_cell_boundaries(ctx, B, d, N, scale, shift, kind):
+    """What the tables leave out: samples on, and within 1e-15 to 1e-4 of, the boundary
+    between two cells, on grids fine against the tables' bins and on grids far from the origin."""
+    rng = np.random.default_rng(N + d)
+    gA, gB = rng.standard_normal((N, d)), rng.standard_normal((N, d))
+    if kind == "cluster":
+        gA[::2] *= 1e-3
+        gB[::3] = gB[0] + 1e-5 * gB[::3]
+    M = 6000
+    X, Y = W.boundary_samples(gA, M, seed=1), W.boundary_samples(gB, M, seed=2)
+    jit = 10.0 ** rng.uniform(-15, -4, (2, M, 1)) * rng.standard_normal((2, M, d))
+    X[M // 4:] += jit[0, M // 4:]
+    Y[M // 4:] += jit[1, M // 4:]
+    gA, gB, X, Y = (shift + scale * v for v in (gA, gB, X, Y))
+    counts, st, ii, jj = ctx.counts_from_samples(_dev(gA), _dev(gB), _dev(X), _dev(Y), B.options(), want_cells=True)
+    np.testing.assert_array_equal(ii.cpu().numpy(), oracle.nearest(gA, X))
+    np.testing.assert_array_equal(jj.cpu().numpy(), oracle.nearest(gB, Y))
+    assert st.device_status == 0 and st.rechecks > 1000
