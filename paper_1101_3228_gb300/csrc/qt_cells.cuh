@@ -16,9 +16,12 @@
 // satisfies |D~ - D| <= err(D) = sqrt(d) (kappa D + e^2 / kappa) + d e^2 +
 // (d + 6) 2^-24 D, e the sum of both coordinates' errors, for any kappa > 0
 // (2 sqrt(D) e <= kappa D + e^2 / kappa).  The best candidate is the exact argmin
-// when second - best > 2 err(second); otherwise the exact FP64 distances of the
-// bin's candidates decide.  A sample whose e is f <= 1 times the grid's bound takes
-// f kappa: 2 err(D) = f (c1 D + c2) + c3 D.
+// when second - best > 2 err(second).  A sample whose e is f <= 1 times the grid's bound
+// takes f kappa: 2 err(D) = f (c1 D + c2) + c3 D, kappa for distances of a bin.  What that
+// does not certify is tried with the square root itself, which holds on the scale of any
+// cell (grids whose points lie much closer together than their box tells): 2 err(D) =
+// f (ce sqrt(D) + ce^2 / 8) + c3 D.  Otherwise the exact FP64 distances of the bin's
+// candidates decide.
 //
 // Why bins: brute force spends 2 d flops on each of N_k + N_{k+1} candidates (1000
 // on the 2-factor workload), and only the few points around a sample can be its
@@ -47,15 +50,23 @@ __device__ __forceinline__ float cell_dist(const float* __restrict__ rec, int j,
     return __fmaf_rn(dy, dy, dx * dx);
 }
 
+// 2 err(D) with the square root, for a sample whose error is f times the grid's bound.
+__device__ __forceinline__ float cell_bound(const CellGrid& G, float f, float D)
+{
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(D));
+    return __fmaf_rn(f, __fmaf_rn(G.ce, r, 0.125f * G.ce * G.ce), __fmaf_rn(G.c3, D, 0x1p-120f));
+}
+
 // Lists longer than an entry: the pool's, or the whole grid (records in shared
 // memory).  The whole grid also serves samples outside the box, whose error grows
 // with their distance: e is scaled by (|a| + R) / S <= 1 + |a| / S there.
 // Returns the index, with the top bit set when the distances do not certify it.
 template <int DM>
-__device__ __noinline__ uint32_t cell_long_list(const float* __restrict__ rec, int N, const uint16_t* __restrict__ pool,
-                                                uint64_t e, float a0, float a1, float f, float c1, float c2, float c3,
-                                                float inv_span)
+__device__ __noinline__ uint32_t cell_long_list(const CellGrid& G, const float* __restrict__ rec,
+                                                const uint16_t* __restrict__ pool, uint64_t e, float a0, float a1, float f)
 {
+    const int N = G.N;
     const bool scan = (int)(e >> 60) == kCellScan;
     const uint16_t* lst = pool + (uint32_t)e;
     const int cnt = scan ? N : (int)((e >> 32) & 0xFFFFu);
@@ -72,10 +83,10 @@ __device__ __noinline__ uint32_t cell_long_list(const float* __restrict__ rec, i
         best = fminf(best, D);
     }
     if (scan) {
-        const float g = 1.0f + (fabsf(a0) + fabsf(a1)) * inv_span;
+        const float g = 1.0f + (fabsf(a0) + fabsf(a1)) * G.inv_span;
         f *= g * g;
     }
-    const bool need = !(second - best > __fmaf_rn(f, __fmaf_rn(c1, second, c2), c3 * second));
+    const bool need = !(second - best > cell_bound(G, f, second));
     return bi | (need ? 0x80000000u : 0u);
 }
 
@@ -111,8 +122,7 @@ __device__ __forceinline__ int cell_search(const CellGrid& G, const unsigned cha
     need = false;
     const float* rec = reinterpret_cast<const float*>(sm + (size_t)((uint32_t)G.nb0 * (uint32_t)G.nb1 * 8u));
     if (cnt > kCellInline) {
-        const uint32_t r = cell_long_list<DM>(rec, G.N, pool, e, a[0], DM == 2 ? a[DM - 1] : 0.0f, f, G.c1, G.c2, G.c3,
-                                              G.inv_span);
+        const uint32_t r = cell_long_list<DM>(G, rec, pool, e, a[0], DM == 2 ? a[DM - 1] : 0.0f, f);
         idx = (int)(r & 0x7FFFFFFFu);
         need = (r >> 31) != 0;
     } else if (cnt > 1) {
@@ -127,6 +137,7 @@ __device__ __forceinline__ int cell_search(const CellGrid& G, const unsigned cha
             best = fminf(best, D);
         }
         need = !(second - best > __fmaf_rn(f, __fmaf_rn(G.c1, second, G.c2), G.c3 * second));
+        if (need) need = !(second - best > cell_bound(G, f, second));
     }
     return idx;
 }

@@ -93,24 +93,39 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
     }
     // the box: the grid's own, a quarter of its width wider on every side (quantizers
     // reach about 3 standard deviations, so the box reaches 4.5); bin b of an axis is
-    // centred on (b - K) h, K an integer
+    // centred on (b - K) h, K an integer.  The enlarged bins must cover the error of the
+    // centred sample and of its bin number, so an axis along which the grid is narrow (a
+    // product grid with one point, two factors of very different size) or a grid far from
+    // its centre takes wider bins than its share of the box
     const float R = __fsqrt_rn(r2) * 1.0001f;
     const int nb[2] = {G.nb0, G.nb1};
-    float K[DM], h[DM], hmin = __int_as_float(0x7F800000), A2 = 0.0f;
+    const float inf = __int_as_float(0x7F800000);
+    float K[DM], h[DM], ext[DM], S = 0.0f;
 #pragma unroll
     for (int l = 0; l < DM; ++l) {
-        const float ext = fmaxf(mx[l] - mn[l], fmaxf(0x1p-16f * R, 1e-30f));
-        h[l] = 1.5f * ext / (float)nb[l];
-        // a grid far from its centre has no bins here: `usable` is false for it
-        K[l] = fminf(fmaxf(rintf((0.25f * ext - mn[l]) / h[l]), -4194304.0f), 4194304.0f);
-        const float far_ = fmaxf(fabsf(mn[l]), fabsf(mx[l])) + 0.25f * ext + 2.0f * h[l];
-        A2 = __fmaf_rn(far_, far_, A2);
-        hmin = fminf(hmin, h[l]);
+        ext[l] = fmaxf(mx[l] - mn[l], 1e-30f);
+        const float far_ = fmaxf(fabsf(mn[l]), fabsf(mx[l])) + ext[l];
+        S = __fmaf_rn(far_, far_, S);
     }
-    const float S = (__fsqrt_rn(A2) + R) * 1.0001f;
+    // (the wider bins make S larger by less than a quarter: 32 2^-21 8192 = 1/8 for d = 1)
+    const float need = 32.0f * 1.3f * (G.err + G.err0 + 0x1p-21f * (__fsqrt_rn(S) + R));
+    S = 0.0f;
+    float hgeo = 1.0f;
+#pragma unroll
+    for (int l = 0; l < DM; ++l) {
+        h[l] = fmaxf(1.5f * ext[l] / (float)nb[l], need);
+        // a grid without finite sizes has no bins here: `usable` is false for it
+        K[l] = fminf(fmaxf(rintf((0.25f * ext[l] - mn[l]) / h[l]), -4194304.0f), 4194304.0f);
+        const float far_ = fmaxf(fabsf(K[l]) + 1.0f, fabsf((float)nb[l] - K[l]) + 1.0f) * h[l];
+        S = __fmaf_rn(far_, far_, S);
+        hgeo *= h[l];
+    }
+    if (DM == 2) hgeo = __fsqrt_rn(hgeo);
+    S = (__fsqrt_rn(S) + R) * 1.0001f;
     const float er = 0x1p-24f * 1.01f * S + G.err0, e = er + G.err;
-    // the enlarged bins must cover the error of the centred sample and of its bin number
-    const bool usable = 32.0f * (G.err + G.err0 + 0x1p-21f * S) <= hmin;
+    bool usable = S < inf;
+#pragma unroll
+    for (int l = 0; l < DM; ++l) usable = usable && 32.0f * (G.err + G.err0 + 0x1p-21f * S) <= h[l];
     // the test's error, as above: rel (D_j + D_i) + fix + slk slack.  (The floors here and in
     // c2: products of the smallest grids fall out of FP32's range)
     constexpr float u2 = 0x1p-23f, slk = 0x1p-20f, sqd = DM == 1 ? 1.0f : 1.41421357f;
@@ -126,7 +141,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
     };
     if (blockIdx.y == 0 && tid == 0) {
         const float sq = DM == 1 ? 1.0f : 1.41421357f;
-        const float kappa = fmaxf(0x1p-22f, e / (2.0f * hmin));
+        const float kappa = fmaxf(0x1p-22f, e / (2.0f * hgeo));
 #pragma unroll
         for (int l = 0; l < DM; ++l) {
             G.inv_h[l] = 1.0f / h[l];
@@ -136,6 +151,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         G.inv_span = 1.0f / S;
         G.c2 = 2.02f * (sq * (e / kappa) * e + (float)DM * e * e) + 0x1p-120f * (e / er);
         G.c3 = 2.02f * (float)(DM + 6) * 0x1p-24f;
+        G.ce = 4.04f * sq * e;
         G.f0 = er / e;
     }
     const int pnx = DM == 1 ? nb[0] / 32 : nb[0] / kPatchX, pny = DM == 1 ? 1 : nb[1] / kPatchY;

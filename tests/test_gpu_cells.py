@@ -254,3 +254,28 @@ def test_located_cells_at_cell_boundaries(ctx, B, d, N, scale, shift, kind):
     np.testing.assert_array_equal(ii.cpu().numpy(), oracle.nearest(gA, X))
     np.testing.assert_array_equal(jj.cpu().numpy(), oracle.nearest(gB, Y))
     assert st.device_status == 0 and st.rechecks > 1000
+
+
+@pytest.mark.parametrize("kind", ["flat", "narrow", "off"])
+def test_located_search_certifies_odd_grids(ctx, B, kind):
+    """Grids with one point along an axis, with axes of very different extent, and far from the
+    centre of the search still have tables and certificates: few searches need FP64.  On
+    the flat grid, 500 points evenly over 8 and samples at most 4 beside it, the certificate
+    asks for 4 sqrt(2) e sqrt(D) <= 1.4e-5, e = 2^-24 of 10 (the box's size), where second
+    and best differ by up to the squared spacing, 2.6e-4: at most 6% are in doubt."""
+    rng = np.random.default_rng(6)
+    M, N, d = 20000, 500, 2
+    g, X = rng.standard_normal((2, N, d)), np.clip(rng.standard_normal((2, M, d)), -4, 4)
+    if kind == "flat":
+        g[:, :, 0], g[:, :, 1] = np.linspace(-4, 4, N), 0.0
+    elif kind == "narrow":
+        g[:, :, 1] *= 1e-3
+        X[:, :, 1] *= 1e-3
+    else:
+        d = 1
+        g, X = 4.6 + 0.1 * g[:, :, :1], 4.6 + 0.1 * X[:, :, :1]
+    counts, st, ii, jj = ctx.counts_from_samples(_dev(g[0]), _dev(g[1]), _dev(X[0]), _dev(X[1]), B.options(),
+                                                 want_cells=True)
+    np.testing.assert_array_equal(ii.cpu().numpy(), oracle.nearest(g[0], X[0]))
+    np.testing.assert_array_equal(jj.cpu().numpy(), oracle.nearest(g[1], X[1]))
+    assert st.rechecks < 0.15 * 2 * M
