@@ -58,36 +58,94 @@ __device__ __forceinline__ float cell_bound(const CellGrid& G, float f, float D)
     return __fmaf_rn(f, __fmaf_rn(G.ce, r, 0.125f * G.ce * G.ce), __fmaf_rn(G.c3, D, 0x1p-120f));
 }
 
+// One step of a running minimum: smallest, second smallest, index of the smallest.
+__device__ __forceinline__ void cell_take(float D, int j, float& best, float& second, int& bi)
+{
+    second = fminf(second, fmaxf(D, best));
+    bi = D < best ? j : bi;
+    best = fminf(best, D);
+}
+
+// Smallest and second smallest distance over the whole grid, eight points at a time: every
+// lane reads the same ones (16-byte broadcasts), and only the minimum of the eight is
+// tracked; which point it was, and the second within its eight, come from that group at the
+// end.  About 4.6 instructions a point for d = 2, as many as the brute-force screen takes: a
+// grid that no table serves costs no more than without one.
+template <int DM>
+__device__ __forceinline__ void cell_scan(const float* __restrict__ rec, int N, const float (&a)[DM], float& best,
+                                          float& second, int& bi)
+{
+    const float inf = __int_as_float(0x7F800000);
+    float b1 = inf, b2 = inf;
+    int g1 = 0;
+    const int N8 = N & ~7;
+    for (int j = 0; j < N8; j += 8) {
+        float m = inf;
+#pragma unroll
+        for (int v = 0; v < 8 * DM; v += 4) {
+            const float4 r = *reinterpret_cast<const float4*>(rec + j * DM + v);
+            if constexpr (DM == 1) {
+                const float x = a[0] - r.x, y = a[0] - r.y, z = a[0] - r.z, w = a[0] - r.w;
+                m = fminf(fminf(m, fminf(x * x, y * y)), fminf(z * z, w * w));
+            } else {
+                const float x = a[0] - r.x, y = a[1] - r.y, z = a[0] - r.z, w = a[1] - r.w;
+                m = fminf(m, fminf(__fmaf_rn(y, y, x * x), __fmaf_rn(w, w, z * z)));
+            }
+        }
+        b2 = fminf(b2, fmaxf(m, b1));
+        g1 = m < b1 ? j : g1;
+        b1 = fminf(b1, m);
+    }
+    // the best group's points in order, then the last N mod 8
+    best = inf;
+    second = inf;
+    bi = 0;
+    if (N8 > 0)
+        for (int q = 0; q < 8; ++q) cell_take(cell_dist(rec, g1 + q, a), g1 + q, best, second, bi);
+    second = fminf(second, b2);
+    for (int j = N8; j < N; ++j) cell_take(cell_dist(rec, j, a), j, best, second, bi);
+}
+
 // Lists longer than an entry: the pool's, or the whole grid (records in shared
 // memory).  The whole grid also serves samples outside the box, whose error grows
-// with their distance: e is scaled by (|a| + R) / S <= 1 + |a| / S there.
+// with their distance: e is scaled by (|a| + R) / S <= 1 + |a| / S there (cell_error).
 // Returns the index, with the top bit set when the distances do not certify it.
+template <int DM>
+__device__ __forceinline__ float cell_error(const CellGrid& G, const float (&a)[DM], float f)
+{
+    float g = 1.0f + fabsf(a[0]) * G.inv_span;
+    if constexpr (DM == 2) g += fabsf(a[1]) * G.inv_span;
+    return f * g * g;
+}
+
 template <int DM>
 __device__ __noinline__ uint32_t cell_long_list(const CellGrid& G, const float* __restrict__ rec,
                                                 const uint16_t* __restrict__ pool, uint64_t e, float a0, float a1, float f)
 {
-    const int N = G.N;
-    const bool scan = (int)(e >> 60) == kCellScan;
-    const uint16_t* lst = pool + (uint32_t)e;
-    const int cnt = scan ? N : (int)((e >> 32) & 0xFFFFu);
     float a[DM];
     a[0] = a0;
     if constexpr (DM == 2) a[1] = a1;
     float best = __int_as_float(0x7F800000), second = best;
-    uint32_t bi = 0;
-    for (int q = 0; q < cnt; ++q) {
-        const int j = scan ? q : (int)lst[q];
-        const float D = cell_dist(rec, j, a);
-        second = fminf(second, fmaxf(D, best));
-        bi = D < best ? (uint32_t)j : bi;
-        best = fminf(best, D);
-    }
-    if (scan) {
-        const float g = 1.0f + (fabsf(a0) + fabsf(a1)) * G.inv_span;
-        f *= g * g;
+    int bi = 0;
+    if ((int)(e >> 60) == kCellScan) {
+        cell_scan<DM>(rec, G.N, a, best, second, bi);
+        f = cell_error<DM>(G, a, f);
+    } else {
+        const uint16_t* lst = pool + (uint32_t)e;
+        const int cnt = (int)((e >> 32) & 0xFFFFu);
+        for (int q = 0; q < cnt; ++q) {
+            const int j = (int)lst[q];
+            cell_take(cell_dist(rec, j, a), j, best, second, bi);
+        }
     }
     const bool need = !(second - best > cell_bound(G, f, second));
-    return bi | (need ? 0x80000000u : 0u);
+    return (uint32_t)bi | (need ? 0x80000000u : 0u);
+}
+
+// A grid's records, after its table.
+__device__ __forceinline__ const float* cell_records(const CellGrid& G, const unsigned char* sm)
+{
+    return reinterpret_cast<const float*>(sm + (size_t)((uint32_t)G.nb0 * (uint32_t)G.nb1 * 8u));
 }
 
 // Number of the bin of coordinate a along one axis: the FMA rounds a / h + origin to
@@ -120,7 +178,7 @@ __device__ __forceinline__ int cell_search(const CellGrid& G, const unsigned cha
     const int cnt = (int)(e >> 60);
     int idx = (int)(e & 1023u);
     need = false;
-    const float* rec = reinterpret_cast<const float*>(sm + (size_t)((uint32_t)G.nb0 * (uint32_t)G.nb1 * 8u));
+    const float* rec = cell_records(G, sm);
     if (cnt > kCellInline) {
         const uint32_t r = cell_long_list<DM>(G, rec, pool, e, a[0], DM == 2 ? a[DM - 1] : 0.0f, f);
         idx = (int)(r & 0x7FFFFFFFu);
@@ -142,21 +200,38 @@ __device__ __forceinline__ int cell_search(const CellGrid& G, const unsigned cha
     return idx;
 }
 
-// Exact FP64 argmin over a bin's candidates (lowest index among equal distances).  A
-// sample without a finite distance has no cell: the index is out of range, and the callers
-// refuse it, as in the other forms.
+// Exact FP64 argmin over a bin's candidates (lowest index among equal distances), for a
+// search that the FP32 distances did not certify: only those that they leave in doubt,
+// D~_j - D~_best <= 2 err(D~_j), are evaluated in FP64 (two of them nearly always; an FP64
+// operation holds a warp's quarter of the SM for 65 cycles, and all 500 of a grid without a
+// table took 50 us of an SM a warp).  A sample without a finite distance has no cell: the
+// index is out of range, and the callers refuse it, as in the other forms.
 template <int DM>
-__device__ __noinline__ int cell_exact(const double (&z)[DM], uint64_t e, const uint16_t* __restrict__ pool,
-                                       const double* __restrict__ g64, int N, int d)
+__device__ __noinline__ int cell_exact(const CellGrid& G, const float* __restrict__ rec, const float (&a)[DM], float f,
+                                       const double (&z)[DM], uint64_t e, const uint16_t* __restrict__ pool,
+                                       const double* __restrict__ g64)
 {
     const int kind = (int)(e >> 60);
-    const int cnt = kind == kCellScan ? N : (kind == kCellPool ? (int)((e >> 32) & 0xFFFFu) : kind);
+    const int cnt = kind == kCellScan ? G.N : (kind == kCellPool ? (int)((e >> 32) & 0xFFFFu) : kind);
+    auto at = [&](int q) {
+        return kind == kCellScan ? q : (kind == kCellPool ? (int)pool[(uint32_t)e + q] : (int)((e >> (10 * q)) & 1023u));
+    };
+    float b = __int_as_float(0x7F800000), second;
+    if (kind == kCellScan) {
+        int i;
+        cell_scan<DM>(rec, G.N, a, b, second, i);
+        f = cell_error<DM>(G, a, f);
+    } else {
+        for (int q = 0; q < cnt; ++q) b = fminf(b, cell_dist(rec, at(q), a));
+    }
     double best = __longlong_as_double(0x7FF0000000000000LL);
     int bi = 0x7FFFFFFF;
+#pragma unroll 4
     for (int q = 0; q < cnt; ++q) {
-        const int j = kind == kCellScan ? q
-                                        : (kind == kCellPool ? (int)pool[(uint32_t)e + q] : (int)((e >> (10 * q)) & 1023u));
-        const double dj = dist64<DM>(z, g64 + (long long)j * d, d);
+        const int j = at(q);
+        const float D = cell_dist(rec, j, a);
+        if (D - b > cell_bound(G, f, D)) continue;
+        const double dj = dist64<DM>(z, g64 + (long long)j * DM, DM);
         if (dj < best) {
             best = dj;
             bi = j;

@@ -268,6 +268,8 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         }
         if (cnt <= kCellInline) {
             ent |= (uint64_t)cnt << 60;
+        } else if (4 * cnt > N) {
+            ent = kCellScanEntry;          // a scan of the whole grid is as fast (12 against 4.6 instructions a point)
         } else {
             const unsigned long long off = atomicAdd(p.cell_cursor, (unsigned long long)cnt);
             if (pool_holds(off, (uint32_t)cnt, p.cell_pool_cap)) {
@@ -289,12 +291,13 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
 // Exact FP64 cell of sample m (X or Y) among the candidates of its bin.
 template <int DM>
 static __device__ __noinline__ int cell_recheck(const ForwardParams& p, const float* spf, const double* spd, int k,
-                                                unsigned long long m, bool wantY, uint64_t e, const CellGrid& G)
+                                                unsigned long long m, bool wantY, uint64_t e, const CellGrid& G,
+                                                const unsigned char* sm, const float (&a)[DM], float f)
 {
     double z[DM];
     exact_sample<DM>(p, spf, spd, k, m, wantY, z);
     atomicAdd(&p.status->rechecks, 1ull);
-    return cell_exact<DM>(z, e, p.cell_pool, p.g64 + G.goff * DM, G.N, DM);
+    return cell_exact<DM>(G, cell_records(G, sm), a, f, z, e, p.cell_pool, p.g64 + G.goff * DM);
 }
 
 // The forward step.  MODE 0: FP32 samples, 1: FP64 samples (drawn in FP32 first,
@@ -406,14 +409,11 @@ __global__ void __launch_bounds__(kCellThreads, 1) forward_cells_kernel(const __
         int i = 0, j = 0;
         uint64_t eA, eB;
         bool needA = false, needB = false;
-        if (s_L.NA > 1)
-            i = cell_search<DM>(s_GA, dsm_c, p.cell_pool, a, MODE == 1 ? __fmaf_rn(f, 1.0f - s_GA.f0, s_GA.f0) : 1.0f, eA,
-                                needA);
-        if (s_L.NB > 1)
-            j = cell_search<DM>(s_GB, smB, p.cell_pool, b, MODE == 1 ? __fmaf_rn(f, 1.0f - s_GB.f0, s_GB.f0) : 1.0f, eB,
-                                needB);
-        if (needA) i = cell_recheck<DM>(p, s_pf, s_pd, k, m, false, eA, s_GA);
-        if (needB) j = cell_recheck<DM>(p, s_pf, s_pd, k, m, true, eB, s_GB);
+        auto share = [&](const CellGrid& G) { return MODE == 1 ? __fmaf_rn(f, 1.0f - G.f0, G.f0) : 1.0f; };
+        if (s_L.NA > 1) i = cell_search<DM>(s_GA, dsm_c, p.cell_pool, a, share(s_GA), eA, needA);
+        if (s_L.NB > 1) j = cell_search<DM>(s_GB, smB, p.cell_pool, b, share(s_GB), eB, needB);
+        if (needA) i = cell_recheck<DM>(p, s_pf, s_pd, k, m, false, eA, s_GA, dsm_c, a, share(s_GA));
+        if (needB) j = cell_recheck<DM>(p, s_pf, s_pd, k, m, true, eB, s_GB, smB, b, share(s_GB));
         // ---- counters p^k_ij (Sec. 3.3), per-sample cells, dumps
         if ((unsigned)i >= (unsigned)s_L.NA || (unsigned)j >= (unsigned)s_L.NB) {
             record_error(p.status, 6 /* QT_EDEVICE */, 52);
