@@ -17,11 +17,20 @@
 // (d + 6) 2^-24 D, e the sum of both coordinates' errors, for any kappa > 0
 // (2 sqrt(D) e <= kappa D + e^2 / kappa).  The best candidate is the exact argmin
 // when second - best > 2 err(second).  A sample whose e is f <= 1 times the grid's bound
-// takes f kappa: 2 err(D) = f (c1 D + c2) + c3 D, kappa for distances of a bin.  What that
-// does not certify is tried with the square root itself, which holds on the scale of any
-// cell (grids whose points lie much closer together than their box tells): 2 err(D) =
-// f (ce sqrt(D) + ce^2 / 8) + c3 D.  Otherwise the exact FP64 distances of the bin's
-// candidates decide.
+// takes f kappa: 2 err(D) = f (c1 D + c2) + c3 D, kappa for distances of a bin and e for
+// the whole box.  What that does not certify is tried with the square root itself and
+// with the rounding of this sample and of points at this distance, u (2 |a| + sqrt(D)) in
+// the place of the box's (cell_doubt): that holds on the scale of any cell, for grids whose
+// points lie much closer together than their box tells, and outside the box.  Otherwise
+// the exact FP64 distances of the bin's candidates decide.
+//
+// Outside the box the whole grid is searched, but for d = 1 the last bin of either side
+// serves up to 2^20 bins beyond: D_j - D_i = (g_i - g_j)(2 x - g_i - g_j) only grows there.
+// (Further out distances tie in FP64: a point is dropped for being 5 u r nearer at least, r
+// > 2 bins the distance to it, so ties begin at 2^51 5 u r / 2.)  There |a| <= R + sqrt(D),
+// and the excess of 4 sqrt(D) u (2 R + 3 sqrt(D)) over the box's bound is the 12 u D that c3
+// has more.  An axis along which all points are equal has one bin of 2^14 of the other's:
+// what it adds to the distances is the same number for all points.
 //
 // Why bins: brute force spends 2 d flops on each of N_k + N_{k+1} candidates (1000
 // on the 2-factor workload), and only the few points around a sample can be its
@@ -50,12 +59,32 @@ __device__ __forceinline__ float cell_dist(const float* __restrict__ rec, int j,
     return __fmaf_rn(dy, dy, dx * dx);
 }
 
-// 2 err(D) with the square root, for a sample whose error is f times the grid's bound.
-__device__ __forceinline__ float cell_bound(const CellGrid& G, float f, float D)
+// A sample's 2 err(D) with the square root: linear in r = sqrt(D) beside r^2.
+struct CellDoubt {
+    float c, s, q;                     // 2 err(D) = c + s r + q D
+    __device__ __forceinline__ float operator()(float D) const
+    {
+        float r;
+        asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(D));
+        return __fmaf_rn(q, D, __fmaf_rn(s, r, c));
+    }
+    // D~_best + this much and more is beyond doubt: K >= 2 err(b + K) for K = max(4 s^2,
+    // 2.1 (c + s sqrt(b) + q b)), because s sqrt(b + K) <= s sqrt(b) + s sqrt(K) and
+    // s sqrt(K) <= K / 2 (q K, q < 2^-17, is in the 2.1)
+    __device__ __forceinline__ float window(float b) const { return fmaxf(4.04f * s * s, 2.12f * (*this)(b)); }
+};
+
+// f: the share of the grid's bound that the search takes.  e = the part beyond FP32
+// rounding (f's e less the box's rounding) + u (2 |a| + r), 1.01 for this arithmetic.
+template <int DM>
+__device__ __forceinline__ CellDoubt cell_doubt(const CellGrid& G, const float (&a)[DM], float f)
 {
-    float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(D));
-    return __fmaf_rn(f, __fmaf_rn(G.ce, r, 0.125f * G.ce * G.ce), __fmaf_rn(G.c3, D, 0x1p-120f));
+    constexpr float sq = DM == 1 ? 1.0f : 1.41421357f, u = 0x1p-24f;
+    float m = fabsf(a[0]);
+    if constexpr (DM == 2) m += fabsf(a[1]);
+    const float e0 = 1.01f * (fmaxf(__fmaf_rn(f, G.e, -G.ebox), 0.0f) + 0x1p-22f * G.e + 2.0f * u * m);
+    // 4 sq (e0 + u r) r + 2 DM (e0 + u r)^2 + 2 (DM + 6) u D
+    return CellDoubt{__fmaf_rn(2.05f * DM * e0, e0, 0x1p-120f), 4.1f * sq * e0, (4.1f * sq + 2.05f * (DM + 6)) * u};
 }
 
 // One step of a running minimum: smallest, second smallest, index of the smallest.
@@ -66,11 +95,30 @@ __device__ __forceinline__ void cell_take(float D, int j, float& best, float& se
     best = fminf(best, D);
 }
 
-// Smallest and second smallest distance over the whole grid, eight points at a time: every
-// lane reads the same ones (16-byte broadcasts), and only the minimum of the eight is
-// tracked; which point it was, and the second within its eight, come from that group at the
-// end.  About 4.6 instructions a point for d = 2, as many as the brute-force screen takes: a
-// grid that no table serves costs no more than without one.
+// Smallest distance to eight consecutive points (every lane reads the same ones: 16-byte
+// broadcasts).
+template <int DM>
+__device__ __forceinline__ float cell_min8(const float* __restrict__ rec, const float (&a)[DM])
+{
+    float m = __int_as_float(0x7F800000);
+#pragma unroll
+    for (int v = 0; v < 8 * DM; v += 4) {
+        const float4 r = *reinterpret_cast<const float4*>(rec + v);
+        if constexpr (DM == 1) {
+            const float x = a[0] - r.x, y = a[0] - r.y, z = a[0] - r.z, w = a[0] - r.w;
+            m = fminf(fminf(m, fminf(x * x, y * y)), fminf(z * z, w * w));
+        } else {
+            const float x = a[0] - r.x, y = a[1] - r.y, z = a[0] - r.z, w = a[1] - r.w;
+            m = fminf(m, fminf(__fmaf_rn(y, y, x * x), __fmaf_rn(w, w, z * z)));
+        }
+    }
+    return m;
+}
+
+// Smallest and second smallest distance over the whole grid, eight points at a time: only
+// the minimum of the eight is tracked; which point it was, and the second within its eight,
+// come from that group at the end.  About 4.6 instructions a point for d = 2, as many as the
+// brute-force screen takes: a grid that no table serves costs no more than without one.
 template <int DM>
 __device__ __forceinline__ void cell_scan(const float* __restrict__ rec, int N, const float (&a)[DM], float& best,
                                           float& second, int& bi)
@@ -80,18 +128,7 @@ __device__ __forceinline__ void cell_scan(const float* __restrict__ rec, int N, 
     int g1 = 0;
     const int N8 = N & ~7;
     for (int j = 0; j < N8; j += 8) {
-        float m = inf;
-#pragma unroll
-        for (int v = 0; v < 8 * DM; v += 4) {
-            const float4 r = *reinterpret_cast<const float4*>(rec + j * DM + v);
-            if constexpr (DM == 1) {
-                const float x = a[0] - r.x, y = a[0] - r.y, z = a[0] - r.z, w = a[0] - r.w;
-                m = fminf(fminf(m, fminf(x * x, y * y)), fminf(z * z, w * w));
-            } else {
-                const float x = a[0] - r.x, y = a[1] - r.y, z = a[0] - r.z, w = a[1] - r.w;
-                m = fminf(m, fminf(__fmaf_rn(y, y, x * x), __fmaf_rn(w, w, z * z)));
-            }
-        }
+        const float m = cell_min8<DM>(rec + j * DM, a);
         b2 = fminf(b2, fmaxf(m, b1));
         g1 = m < b1 ? j : g1;
         b1 = fminf(b1, m);
@@ -107,19 +144,10 @@ __device__ __forceinline__ void cell_scan(const float* __restrict__ rec, int N, 
 }
 
 // Lists longer than an entry: the pool's, or the whole grid (records in shared
-// memory).  The whole grid also serves samples outside the box, whose error grows
-// with their distance: e is scaled by (|a| + R) / S <= 1 + |a| / S there (cell_error).
-// Returns the index, with the top bit set when the distances do not certify it.
+// memory), which also serves samples outside the box.  Returns the index, with the top
+// bit set when the distances do not certify it, and above it the smallest distance.
 template <int DM>
-__device__ __forceinline__ float cell_error(const CellGrid& G, const float (&a)[DM], float f)
-{
-    float g = 1.0f + fabsf(a[0]) * G.inv_span;
-    if constexpr (DM == 2) g += fabsf(a[1]) * G.inv_span;
-    return f * g * g;
-}
-
-template <int DM>
-__device__ __noinline__ uint32_t cell_long_list(const CellGrid& G, const float* __restrict__ rec,
+__device__ __noinline__ uint64_t cell_long_list(const CellGrid& G, const float* __restrict__ rec,
                                                 const uint16_t* __restrict__ pool, uint64_t e, float a0, float a1, float f)
 {
     float a[DM];
@@ -129,17 +157,17 @@ __device__ __noinline__ uint32_t cell_long_list(const CellGrid& G, const float* 
     int bi = 0;
     if ((int)(e >> 60) == kCellScan) {
         cell_scan<DM>(rec, G.N, a, best, second, bi);
-        f = cell_error<DM>(G, a, f);
     } else {
         const uint16_t* lst = pool + (uint32_t)e;
         const int cnt = (int)((e >> 32) & 0xFFFFu);
+#pragma unroll 4
         for (int q = 0; q < cnt; ++q) {
             const int j = (int)lst[q];
             cell_take(cell_dist(rec, j, a), j, best, second, bi);
         }
     }
-    const bool need = !(second - best > cell_bound(G, f, second));
-    return (uint32_t)bi | (need ? 0x80000000u : 0u);
+    const bool need = !(second - best > cell_doubt<DM>(G, a, f)(second));
+    return (uint32_t)bi | (need ? 0x80000000u : 0u) | ((uint64_t)__float_as_uint(best) << 32);
 }
 
 // A grid's records, after its table.
@@ -167,7 +195,12 @@ __device__ __forceinline__ int cell_search(const CellGrid& G, const unsigned cha
     const float4 axes = *reinterpret_cast<const float4*>(G.inv_h);
     uint32_t b = cell_bin(a[0], axes.x, axes.z);
     bool in = b < (uint32_t)G.nb0;
-    if constexpr (DM == 2) {
+    if constexpr (DM == 1) {
+        // the last bins serve what lies up to 2^20 bins beyond them
+        const float v = __fmaf_rn(a[0], axes.x, axes.z);
+        b = (uint32_t)__float_as_int(fminf(fmaxf(v, 8388608.0f), 8388607.0f + (float)G.nb0)) - 0x4B000000u;
+        in = fabsf(v - 8388608.0f) <= 1048576.0f;
+    } else {
         const uint32_t b1 = cell_bin(a[1], axes.y, axes.w);
         in = in && b1 < (uint32_t)G.nb1;
         b += b1 * (uint32_t)G.nb0;
@@ -180,9 +213,10 @@ __device__ __forceinline__ int cell_search(const CellGrid& G, const unsigned cha
     need = false;
     const float* rec = cell_records(G, sm);
     if (cnt > kCellInline) {
-        const uint32_t r = cell_long_list<DM>(G, rec, pool, e, a[0], DM == 2 ? a[DM - 1] : 0.0f, f);
-        idx = (int)(r & 0x7FFFFFFFu);
-        need = (r >> 31) != 0;
+        const uint64_t r = cell_long_list<DM>(G, rec, pool, e, a[0], DM == 2 ? a[DM - 1] : 0.0f, f);
+        idx = (int)((uint32_t)r & 0x7FFFFFFFu);
+        need = ((uint32_t)r >> 31) != 0;
+        if (cnt == kCellScan) entry = kCellScanEntry | (r >> 32);
     } else if (cnt > 1) {
         float best = cell_dist(rec, idx, a), second = __int_as_float(0x7F800000);
         uint64_t r = e;
@@ -195,17 +229,18 @@ __device__ __forceinline__ int cell_search(const CellGrid& G, const unsigned cha
             best = fminf(best, D);
         }
         need = !(second - best > __fmaf_rn(f, __fmaf_rn(G.c1, second, G.c2), G.c3 * second));
-        if (need) need = !(second - best > cell_bound(G, f, second));
+        if (need) need = !(second - best > cell_doubt<DM>(G, a, f)(second));
     }
     return idx;
 }
 
 // Exact FP64 argmin over a bin's candidates (lowest index among equal distances), for a
 // search that the FP32 distances did not certify: only those that they leave in doubt,
-// D~_j - D~_best <= 2 err(D~_j), are evaluated in FP64 (two of them nearly always; an FP64
-// operation holds a warp's quarter of the SM for 65 cycles, and all 500 of a grid without a
-// table took 50 us of an SM a warp).  A sample without a finite distance has no cell: the
-// index is out of range, and the callers refuse it, as in the other forms.
+// D~_j <= D~_best + window, are evaluated in FP64 (two of them nearly always; an FP64
+// operation holds a warp's quarter of the SM for 65 cycles whether one lane takes part or
+// all, so the points in doubt are put into an entry first and evaluated side by side).  A
+// sample without a finite distance has no cell: the index is out of range, and the callers
+// refuse it, as in the other forms.
 template <int DM>
 __device__ __noinline__ int cell_exact(const CellGrid& G, const float* __restrict__ rec, const float (&a)[DM], float f,
                                        const double (&z)[DM], uint64_t e, const uint16_t* __restrict__ pool,
@@ -216,21 +251,36 @@ __device__ __noinline__ int cell_exact(const CellGrid& G, const float* __restric
     auto at = [&](int q) {
         return kind == kCellScan ? q : (kind == kCellPool ? (int)pool[(uint32_t)e + q] : (int)((e >> (10 * q)) & 1023u));
     };
-    float b = __int_as_float(0x7F800000), second;
+    float b = __int_as_float(0x7F800000);
     if (kind == kCellScan) {
-        int i;
-        cell_scan<DM>(rec, G.N, a, b, second, i);
-        f = cell_error<DM>(G, a, f);
+        b = __uint_as_float((uint32_t)e);
     } else {
+#pragma unroll 4
         for (int q = 0; q < cnt; ++q) b = fminf(b, cell_dist(rec, at(q), a));
+    }
+    const float lim = b + cell_doubt<DM>(G, a, f).window(b);
+    uint64_t in_doubt = 0;
+    int n = 0;
+    auto look = [&](int j) {
+        if (cell_dist(rec, j, a) > lim) return;
+        if (n < kCellInline) in_doubt |= (uint64_t)j << (10 * n);
+        ++n;
+    };
+    if (kind == kCellScan) {
+        const int N8 = G.N & ~7;
+        for (int j = 0; j < N8; j += 8)
+            if (!(cell_min8<DM>(rec + j * DM, a) > lim))
+                for (int q = 0; q < 8; ++q) look(j + q);
+        for (int j = N8; j < G.N; ++j) look(j);
+    } else {
+        for (int q = 0; q < cnt; ++q) look(at(q));
     }
     double best = __longlong_as_double(0x7FF0000000000000LL);
     int bi = 0x7FFFFFFF;
-#pragma unroll 4
-    for (int q = 0; q < cnt; ++q) {
-        const int j = at(q);
-        const float D = cell_dist(rec, j, a);
-        if (D - b > cell_bound(G, f, D)) continue;
+    const bool all = n > kCellInline;
+    for (int q = 0; q < (all ? cnt : n); ++q) {
+        const int j = all ? at(q) : (int)((in_doubt >> (10 * q)) & 1023u);
+        if (all && cell_dist(rec, j, a) > lim) continue;
         const double dj = dist64<DM>(z, g64 + (long long)j * DM, DM);
         if (dj < best) {
             best = dj;

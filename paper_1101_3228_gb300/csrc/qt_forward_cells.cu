@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
     __shared__ float s_g[kCellMaxN * DM];
     __shared__ uint16_t s_surv[kBuildWarps][kCellMaxN];
     __shared__ float s_red[kBuildWarps][2 * DM + 1];
+    __shared__ int s_some[kBuildWarps];
     CellGrid& G = p.cells[p.cell_g0 + blockIdx.x];
     const int N = G.N;
     if (N <= 1) return;
@@ -58,11 +59,16 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         mn[l] = __int_as_float(0x7F800000);
         mx[l] = -__int_as_float(0x7F800000);
     }
+    bool flat[DM];
+#pragma unroll
+    for (int l = 0; l < DM; ++l) flat[l] = DM == 2;
     for (int j = tid; j < N; j += kBuildThreads) {
         float n2 = 0.0f;
 #pragma unroll
         for (int l = 0; l < DM; ++l) {
-            const float v = __double2float_rn(__dsub_rn(g64[(long long)j * DM + l], (double)G.mu[l]));
+            const double c = g64[(long long)j * DM + l];
+            const float v = __double2float_rn(__dsub_rn(c, (double)G.mu[l]));
+            flat[l] = flat[l] && c == g64[l];
             s_g[j * DM + l] = v;
             mn[l] = fminf(mn[l], v);
             mx[l] = fmaxf(mx[l], v);
@@ -82,7 +88,15 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
     }
     r2 = warp_max(r2);
     if (lane == 0) s_red[warp][2 * DM] = r2;
+    int some = 0;                                      // bit l: axis l is not flat
+#pragma unroll
+    for (int l = 0; l < DM; ++l) some |= flat[l] ? 0 : 1 << l;
+    some = (int)__reduce_or_sync(0xFFFFFFFFu, (unsigned)some);
+    if (lane == 0) s_some[warp] = some;
     __syncthreads();
+    for (int w = 0; w < kBuildWarps; ++w) some |= s_some[w];
+#pragma unroll
+    for (int l = 0; l < DM; ++l) flat[l] = (some & (1 << l)) == 0;
     for (int w = 0; w < kBuildWarps; ++w) {
 #pragma unroll
         for (int l = 0; l < DM; ++l) {
@@ -112,20 +126,42 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
     S = 0.0f;
     float hgeo = 1.0f;
 #pragma unroll
-    for (int l = 0; l < DM; ++l) {
-        h[l] = fmaxf(1.5f * ext[l] / (float)nb[l], need);
-        // a grid without finite sizes has no bins here: `usable` is false for it
-        K[l] = fminf(fmaxf(rintf((0.25f * ext[l] - mn[l]) / h[l]), -4194304.0f), 4194304.0f);
-        const float far_ = fmaxf(fabsf(K[l]) + 1.0f, fabsf((float)nb[l] - K[l]) + 1.0f) * h[l];
-        S = __fmaf_rn(far_, far_, S);
-        hgeo *= h[l];
+    for (int l = 0; l < DM; ++l) h[l] = fmaxf(1.5f * ext[l] / (float)nb[l], need);
+    // an axis along which all points are equal adds the same number y^2 to every distance: one
+    // bin of it serves, `wide` across, and the margins allow for the FP64 rounding of sums
+    // with y^2 (|y| < 0.75 wide: 2^-50 wide^2)
+    float ties = 0x1p-120f;
+    if constexpr (DM == 2) {
+        const float wide[2] = {16384.0f * h[1], 16384.0f * h[0]};
+#pragma unroll
+        for (int l = 0; l < DM; ++l) {
+            flat[l] = flat[l] && !flat[1 - l] && 4.0f * fabsf(mn[l]) <= wide[l];
+            if (flat[l]) {
+                h[l] = wide[l];
+                ties = __fmaf_rn(0x1p-50f * h[l], h[l], ties);
+            }
+        }
     }
-    if (DM == 2) hgeo = __fsqrt_rn(hgeo);
+#pragma unroll
+    for (int l = 0; l < DM; ++l) {
+        // two bins beyond the points at least, for d = 1, where the last ones go on.  A
+        // grid without finite sizes has no bins here: `usable` is false for it
+        K[l] = fminf(fmaxf(rintf((fmaxf(0.25f * ext[l], 2.0f * h[l]) - mn[l]) / h[l]), -4194304.0f), 4194304.0f);
+        float far_ = fmaxf(fabsf(K[l]) + 1.0f, fabsf((float)nb[l] - K[l]) + 1.0f) * h[l];
+        if (flat[l]) {
+            K[l] = (float)(nb[l] / 2);
+            far_ = fabsf(mn[l]);
+        } else {
+            hgeo *= h[l];
+        }
+        S = __fmaf_rn(far_, far_, S);
+    }
+    if (DM == 2 && !flat[0] && !flat[DM - 1]) hgeo = __fsqrt_rn(hgeo);
     S = (__fsqrt_rn(S) + R) * 1.0001f;
-    const float er = 0x1p-24f * 1.01f * S + G.err0, e = er + G.err;
+    const float ebox = 0x1p-24f * 1.01f * S, er = ebox + G.err0, e = er + G.err;
     bool usable = S < inf;
 #pragma unroll
-    for (int l = 0; l < DM; ++l) usable = usable && 32.0f * (G.err + G.err0 + 0x1p-21f * S) <= h[l];
+    for (int l = 0; l < DM; ++l) usable = usable && (flat[l] || 32.0f * (G.err + G.err0 + 0x1p-21f * S) <= h[l]);
     // the test's error, as above: rel (D_j + D_i) + fix + slk slack.  (The floors here and in
     // c2: products of the smallest grids fall out of FP32's range)
     constexpr float u2 = 0x1p-23f, slk = 0x1p-20f, sqd = DM == 1 ? 1.0f : 1.41421357f;
@@ -137,7 +173,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
             sum += hw[1];
         }
         rel = u2 * ((float)(DM + 4) + R * sqd / s);
-        fix = u2 * R * (2.0f * sqd * s + 4.0f * sum) + 0x1p-120f;
+        fix = u2 * R * (2.0f * sqd * s + 4.0f * sum) + ties;
     };
     if (blockIdx.y == 0 && tid == 0) {
         const float sq = DM == 1 ? 1.0f : 1.41421357f;
@@ -148,12 +184,21 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
             G.org[l] = 8388608.0f + K[l];
         }
         G.c1 = 2.02f * sq * kappa;
-        G.inv_span = 1.0f / S;
         G.c2 = 2.02f * (sq * (e / kappa) * e + (float)DM * e * e) + 0x1p-120f * (e / er);
-        G.c3 = 2.02f * (float)(DM + 6) * 0x1p-24f;
-        G.ce = 4.04f * sq * e;
+        G.c3 = 2.02f * (float)(DM + (DM == 1 ? 12 : 6)) * 0x1p-24f;   // 12 u D: 2.02 x 6 of them
+        G.e = e;
+        G.ebox = ebox;
         G.f0 = er / e;
     }
+    // a flat axis' bin lies at the points' own coordinate and has no width
+    auto on_axis = [&](float (&c)[DM], float (&hw)[DM]) {
+#pragma unroll
+        for (int l = 0; l < DM; ++l)
+            if (DM == 2 && flat[l]) {
+                c[l] = mn[l];
+                hw[l] = 0.0f;
+            }
+    };
     const int pnx = DM == 1 ? nb[0] / 32 : nb[0] / kPatchX, pny = DM == 1 ? 1 : nb[1] / kPatchY;
     unsigned long long* tab = p.cell_tab + G.toff;
     uint16_t* surv = s_surv[warp];
@@ -174,6 +219,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
             c[1] = ((float)(py * kPatchY) + 1.5f - K[1]) * h[1];
             hw[1] = h[1] * 2.1f;
         }
+        on_axis(c, hw);
         margins(hw);
         float bD = __int_as_float(0x7F800000);
         int bi = 0x7FFFFFFF;
@@ -225,6 +271,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
             c[1] = ((float)y - K[1]) * h[1];
             hw[1] = 0.5f * 1.125f * h[1];
         }
+        on_axis(c, hw);
         margins(hw);
         float D0 = __int_as_float(0x7F800000), D1 = D0;
         int i0 = surv[0], i1 = surv[0];
@@ -266,7 +313,10 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
             if (cnt < kCellInline) ent |= (uint64_t)j << (10 * cnt);
             ++cnt;
         }
-        if (cnt <= kCellInline) {
+        const bool beside = DM == 2 && ((flat[0] && x != nb[0] / 2) || (flat[DM - 1] && y != nb[1] / 2));
+        if (beside) {
+            ent = kCellScanEntry;          // a flat axis has one bin
+        } else if (cnt <= kCellInline) {
             ent |= (uint64_t)cnt << 60;
         } else if (4 * cnt > N) {
             ent = kCellScanEntry;          // a scan of the whole grid is as fast (12 against 4.6 instructions a point)

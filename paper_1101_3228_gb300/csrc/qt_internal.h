@@ -73,9 +73,9 @@ struct alignas(16) CellGrid {
     float inv_h[2];                // bins per unit length
     float org[2];                  // 2^23 + number of the bin centred on 0
     float mu[2];                   // centre (FP32)
-    float c1, c2, c3, ce;          // certificate: 2 err(D) = f (c1 D + c2) + c3 D, 0 < f <= 1; or f (ce sqrt(D) + c2) + c3 D
+    float c1, c2, c3;              // certificate: 2 err(D) = f (c1 D + c2) + c3 D, 0 < f <= 1
+    float e, ebox;                 // bound of a coordinate's error, and the part of it that is FP32 rounding in the box
     float f0;                      // the part of f that does not shrink with the sample's radius
-    float inv_span;                // 1 / S, S = |farthest corner of the box| + R
     float err, err0;               // bounds of the centred samples' error per coordinate beyond FP32 rounding:
                                    // in proportion to their radius, and whatever it is (qt_near.h)
     int32_t N, nb0, nb1;           // points, bins along each axis (nb1 = 1 for d = 1)

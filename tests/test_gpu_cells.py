@@ -279,3 +279,32 @@ def test_located_search_certifies_odd_grids(ctx, B, kind):
     np.testing.assert_array_equal(ii.cpu().numpy(), oracle.nearest(g[0], X[0]))
     np.testing.assert_array_equal(jj.cpu().numpy(), oracle.nearest(g[1], X[1]))
     assert st.rechecks < 0.15 * 2 * M
+
+
+@pytest.mark.parametrize("d", [1, 2])
+@pytest.mark.parametrize("kind", ["flat0", "flat1", "point", "plain"])
+def test_located_cells_far_beyond_the_box(ctx, B, d, kind):
+    """Samples beside the tables, near and very far (1e-3 to 1e18 of the grid's width), where
+    distances tie in FP64; grids with all points equal along an axis, whose table has one bin
+    without an end there, and grids of one distinct point and another next to it."""
+    rng = np.random.default_rng(8)
+    N, M = 300, 40000
+    g = rng.standard_normal((2, N, d))
+    if kind == "point":
+        g[0] = g[0, 0]
+        g[1] = g[1, 0]
+        g[1, 7] += 1e-12
+    elif d == 2 and kind != "plain":
+        g[:, :, int(kind[-1])] = 0.3
+    X = rng.standard_normal((2, M, d)) * 10.0 ** rng.uniform(-3, 18, (2, M, 1))
+    X[:, ::3, 0] = rng.standard_normal((2, len(X[0, ::3])))           # far along one axis only
+    if d == 2:
+        X[:, 1::3, 1] = rng.standard_normal((2, len(X[0, 1::3])))
+    for k in range(2):
+        tie = W.boundary_samples(g[k], 2000, seed=k) if kind != "point" else X[k, :2000]
+        X[k, 2:6000:3] = tie
+    counts, st, ii, jj = ctx.counts_from_samples(_dev(g[0]), _dev(g[1]), _dev(X[0]), _dev(X[1]), B.options(),
+                                                 want_cells=True)
+    np.testing.assert_array_equal(ii.cpu().numpy(), oracle.nearest(g[0], X[0]))
+    np.testing.assert_array_equal(jj.cpu().numpy(), oracle.nearest(g[1], X[1]))
+    assert st.device_status == 0
