@@ -10,6 +10,7 @@ namespace {
 
 constexpr int kBuildThreads = 256;
 constexpr int kBuildWarps = kBuildThreads / 32;
+constexpr int kBuildList = 24;            // kept points of a bin held by its lane
 constexpr int kPatchX = 8, kPatchY = 4;   // bins of a patch, one per lane (d = 1: 32 x 1)
 
 __device__ __forceinline__ float warp_min(float v)
@@ -62,13 +63,15 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
     bool flat[DM];
 #pragma unroll
     for (int l = 0; l < DM; ++l) flat[l] = DM == 2;
+    const long long* g0bits = reinterpret_cast<const long long*>(g64);
+#pragma unroll 4
     for (int j = tid; j < N; j += kBuildThreads) {
         float n2 = 0.0f;
 #pragma unroll
         for (int l = 0; l < DM; ++l) {
-            const double c = g64[(long long)j * DM + l];
-            const float v = __double2float_rn(__dsub_rn(c, (double)G.mu[l]));
-            flat[l] = flat[l] && c == g64[l];
+            const long long bits = g0bits[(long long)j * DM + l];
+            const float v = __double2float_rn(__dsub_rn(__longlong_as_double(bits), (double)G.mu[l]));
+            flat[l] = flat[l] && bits == g0bits[l];
             s_g[j * DM + l] = v;
             mn[l] = fminf(mn[l], v);
             mx[l] = fmaxf(mx[l], v);
@@ -113,7 +116,6 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
     // its centre takes wider bins than its share of the box
     const float R = __fsqrt_rn(r2) * 1.0001f;
     const int nb[2] = {G.nb0, G.nb1};
-    const float inf = __int_as_float(0x7F800000);
     float K[DM], h[DM], ext[DM], S = 0.0f;
 #pragma unroll
     for (int l = 0; l < DM; ++l) {
@@ -159,13 +161,14 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
     if (DM == 2 && !flat[0] && !flat[DM - 1]) hgeo = __fsqrt_rn(hgeo);
     S = (__fsqrt_rn(S) + R) * 1.0001f;
     const float ebox = 0x1p-24f * 1.01f * S, er = ebox + G.err0, e = er + G.err;
-    bool usable = S < inf;
+    bool usable = S < 1e18f;                           // its square is far from overflow
 #pragma unroll
     for (int l = 0; l < DM; ++l) usable = usable && (flat[l] || 32.0f * (G.err + G.err0 + 0x1p-21f * S) <= h[l]);
-    // the test's error, as above: rel (D_j + D_i) + fix + slk slack.  (The floors here and in
-    // c2: products of the smallest grids fall out of FP32's range)
-    constexpr float u2 = 0x1p-23f, slk = 0x1p-20f, sqd = DM == 1 ? 1.0f : 1.41421357f;
-    float rel, fix;
+    // the test's error, as above: rel (D_j + D_i) + fix + 16 u slack; a point is dropped when
+    // D_j (1 - rel) - slack (2 + 16 u) > D_i (1 + rel) + fix.  (The floors here and in c2:
+    // products of the smallest grids fall out of FP32's range)
+    constexpr float u2 = 0x1p-23f, sqd = DM == 1 ? 1.0f : 1.41421357f;
+    float rel, fix, wh[DM];                            // wh: half-widths times 2 + 16 u, for 2 slack + 16 u slack
     auto margins = [&](const float (&hw)[DM]) {
         float s = hw[0], sum = hw[0];
         if constexpr (DM == 2) {
@@ -174,6 +177,8 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         }
         rel = u2 * ((float)(DM + 4) + R * sqd / s);
         fix = u2 * R * (2.0f * sqd * s + 4.0f * sum) + ties;
+#pragma unroll
+        for (int l = 0; l < DM; ++l) wh[l] = hw[l] * (2.0f + 0x1p-20f);
     };
     if (blockIdx.y == 0 && tid == 0) {
         const float sq = DM == 1 ? 1.0f : 1.41421357f;
@@ -223,6 +228,9 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         margins(hw);
         float bD = __int_as_float(0x7F800000);
         int bi = 0x7FFFFFFF;
+        // (unrolled here and below: with few grids a warp has one patch and its SM hardly a
+        // second warp, so that one point at a time costs its latency)
+#pragma unroll 4
         for (int j = lane; j < N; j += 32) {
             float D = 0.0f;
 #pragma unroll
@@ -245,7 +253,12 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
             }
         }
         if (bi >= N) bi = 0;                        // non-finite points: nothing is dropped below
+        float gb[DM];
+#pragma unroll
+        for (int l = 0; l < DM; ++l) gb[l] = s_g[bi * DM + l];
+        const float keepD = 1.0f - rel, over = __fmaf_rn(1.0f + rel, bD, fix);
         int ns = 0;
+#pragma unroll 4
         for (int j0 = 0; j0 < N; j0 += 32) {
             const int j = j0 + lane;
             bool keep = false;
@@ -253,11 +266,11 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
                 float D = 0.0f, slack = 0.0f;
 #pragma unroll
                 for (int l = 0; l < DM; ++l) {
-                    const float t = s_g[j * DM + l] - c[l];
+                    const float gj = s_g[j * DM + l], t = gj - c[l];
                     D = __fmaf_rn(t, t, D);
-                    slack = __fmaf_rn(fabsf(s_g[j * DM + l] - s_g[bi * DM + l]), hw[l], slack);
+                    slack = __fmaf_rn(fabsf(gj - gb[l]), wh[l], slack);
                 }
-                keep = !(D - bD - 2.0f * slack > __fmaf_rn(rel, D + bD, __fmaf_rn(slk, slack, fix)));
+                keep = !(__fmaf_rn(D, keepD, -slack) > over);
             }
             const unsigned m = __ballot_sync(0xFFFFFFFFu, keep);
             if (keep) surv[ns + __popc(m & ((1u << lane) - 1u))] = (uint16_t)j;
@@ -275,6 +288,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         margins(hw);
         float D0 = __int_as_float(0x7F800000), D1 = D0;
         int i0 = surv[0], i1 = surv[0];
+#pragma unroll 4
         for (int t = 0; t < ns; ++t) {
             const int j = surv[t];
             float D = 0.0f;
@@ -283,36 +297,45 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
                 const float v = s_g[j * DM + l] - c[l];
                 D = __fmaf_rn(v, v, D);
             }
-            if (D < D0) {
-                D1 = D0;
-                i1 = i0;
-                D0 = D;
-                i0 = j;
-            } else if (D < D1) {
-                D1 = D;
-                i1 = j;
-            }
+            const bool first = D < D0, next = D < D1;
+            i1 = first ? i0 : (next ? j : i1);
+            D1 = first ? D0 : (next ? D : D1);
+            i0 = first ? j : i0;
+            D0 = first ? D : D0;
         }
+        float g0[DM], g1[DM];
+#pragma unroll
+        for (int l = 0; l < DM; ++l) {
+            g0[l] = s_g[i0 * DM + l];
+            g1[l] = s_g[i1 * DM + l];
+        }
+        const float rest = 1.0f - rel, o0 = __fmaf_rn(1.0f + rel, D0, fix), o1 = __fmaf_rn(1.0f + rel, D1, fix);
         auto keeps = [&](int j) {
             float D = 0.0f, sl0 = 0.0f, sl1 = 0.0f;
 #pragma unroll
             for (int l = 0; l < DM; ++l) {
                 const float gj = s_g[j * DM + l], v = gj - c[l];
                 D = __fmaf_rn(v, v, D);
-                sl0 = __fmaf_rn(fabsf(gj - s_g[i0 * DM + l]), hw[l], sl0);
-                sl1 = __fmaf_rn(fabsf(gj - s_g[i1 * DM + l]), hw[l], sl1);
+                sl0 = __fmaf_rn(fabsf(gj - g0[l]), wh[l], sl0);
+                sl1 = __fmaf_rn(fabsf(gj - g1[l]), wh[l], sl1);
             }
-            return !(D - D0 - 2.0f * sl0 > __fmaf_rn(rel, D + D0, __fmaf_rn(slk, sl0, fix))) &&
-                   !(D - D1 - 2.0f * sl1 > __fmaf_rn(rel, D + D1, __fmaf_rn(slk, sl1, fix)));
+            return !(__fmaf_rn(D, rest, -sl0) > o0) && !(__fmaf_rn(D, rest, -sl1) > o1);
         };
-        uint64_t ent = 0;
+        // kept points, in order, 32 survivors at a time; a lane keeps one or two
+        uint16_t list[kBuildList];
         int cnt = 0;
-        for (int t = 0; t < ns; ++t) {
-            const int j = surv[t];
-            if (!keeps(j)) continue;
-            if (cnt < kCellInline) ent |= (uint64_t)j << (10 * cnt);
-            ++cnt;
+        for (int t0 = 0; t0 < ns; t0 += 32) {
+            const int nt = min(32, ns - t0);
+            uint32_t kept = 0;
+#pragma unroll 8
+            for (int t = 0; t < nt; ++t) kept |= keeps(surv[t0 + t]) ? 1u << t : 0u;
+            for (; kept; kept &= kept - 1) {
+                if (cnt < kBuildList) list[cnt] = surv[t0 + __ffs((int)kept) - 1];
+                ++cnt;
+            }
         }
+        uint64_t ent = 0;
+        for (int t = 0; t < min(cnt, kCellInline); ++t) ent |= (uint64_t)list[t] << (10 * t);
         const bool beside = DM == 2 && ((flat[0] && x != nb[0] / 2) || (flat[DM - 1] && y != nb[1] / 2));
         if (beside) {
             ent = kCellScanEntry;          // a flat axis has one bin
@@ -323,10 +346,12 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         } else {
             const unsigned long long off = atomicAdd(p.cell_cursor, (unsigned long long)cnt);
             if (pool_holds(off, (uint32_t)cnt, p.cell_pool_cap)) {
-                int w = 0;
-                for (int t = 0; t < ns; ++t) {
-                    const int j = surv[t];
-                    if (keeps(j)) p.cell_pool[off + w++] = (uint16_t)j;
+                if (cnt <= kBuildList) {
+                    for (int t = 0; t < cnt; ++t) p.cell_pool[off + t] = list[t];
+                } else {
+                    int w = 0;
+                    for (int t = 0; t < ns; ++t)
+                        if (keeps(surv[t])) p.cell_pool[off + w++] = surv[t];
                 }
                 ent = off | ((uint64_t)cnt << 32) | ((uint64_t)kCellPool << 60);
             } else {
