@@ -543,7 +543,11 @@ qt_status make_plan_full(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
     for (int g = 0; g < P.ngrids; ++g) {
         GridInfo& G = P.grids[g];
         memset(&G, 0, sizeof G);
-        for (int l = 0; l < d; ++l) G.mu[l] = (float)mus[(long long)g * d + l];
+        // (any centre serves; the path-wise form's model need not state the later layers')
+        for (int l = 0; l < d; ++l) {
+            const float c = (float)mus[(long long)g * d + l];
+            G.mu[l] = std::isfinite(c) ? c : 0.0f;
+        }
         G.R = 0.0f;
         G.N = (int)Ns[g];
         G.Npad = P.form != kPlainF64 ? (int)round_up(Ns[g], kChunk) : (int)Ns[g];
@@ -565,7 +569,7 @@ qt_status make_plan_full(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
         for (int g = 0; g < P.ngrids; ++g) {
             CellGrid& C = P.cells[g];
             memset(&C, 0, sizeof C);
-            for (int l = 0; l < d; ++l) C.mu[l] = P.grids[g].mu[l];
+            for (int l = 0; l < d; ++l) C.mu[l] = C.mu0[l] = P.grids[g].mu[l];
             C.N = (int)Ns[g];
             C.goff = P.grids[g].goff;
             C.toff = P.cell_entries;
@@ -932,6 +936,7 @@ qt_status enqueue_forward(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long
         fp.cell_g0 = P.cell_g0;
         fp.cell_g1 = P.cell_g1;
         fp.cell_near = (const float*)(dt + T.near);
+        fp.cell_recentre = !(source == kSampler && P.form == kCells && o->sample_prec == QT_PREC_F64);
         fp.cell_tile = P.cell_tile;
         fp.cell_ipl = P.cell_g1 - P.cell_g0 == P.ngrids ? P.layers[0].items : 0;
         cudaError_t ce = launch_build_cells(P.d, fp, ctx->num_sms, st);

@@ -54,59 +54,79 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
     if (N <= 1) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const double* g64 = p.g64 + G.goff * DM;
-    float mn[DM], mx[DM], r2 = 0.0f;
-#pragma unroll
-    for (int l = 0; l < DM; ++l) {
-        mn[l] = __int_as_float(0x7F800000);
-        mx[l] = -__int_as_float(0x7F800000);
-    }
+    // centred points, their extent and norm.  A grid far from the host's centre (given samples
+    // come with none, and the path-wise form's model states the first layer's only) is
+    // centred on its own middle instead: rounding is relative to the distance from it
+    float mn[DM], mx[DM], mu[DM], r2;
     bool flat[DM];
-#pragma unroll
-    for (int l = 0; l < DM; ++l) flat[l] = DM == 2;
     const long long* g0bits = reinterpret_cast<const long long*>(g64);
+#pragma unroll
+    for (int l = 0; l < DM; ++l) mu[l] = G.mu0[l];
+    for (int pass = 0;; ++pass) {
+        r2 = 0.0f;
+#pragma unroll
+        for (int l = 0; l < DM; ++l) {
+            mn[l] = __int_as_float(0x7F800000);
+            mx[l] = -__int_as_float(0x7F800000);
+            flat[l] = DM == 2;
+        }
 #pragma unroll 4
-    for (int j = tid; j < N; j += kBuildThreads) {
-        float n2 = 0.0f;
+        for (int j = tid; j < N; j += kBuildThreads) {
+            float n2 = 0.0f;
+#pragma unroll
+            for (int l = 0; l < DM; ++l) {
+                const long long bits = g0bits[(long long)j * DM + l];
+                const float v = __double2float_rn(__dsub_rn(__longlong_as_double(bits), (double)mu[l]));
+                flat[l] = flat[l] && bits == g0bits[l];
+                s_g[j * DM + l] = v;
+                mn[l] = fminf(mn[l], v);
+                mx[l] = fmaxf(mx[l], v);
+                n2 = __fmaf_rn(v, v, n2);
+                if (blockIdx.y == 0) p.cell_rec[G.roff + (long long)j * DM + l] = v;
+            }
+            r2 = fmaxf(r2, n2);
+        }
 #pragma unroll
         for (int l = 0; l < DM; ++l) {
-            const long long bits = g0bits[(long long)j * DM + l];
-            const float v = __double2float_rn(__dsub_rn(__longlong_as_double(bits), (double)G.mu[l]));
-            flat[l] = flat[l] && bits == g0bits[l];
-            s_g[j * DM + l] = v;
-            mn[l] = fminf(mn[l], v);
-            mx[l] = fmaxf(mx[l], v);
-            n2 = __fmaf_rn(v, v, n2);
-            if (blockIdx.y == 0) p.cell_rec[G.roff + (long long)j * DM + l] = v;
+            mn[l] = warp_min(mn[l]);
+            mx[l] = warp_max(mx[l]);
+            if (lane == 0) {
+                s_red[warp][2 * l] = mn[l];
+                s_red[warp][2 * l + 1] = mx[l];
+            }
         }
-        r2 = fmaxf(r2, n2);
-    }
+        r2 = warp_max(r2);
+        if (lane == 0) s_red[warp][2 * DM] = r2;
+        int some = 0;                                  // bit l: axis l is not flat
 #pragma unroll
-    for (int l = 0; l < DM; ++l) {
-        mn[l] = warp_min(mn[l]);
-        mx[l] = warp_max(mx[l]);
-        if (lane == 0) {
-            s_red[warp][2 * l] = mn[l];
-            s_red[warp][2 * l + 1] = mx[l];
+        for (int l = 0; l < DM; ++l) some |= flat[l] ? 0 : 1 << l;
+        some = (int)__reduce_or_sync(0xFFFFFFFFu, (unsigned)some);
+        if (lane == 0) s_some[warp] = some;
+        __syncthreads();
+        for (int w = 0; w < kBuildWarps; ++w) {
+            some |= s_some[w];
+#pragma unroll
+            for (int l = 0; l < DM; ++l) {
+                mn[l] = fminf(mn[l], s_red[w][2 * l]);
+                mx[l] = fmaxf(mx[l], s_red[w][2 * l + 1]);
+            }
+            r2 = fmaxf(r2, s_red[w][2 * DM]);
         }
-    }
-    r2 = warp_max(r2);
-    if (lane == 0) s_red[warp][2 * DM] = r2;
-    int some = 0;                                      // bit l: axis l is not flat
 #pragma unroll
-    for (int l = 0; l < DM; ++l) some |= flat[l] ? 0 : 1 << l;
-    some = (int)__reduce_or_sync(0xFFFFFFFFu, (unsigned)some);
-    if (lane == 0) s_some[warp] = some;
-    __syncthreads();
-    for (int w = 0; w < kBuildWarps; ++w) some |= s_some[w];
-#pragma unroll
-    for (int l = 0; l < DM; ++l) flat[l] = (some & (1 << l)) == 0;
-    for (int w = 0; w < kBuildWarps; ++w) {
+        for (int l = 0; l < DM; ++l) flat[l] = (some & (1 << l)) == 0;
+        if (pass > 0 || !p.cell_recentre) break;
+        bool off = false;
+        float mid[DM];
 #pragma unroll
         for (int l = 0; l < DM; ++l) {
-            mn[l] = fminf(mn[l], s_red[w][2 * l]);
-            mx[l] = fmaxf(mx[l], s_red[w][2 * l + 1]);
+            mid[l] = (float)((double)mu[l] + 0.5 * ((double)mn[l] + (double)mx[l]));
+            off = off || fabsf(mn[l] + mx[l]) > 4.0f * (mx[l] - mn[l]);
         }
-        r2 = fmaxf(r2, s_red[w][2 * DM]);
+        // (sizes that are not finite stay with the host's centre; the same in every CTA)
+        if (!off || !(fabsf(mid[0]) < 1e30f) || !(fabsf(mid[DM - 1]) < 1e30f)) break;
+#pragma unroll
+        for (int l = 0; l < DM; ++l) mu[l] = mid[l];
+        __syncthreads();
     }
     // the box: the grid's own, a quarter of its width wider on every side (quantizers
     // reach about 3 standard deviations, so the box reaches 4.5); bin b of an axis is
@@ -185,6 +205,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         const float kappa = fmaxf(0x1p-22f, e / (2.0f * hgeo));
 #pragma unroll
         for (int l = 0; l < DM; ++l) {
+            G.mu[l] = mu[l];
             G.inv_h[l] = 1.0f / h[l];
             G.org[l] = 8388608.0f + K[l];
         }

@@ -72,7 +72,8 @@ struct GridInfo {
 struct alignas(16) CellGrid {
     float inv_h[2];                // bins per unit length
     float org[2];                  // 2^23 + number of the bin centred on 0
-    float mu[2];                   // centre (FP32)
+    float mu[2];                   // centre (FP32): the host's or the grid's own
+    float mu0[2];                  // the host's
     float c1, c2, c3;              // certificate: 2 err(D) = f (c1 D + c2) + c3 D, 0 < f <= 1
     float e, ebox;                 // bound of a coordinate's error, and the part of it that is FP32 rounding in the box
     float f0;                      // the part of f that does not shrink with the sample's radius
@@ -164,6 +165,7 @@ struct ForwardParams {
     unsigned long long* cell_cursor; // pool words asked for
     uint32_t cell_pool_cap;        // pool words
     int32_t cell_g0, cell_g1;      // grids [g0, g1) to build
+    int32_t cell_recentre;         // the search may take the grids' own centres
     const float* cell_near;        // [n][kCellNearStride] combined FP32 parameters of FP64 layers
     long long cell_tile;           // path-wise form: paths per work item
     long long cell_ipl;            // work items of every layer (0: only one layer has any)

@@ -308,3 +308,37 @@ def test_located_cells_far_beyond_the_box(ctx, B, d, kind):
     np.testing.assert_array_equal(ii.cpu().numpy(), oracle.nearest(g[0], X[0]))
     np.testing.assert_array_equal(jj.cpu().numpy(), oracle.nearest(g[1], X[1]))
     assert st.device_status == 0
+
+
+@pytest.mark.parametrize("d", [1, 2])
+def test_located_search_centres_far_grids(ctx, B, d):
+    """Given samples at 100 with a spread of 1e-4: FP32 coordinates about zero have steps of
+    7.6e-6, about the grid's own middle 1e-11, so that few searches need FP64."""
+    rng = np.random.default_rng(12)
+    M, N = 20000, 400
+    g, X = 100.0 + 1e-4 * rng.standard_normal((2, N, d)), 100.0 + 1e-4 * rng.standard_normal((2, M, d))
+    counts, st, ii, jj = ctx.counts_from_samples(_dev(g[0]), _dev(g[1]), _dev(X[0]), _dev(X[1]), B.options(),
+                                                 want_cells=True)
+    np.testing.assert_array_equal(ii.cpu().numpy(), oracle.nearest(g[0], X[0]))
+    np.testing.assert_array_equal(jj.cpu().numpy(), oracle.nearest(g[1], X[1]))
+    assert st.rechecks < 0.15 * 2 * M
+
+
+@pytest.mark.parametrize("d,prec", [(1, W.PREC_F32), (1, W.PREC_F64), (2, W.PREC_F32), (2, W.PREC_F64), (3, W.PREC_F32)])
+@pytest.mark.parametrize("later", [0.0, np.nan])
+def test_paths_read_the_first_mean_only(ctx, B, d, prec, later):
+    """Algorithm II reads the model's mean for the first layer only: zero or undefined later
+    ones change nothing."""
+    M, n = 20011, 3
+    model, g = _chain(d, n, (60, 200, 33), M, 0.1, 4.6)
+    m = model.m.copy()
+    m[1:] = later
+    ref = oracle.pathwise(model, g, M, model.seed, prec)
+    ref = ref[0] if isinstance(ref, tuple) else ref
+    other = W.Model("m", d, n, model.N, model.A, model.b, model.T, m, model.L, model.t, 0.0, "put_exp1d", 1.0, None, M, 99,
+                    prec, "kmeans")
+    counts, st, _ = ctx.transitions_pathwise(other, _dev(g), M, model.seed, B.options(prec=prec))
+    got = B.split_counts(model.N, counts.cpu().numpy())
+    for k in range(n):
+        np.testing.assert_array_equal(got[k], ref[k], err_msg=f"layer {k}")
+    assert st.device_status == 0
