@@ -575,8 +575,9 @@ qt_status make_plan_full(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
             C.toff = P.cell_entries;
             C.roff = P.cell_floats;
             if (C.N > 1) {
-                cell_bins(d, C.N, &C.nb0, &C.nb1);
-                P.cell_entries += (long long)C.nb0 * C.nb1;
+                int nb1;
+                cell_bins(d, C.N, &C.nb, &nb1);
+                P.cell_entries += (long long)C.nb * nb1;
                 P.cell_floats += round_up((long long)C.N * d, 4);
             }
             const size_t b = cell_bytes(d, C.N);

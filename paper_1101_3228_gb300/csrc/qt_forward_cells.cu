@@ -135,13 +135,22 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
     // product grid with one point, two factors of very different size) or a grid far from
     // its centre takes wider bins than its share of the box
     const float R = __fsqrt_rn(r2) * 1.0001f;
-    const int nb[2] = {G.nb0, G.nb1};
+    int nb[2] = {G.nb, DM == 2 ? G.nb : 1};
     float K[DM], h[DM], ext[DM], S = 0.0f;
 #pragma unroll
     for (int l = 0; l < DM; ++l) {
         ext[l] = fmaxf(mx[l] - mn[l], 1e-30f);
         const float far_ = fmaxf(fabsf(mn[l]), fabsf(mx[l])) + ext[l];
         S = __fmaf_rn(far_, far_, S);
+    }
+    if constexpr (DM == 2) {
+        // about as wide as high, where the extents differ by more than two: Voronoi cells are
+        // (ten times as long as high, 1000 points: 6 candidates a bin against 3)
+        const float room = (float)(nb[0] * nb[0]), r = ext[0] / ext[DM - 1];
+        float n0 = r > 2.0f || r < 0.5f ? (float)nb[0] * __fsqrt_rn(r) : (float)nb[0];
+        if (flat[0] != flat[DM - 1]) n0 = flat[0] ? 8.0f : 0.25f * room;
+        nb[0] = (int)(fminf(fmaxf(n0, 8.0f), 0.125f * room) * 0.125f) * 8;
+        nb[1] = (int)(room / (float)nb[0] * 0.25f) * 4;
     }
     // (the wider bins make S larger by less than a quarter: 32 2^-21 8192 = 1/8 for d = 1)
     const float need = 32.0f * 1.3f * (G.err + G.err0 + 0x1p-21f * (__fsqrt_rn(S) + R));
@@ -214,6 +223,8 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         G.c3 = 2.02f * (float)(DM + (DM == 1 ? 12 : 6)) * 0x1p-24f;   // 12 u D: 2.02 x 6 of them
         G.e = e;
         G.ebox = ebox;
+        G.nb0 = nb[0];
+        G.nb1 = nb[1];
         G.f0 = er / e;
     }
     // a flat axis' bin lies at the points' own coordinate and has no width

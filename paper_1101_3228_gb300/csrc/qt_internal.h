@@ -79,7 +79,8 @@ struct alignas(16) CellGrid {
     float f0;                      // the part of f that does not shrink with the sample's radius
     float err, err0;               // bounds of the centred samples' error per coordinate beyond FP32 rounding:
                                    // in proportion to their radius, and whatever it is (qt_near.h)
-    int32_t N, nb0, nb1;           // points, bins along each axis (nb1 = 1 for d = 1)
+    int32_t N, nb;                 // points, bins an axis that the table has room for
+    int32_t nb0, nb1;              // bins along each axis (nb1 = 1 for d = 1), nb0 nb1 <= nb^d
     long long goff;                // first point in the FP64 grids
     long long toff;                // first entry of the table
     long long roff;                // first float of the FP32 records

@@ -342,3 +342,20 @@ def test_paths_read_the_first_mean_only(ctx, B, d, prec, later):
     for k in range(n):
         np.testing.assert_array_equal(got[k], ref[k], err_msg=f"layer {k}")
     assert st.device_status == 0
+
+
+@pytest.mark.parametrize("ratio", [1e-6, 1e-3, 0.01, 0.1, 0.4, 3.0, 30.0, 1e4])
+@pytest.mark.parametrize("N", [2, 3, 17, 1024])
+def test_located_cells_of_long_grids(ctx, B, ratio, N):
+    """Grids much longer than high and the reverse: the table's bins follow the extents (8 bins
+    at least along either axis)."""
+    rng = np.random.default_rng(N)
+    g, X = rng.standard_normal((2, N, 2)), 1.5 * rng.standard_normal((2, 9001, 2))
+    g[:, :, 1] *= ratio
+    X[:, :, 1] *= ratio
+    X[0, ::3], X[1, ::3] = W.boundary_samples(g[0], 3001, 1, 1e-9), W.boundary_samples(g[1], 3001, 2, 1e-9)
+    counts, st, ii, jj = ctx.counts_from_samples(_dev(g[0]), _dev(g[1]), _dev(X[0]), _dev(X[1]), B.options(),
+                                                 want_cells=True)
+    np.testing.assert_array_equal(ii.cpu().numpy(), oracle.nearest(g[0], X[0]))
+    np.testing.assert_array_equal(jj.cpu().numpy(), oracle.nearest(g[1], X[1]))
+    assert st.device_status == 0
