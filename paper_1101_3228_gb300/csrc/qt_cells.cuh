@@ -24,12 +24,14 @@
 // points lie much closer together than their box tells, and outside the box.  Otherwise
 // the exact FP64 distances of the bin's candidates decide.
 //
-// Outside the box the whole grid is searched, but for d = 1 the last bin of either side
-// serves up to 2^20 bins beyond: D_j - D_i = (g_i - g_j)(2 x - g_i - g_j) only grows there.
-// (Further out distances tie in FP64: a point is dropped for being 5 u r nearer at least, r
-// > 2 bins the distance to it, so ties begin at 2^51 5 u r / 2.)  There |a| <= R + sqrt(D),
-// and the excess of 4 sqrt(D) u (2 R + 3 sqrt(D)) over the box's bound is the 12 u D that c3
-// has more.  An axis along which all points are equal has one bin of 2^14 of the other's:
+// Outside the box the first and last bins go on.  For d = 1 they do for 2^20 bins without
+// further ado: D_j - D_i = (g_i - g_j)(2 x - g_i - g_j) only grows there.  For d = 2 a point
+// further out than the witness may be dropped from such a bin only if it is further away all
+// along the 4096 bins beyond.  (Further out distances tie in FP64, 2^-52 r^2; a point is
+// dropped for being 5 u D nearer at least, D the squared distance from the bin, or u R h.)
+// Beside the box |a| <= R + sqrt(D), and the excess of 4 sqrt(d D) u (2 R + 3 sqrt(D)) over
+// the box's bound is the 12 sqrt(d) u D that c3 has more.  Beyond that the whole grid is
+// searched.  An axis along which all points are equal has one bin of 2^14 of the other's:
 // what it adds to the distances is the same number for all points.
 //
 // Why bins: brute force spends 2 d flops on each of N_k + N_{k+1} candidates (1000
@@ -43,6 +45,7 @@
 namespace qt {
 
 constexpr int kCellInline = 6;         // indices held in an entry
+constexpr int kCellBeyond = 4096;      // d = 2: bins beyond the table that its first and last ones serve
 constexpr int kCellPool = 15;          // entry refers to the pool
 constexpr int kCellScan = 14;          // entry stands for the whole grid
 constexpr uint64_t kCellScanEntry = (uint64_t)kCellScan << 60;
@@ -201,8 +204,15 @@ __device__ __forceinline__ int cell_search(const CellGrid& G, const unsigned cha
         b = (uint32_t)__float_as_int(fminf(fmaxf(v, 8388608.0f), 8388607.0f + (float)G.nb0)) - 0x4B000000u;
         in = fabsf(v - 8388608.0f) <= 1048576.0f;
     } else {
-        const uint32_t b1 = cell_bin(a[1], axes.y, axes.w);
+        uint32_t b1 = cell_bin(a[1], axes.y, axes.w);
         in = in && b1 < (uint32_t)G.nb1;
+        if (!in) {
+            // beside the table: the first and last bins go on for kCellBeyond more
+            const float v0 = __fmaf_rn(a[0], axes.x, axes.z) - 8388608.0f, v1 = __fmaf_rn(a[1], axes.y, axes.w) - 8388608.0f;
+            in = fabsf(v0) <= (float)kCellBeyond && fabsf(v1) <= (float)kCellBeyond;
+            b = (uint32_t)fminf(fmaxf(v0, 0.0f), (float)G.nb0 - 1.0f);
+            b1 = (uint32_t)fminf(fmaxf(v1, 0.0f), (float)G.nb1 - 1.0f);
+        }
         b += b1 * (uint32_t)G.nb0;
     }
     uint64_t e = kCellScanEntry;

@@ -198,16 +198,26 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
     // products of the smallest grids fall out of FP32's range)
     constexpr float u2 = 0x1p-23f, sqd = DM == 1 ? 1.0f : 1.41421357f;
     float rel, fix, wh[DM];                            // wh: half-widths times 2 + 16 u, for 2 slack + 16 u slack
+    // edge[l]: the box (of a patch or a bin) is the first (bit 0) or last (bit 1) of axis l and
+    // goes on for kCellBeyond bins there (d = 2): outwards `far_wh` takes the place of wh
+    float far_wh[DM];
+    int edge[DM];
     auto margins = [&](const float (&hw)[DM]) {
         float s = hw[0], sum = hw[0];
         if constexpr (DM == 2) {
             s = fmaxf(s, hw[1]);
             sum += hw[1];
         }
+#pragma unroll
+        for (int l = 0; l < DM; ++l)
+            if (edge[l] != 0) sum += (float)(kCellBeyond + 1) * h[l];
         rel = u2 * ((float)(DM + 4) + R * sqd / s);
         fix = u2 * R * (2.0f * sqd * s + 4.0f * sum) + ties;
 #pragma unroll
-        for (int l = 0; l < DM; ++l) wh[l] = hw[l] * (2.0f + 0x1p-20f);
+        for (int l = 0; l < DM; ++l) {
+            wh[l] = hw[l] * (2.0f + 0x1p-20f);
+            far_wh[l] = (float)(kCellBeyond + 1) * h[l] * (2.0f + 0x1p-20f);
+        }
     };
     if (blockIdx.y == 0 && tid == 0) {
         const float sq = DM == 1 ? 1.0f : 1.41421357f;
@@ -220,13 +230,20 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         }
         G.c1 = 2.02f * sq * kappa;
         G.c2 = 2.02f * (sq * (e / kappa) * e + (float)DM * e * e) + 0x1p-120f * (e / er);
-        G.c3 = 2.02f * (float)(DM + (DM == 1 ? 12 : 6)) * 0x1p-24f;   // 12 u D: 2.02 x 6 of them
+        G.c3 = 2.02f * (float)(DM + (DM == 1 ? 12 : 15)) * 0x1p-24f;   // 12 sqrt(d) u D: 2.02 x 6 and 9 of them
         G.e = e;
         G.ebox = ebox;
         G.nb0 = nb[0];
         G.nb1 = nb[1];
         G.f0 = er / e;
     }
+    // 2 slack + 16 u slack of axis l for two points whose coordinates differ by dl, on a box with
+    // or without an edge
+    auto slack_in = [&](float dl, int l, float acc) { return __fmaf_rn(fabsf(dl), wh[l], acc); };
+    auto slack_edge = [&](float dl, int l, float acc) {
+        const bool out = (edge[l] & (dl > 0.0f ? 2 : 1)) != 0;
+        return __fmaf_rn(fabsf(dl), out ? far_wh[l] : wh[l], acc);
+    };
     // a flat axis' bin lies at the points' own coordinate and has no width
     auto on_axis = [&](float (&c)[DM], float (&hw)[DM]) {
 #pragma unroll
@@ -257,6 +274,15 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
             hw[1] = h[1] * 2.1f;
         }
         on_axis(c, hw);
+        edge[0] = DM == 1 ? 0 : (px == 0 ? 1 : 0) | (px == pnx - 1 ? 2 : 0);
+        if constexpr (DM == 2) edge[1] = (py == 0 ? 1 : 0) | (py == pny - 1 ? 2 : 0);
+        bool at_edge = false;
+#pragma unroll
+        for (int l = 0; l < DM; ++l) {
+            if (flat[l]) edge[l] = 0;
+            at_edge = at_edge || edge[l] != 0;
+        }
+        const int patch_edge[2] = {edge[0], DM == 2 ? edge[DM - 1] : 0};
         margins(hw);
         float bD = __int_as_float(0x7F800000);
         int bi = 0x7FFFFFFF;
@@ -290,24 +316,28 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
         for (int l = 0; l < DM; ++l) gb[l] = s_g[bi * DM + l];
         const float keepD = 1.0f - rel, over = __fmaf_rn(1.0f + rel, bD, fix);
         int ns = 0;
+        auto survivors = [&](auto slack_of) {
 #pragma unroll 4
-        for (int j0 = 0; j0 < N; j0 += 32) {
-            const int j = j0 + lane;
-            bool keep = false;
-            if (j < N) {
-                float D = 0.0f, slack = 0.0f;
+            for (int j0 = 0; j0 < N; j0 += 32) {
+                const int j = j0 + lane;
+                bool keep = false;
+                if (j < N) {
+                    float D = 0.0f, slack = 0.0f;
 #pragma unroll
-                for (int l = 0; l < DM; ++l) {
-                    const float gj = s_g[j * DM + l], t = gj - c[l];
-                    D = __fmaf_rn(t, t, D);
-                    slack = __fmaf_rn(fabsf(gj - gb[l]), wh[l], slack);
+                    for (int l = 0; l < DM; ++l) {
+                        const float gj = s_g[j * DM + l], t = gj - c[l];
+                        D = __fmaf_rn(t, t, D);
+                        slack = slack_of(gj - gb[l], l, slack);
+                    }
+                    keep = !(__fmaf_rn(D, keepD, -slack) > over);
                 }
-                keep = !(__fmaf_rn(D, keepD, -slack) > over);
+                const unsigned m = __ballot_sync(0xFFFFFFFFu, keep);
+                if (keep) surv[ns + __popc(m & ((1u << lane) - 1u))] = (uint16_t)j;
+                ns += __popc(m);
             }
-            const unsigned m = __ballot_sync(0xFFFFFFFFu, keep);
-            if (keep) surv[ns + __popc(m & ((1u << lane) - 1u))] = (uint16_t)j;
-            ns += __popc(m);
-        }
+        };
+        if (at_edge) survivors(slack_edge);
+        else survivors(slack_in);
         __syncwarp();
         // ---- this lane's bin
         c[0] = ((float)x - K[0]) * h[0];
@@ -317,6 +347,8 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
             hw[1] = 0.5f * 1.125f * h[1];
         }
         on_axis(c, hw);
+        edge[0] = patch_edge[0] & ((x == 0 ? 1 : 0) | (x == nb[0] - 1 ? 2 : 0));
+        if constexpr (DM == 2) edge[1] = patch_edge[1] & ((y == 0 ? 1 : 0) | (y == nb[1] - 1 ? 2 : 0));
         margins(hw);
         float D0 = __int_as_float(0x7F800000), D1 = D0;
         int i0 = surv[0], i1 = surv[0];
@@ -342,30 +374,34 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
             g1[l] = s_g[i1 * DM + l];
         }
         const float rest = 1.0f - rel, o0 = __fmaf_rn(1.0f + rel, D0, fix), o1 = __fmaf_rn(1.0f + rel, D1, fix);
-        auto keeps = [&](int j) {
+        auto keeps = [&](int j, auto slack_of) {
             float D = 0.0f, sl0 = 0.0f, sl1 = 0.0f;
 #pragma unroll
             for (int l = 0; l < DM; ++l) {
                 const float gj = s_g[j * DM + l], v = gj - c[l];
                 D = __fmaf_rn(v, v, D);
-                sl0 = __fmaf_rn(fabsf(gj - g0[l]), wh[l], sl0);
-                sl1 = __fmaf_rn(fabsf(gj - g1[l]), wh[l], sl1);
+                sl0 = slack_of(gj - g0[l], l, sl0);
+                sl1 = slack_of(gj - g1[l], l, sl1);
             }
             return !(__fmaf_rn(D, rest, -sl0) > o0) && !(__fmaf_rn(D, rest, -sl1) > o1);
         };
         // kept points, in order, 32 survivors at a time; a lane keeps one or two
         uint16_t list[kBuildList];
         int cnt = 0;
-        for (int t0 = 0; t0 < ns; t0 += 32) {
-            const int nt = min(32, ns - t0);
-            uint32_t kept = 0;
+        auto collect = [&](auto slack_of) {
+            for (int t0 = 0; t0 < ns; t0 += 32) {
+                const int nt = min(32, ns - t0);
+                uint32_t kept = 0;
 #pragma unroll 8
-            for (int t = 0; t < nt; ++t) kept |= keeps(surv[t0 + t]) ? 1u << t : 0u;
-            for (; kept; kept &= kept - 1) {
-                if (cnt < kBuildList) list[cnt] = surv[t0 + __ffs((int)kept) - 1];
-                ++cnt;
+                for (int t = 0; t < nt; ++t) kept |= keeps(surv[t0 + t], slack_of) ? 1u << t : 0u;
+                for (; kept; kept &= kept - 1) {
+                    if (cnt < kBuildList) list[cnt] = surv[t0 + __ffs((int)kept) - 1];
+                    ++cnt;
+                }
             }
-        }
+        };
+        if (at_edge) collect(slack_edge);
+        else collect(slack_in);
         uint64_t ent = 0;
         for (int t = 0; t < min(cnt, kCellInline); ++t) ent |= (uint64_t)list[t] << (10 * t);
         const bool beside = DM == 2 && ((flat[0] && x != nb[0] / 2) || (flat[DM - 1] && y != nb[1] / 2));
@@ -383,7 +419,7 @@ __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid
                 } else {
                     int w = 0;
                     for (int t = 0; t < ns; ++t)
-                        if (keeps(surv[t])) p.cell_pool[off + w++] = surv[t];
+                        if (keeps(surv[t], slack_edge)) p.cell_pool[off + w++] = surv[t];
                 }
                 ent = off | ((uint64_t)cnt << 32) | ((uint64_t)kCellPool << 60);
             } else {
