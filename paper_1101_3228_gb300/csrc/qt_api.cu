@@ -407,7 +407,7 @@ struct FwdIO {
 };
 
 qt_status make_plan_full(qt_ctx* ctx, int d, int n, const int64_t* Ns, const double* mus, long long M,
-                         const qt_options* o, bool from_arrays, Plan& P, int algo);
+                         const qt_options* o, bool from_arrays, Plan& P, int algo, bool one_layer);
 
 // Bins along each axis of a grid's table: about 20 per point for d = 2 (the 2-factor
 // grids: 2.6 candidates per search, against 4.3 at 8 per point), at most 104 x 104, so
@@ -431,12 +431,33 @@ size_t cell_bytes(int d, long long N)
     return (size_t)a * b * 8 + (size_t)round_up(N * d, 4) * 4;
 }
 
-// Whether the automatic form takes the located search: d <= 2, indices of ten
-// bits, two tables within one CTA's shared memory and all of them within 1 GiB.  It
-// is the faster one at every size measured (us per call, brute force / located:
-// 4 dates x 3000 pairs on 64 points 125 / 66, 365 x 10^5 on 500 points 5500 / 1200,
-// 100 x 10^7 on 500 points 142900 / 19500, ten FP64 dates x 10^6 on 100 points
-// 3190 / 290); callers that name a form, a tile or the shared-memory histogram get
+// Whether the tables of a located search cost more than they save: n layer pairs of M
+// draws each.  A table takes about (3.5e-5 + 1e-7 N) us a bin for d = 2 and 1.9e-5 for d = 1
+// (all SMs busy; 0.9 us for 500 points, 1.5 for 1000), brute force 1.6e-7 us a pair and
+// candidate and 4.5e-4 d more where the pairs are drawn in FP64.  Few tables hide behind the latency
+// that either form has, so the rule asks only from 20 us of tables on (us per call, brute
+// force / located, d = 2: 365 dates of 500 points, M = 100 234 / 400, 1000 264 / 410, 10000
+// 814 / 520; 20 dates of 500 points, M = 100 73 / 79, and the graph of a repeated call less).
+bool cells_cost_more(int d, int n, const int64_t* Ns, long long M, bool f64)
+{
+    double tables = 0.0, pairs = 0.0;
+    for (int k = 0; k <= n; ++k) {
+        if (Ns[k] > 1) {
+            int x, y;
+            cell_bins(d, Ns[k], &x, &y);
+            tables += (double)x * y * (d == 1 ? 1.9e-5 : 3.5e-5 + 1e-7 * (double)Ns[k]);
+        }
+        if (k < n) pairs += (double)M * (1.6e-7 * (double)(Ns[k] + Ns[k + 1]) + (f64 ? 4.5e-4 * d : 0.0));
+    }
+    return tables > 20.0 && tables > pairs;
+}
+
+// Whether the automatic form can take the located search: d <= 2, indices of ten
+// bits, two tables within one CTA's shared memory and all of them within 1 GiB.  With
+// pairs enough to pay for the tables it is the faster one at every size measured (us per
+// call, brute force / located: 4 dates x 3000 pairs on 64 points 125 / 62, 365 x 10^5 on 500
+// points 5500 / 1100, 100 x 10^7 on 500 points 142900 / 17700, ten FP64 dates x 10^6 on 100
+// points 3190 / 265); callers that name a form, a tile or the shared-memory histogram get
 // the brute-force kernels.
 bool cells_apply(size_t smem, int d, int n, const int64_t* Ns, const qt_options* o)
 {
@@ -472,7 +493,7 @@ long long tc_chunk(const Plan& P, const qt_options* o)
 qt_status make_plan(qt_ctx* ctx, int d, int n, const int64_t* Ns, const double* mus, long long M, const qt_options* o,
                     bool from_arrays, Plan& P, int only_layer = -1, int algo = 3)
 {
-    qt_status s = make_plan_full(ctx, d, n, Ns, mus, M, o, from_arrays, P, algo);
+    qt_status s = make_plan_full(ctx, d, n, Ns, mus, M, o, from_arrays, P, algo, only_layer >= 0);
     if (!s && algo == 2 && only_layer >= 0) return fail(ctx, QT_EUNSUPPORTED, "the path-wise form runs every layer");
     if (s || only_layer < 0) return s;
     if (only_layer >= n) return fail(ctx, QT_EINVAL, "layer %d of %d", only_layer, n);
@@ -495,7 +516,7 @@ qt_status make_plan(qt_ctx* ctx, int d, int n, const int64_t* Ns, const double* 
 // by grid sizes Ns (n+1 entries) and centres mus ((n+1) x d).  algo = 3 is
 // Algorithm III (independent layer pairs), algo = 2 Algorithm II (paths).
 qt_status make_plan_full(qt_ctx* ctx, int d, int n, const int64_t* Ns, const double* mus, long long M,
-                         const qt_options* o, bool from_arrays, Plan& P, int algo)
+                         const qt_options* o, bool from_arrays, Plan& P, int algo, bool one_layer)
 {
     P.d = d;
     P.n = n;
@@ -508,7 +529,8 @@ qt_status make_plan_full(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
         if (from_arrays) return fail(ctx, QT_EUNSUPPORTED, "the path-wise form draws its own paths");
         form = QT_FORM_F32_RECHECK;
     }
-    const bool cells = cells_apply(ctx->smem_optin, d, n, Ns, o);
+    const bool cells = cells_apply(ctx->smem_optin, d, n, Ns, o) &&
+                       (algo == 2 || one_layer || !cells_cost_more(d, n, Ns, M, !from_arrays && o->sample_prec == QT_PREC_F64));
     // automatic choice: the fastest certified form measured on GB300 -- the
     // tensor-core screen for 3 <= d <= 10, the FP32 screen otherwise (for d <= 2 on
     // the few candidates that the located search leaves)

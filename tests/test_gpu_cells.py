@@ -359,3 +359,22 @@ def test_located_cells_of_long_grids(ctx, B, ratio, N):
     np.testing.assert_array_equal(ii.cpu().numpy(), oracle.nearest(g[0], X[0]))
     np.testing.assert_array_equal(jj.cpu().numpy(), oracle.nearest(g[1], X[1]))
     assert st.device_status == 0
+
+
+@pytest.mark.parametrize("d,n,N,Ms", [(2, 80, 500, (60, 5000, 9000)), (2, 300, 100, (50, 1500, 4000)), (1, 300, 500, (40, 900, 3000))])
+@pytest.mark.parametrize("prec", [W.PREC_F32, W.PREC_F64])
+def test_located_and_brute_force_over_the_number_of_pairs(ctx, B, d, n, N, Ms, prec):
+    """Few pairs a date do not pay for the tables of many dates: either side of the line, and
+    the fused price, which takes one date at a time, give the oracle's counts."""
+    model, g = _chain(d, n, [N] * n, max(Ms))
+    G = _dev(g)
+    for M in Ms:
+        ref = np.concatenate([c.reshape(-1) for c in oracle.transitions(model, g, M, model.seed, prec)])
+        counts, st, _ = ctx.transitions(model, G, M, model.seed, B.options(prec=prec))
+        np.testing.assert_array_equal(counts.cpu().numpy(), ref)
+        assert st.form_used == B.FORM_F32_RECHECK and st.device_status == 0
+    phi = np.maximum(1.0 - np.exp(g.sum(1)), 0.0)
+    blocks = oracle.transitions(model, g, Ms[0], model.seed, prec)
+    price, _ = ctx.price(model, g, Ms[0], model.seed, phi, B.options(prec=prec, flags=B.FLAG_FUSED_BACKWARD))
+    want = oracle.price(model.N, blocks, phi)
+    assert abs(price - want) <= 1e-12 * max(abs(want), 1e-300)
