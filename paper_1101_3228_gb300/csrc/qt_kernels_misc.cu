@@ -198,7 +198,7 @@ __device__ __forceinline__ void row_reduce(double& acc, long long& ci)
 }
 
 // One layer, one warp per row; V_{k+1} in shared memory (dynamic: Nk1 doubles) when
-// `staged`, else in device memory and every entry walked.
+// `staged`, else read from L2 by the lists' entries.
 template <typename C>
 __global__ void __launch_bounds__(kRowWarps * 32) backward_layer_kernel(const C* __restrict__ counts, long long coff,
                                                                         int Nk, int Nk1, int staged,
@@ -208,13 +208,12 @@ __global__ void __launch_bounds__(kRowWarps * 32) backward_layer_kernel(const C*
     extern __shared__ __align__(16) double s_v[];
     __shared__ uint32_t s_lst[kRowWarps][kRowSlots][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    bool odd = !staged;
-    if (staged)
-        for (int j = threadIdx.x; j < Nk1; j += kRowWarps * 32) {
-            const double v = Vnext[j];
-            odd = odd || !finite_f64(v);
-            s_v[j] = v;
-        }
+    bool odd = false;
+    for (int j = threadIdx.x; j < Nk1; j += kRowWarps * 32) {
+        const double v = Vnext[j];
+        odd = odd || !finite_f64(v);
+        if (staged) s_v[j] = v;
+    }
     const bool dense = __syncthreads_or(odd) != 0;
     const double* V = staged ? s_v : Vnext;
     for (int i = blockIdx.x * kRowWarps + warp; i < Nk; i += gridDim.x * kRowWarps) {
@@ -236,6 +235,15 @@ __global__ void __launch_bounds__(kRowWarps * 32) backward_layer_kernel(const C*
     }
 }
 
+// Dynamic shared memory beside the lists: up to 16 KB need no leave (a call of its own, 2 us).
+template <typename F>
+static cudaError_t allow_dynamic(F kernel, size_t dyn)
+{
+    constexpr size_t kLists = sizeof(uint32_t) * kRowWarps * kRowSlots * 32;
+    if (kLists + dyn <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+}
+
 cudaError_t launch_backward_layer(const void* counts, int u32, long long coff, int Nk, int Nk1, const double* phik,
                                   const double* Vnext, double* Vk, int num_sms, cudaStream_t st)
 {
@@ -244,15 +252,15 @@ cudaError_t launch_backward_layer(const void* counts, int u32, long long coff, i
     // the CTAs of a large layer take several rows each, so that V is read once for each
     const int per_sm = dyn <= 40 * 1024 ? 3 : (dyn <= 72 * 1024 ? 2 : 1);
     int blocks = (Nk + kRowWarps - 1) / kRowWarps;
-    if (staged && blocks > num_sms * per_sm) blocks = num_sms * per_sm;
+    if (blocks > num_sms * per_sm) blocks = num_sms * per_sm;
     cudaError_t e;
     if (u32) {
-        e = cudaFuncSetAttribute(backward_layer_kernel<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+        e = allow_dynamic(backward_layer_kernel<uint32_t>, dyn);
         if (e != cudaSuccess) return e;
         backward_layer_kernel<uint32_t><<<(unsigned)blocks, kRowWarps * 32, dyn, st>>>((const uint32_t*)counts, coff, Nk,
                                                                                       Nk1, staged, phik, Vnext, Vk);
     } else {
-        e = cudaFuncSetAttribute(backward_layer_kernel<long long>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+        e = allow_dynamic(backward_layer_kernel<long long>, dyn);
         if (e != cudaSuccess) return e;
         backward_layer_kernel<long long><<<(unsigned)blocks, kRowWarps * 32, dyn, st>>>((const long long*)counts, coff,
                                                                                        Nk, Nk1, staged, phik, Vnext, Vk);
@@ -529,14 +537,13 @@ __global__ void __launch_bounds__(kRowWarps * 32) swing_layer_kernel(const C* __
     // consumption states of the chunk whose continuation is feasible at date k + 1
     const int lo = max(0, Qmin - (n - k - 1) - q0), hi = min(kSwingQ, Qmax - q0);
     const double ninf = __longlong_as_double(0xFFF0000000000000LL);
-    bool odd = !staged;
-    if (staged)
-        for (int q = lo; q <= hi; ++q)
-            for (int j = threadIdx.x; j < Nk1; j += kRowWarps * 32) {
-                const double v = Pnext[(long long)(q0 + q) * Nk1 + j];
-                odd = odd || !finite_f64(v);
-                s_P[q * Nk1 + j] = v;
-            }
+    bool odd = false;
+    for (int q = lo; q <= hi; ++q)
+        for (int j = threadIdx.x; j < Nk1; j += kRowWarps * 32) {
+            const double v = Pnext[(long long)(q0 + q) * Nk1 + j];
+            odd = odd || !finite_f64(v);
+            if (staged) s_P[q * Nk1 + j] = v;
+        }
     const bool dense = __syncthreads_or(odd) != 0;
     const double* P = staged ? s_P : Pnext + (long long)q0 * Nk1;
     for (int i = blockIdx.y * kRowWarps + warp; i < Nk; i += gridDim.y * kRowWarps) {
@@ -610,17 +617,17 @@ cudaError_t launch_swing_layer(const void* counts, int u32, long long coff, int 
     // as many row blocks as fill the SMs (a CTA loads the chunk's P once for all its rows)
     const int per_sm = dyn <= 40 * 1024 ? 3 : (dyn <= 72 * 1024 ? 2 : 1);
     int by = (Nk + kRowWarps - 1) / kRowWarps;
-    const int most = staged ? (num_sms * per_sm + chunks - 1) / chunks : 65535;
+    const int most = (num_sms * per_sm + chunks - 1) / chunks;
     if (by > most) by = most;
     const dim3 grid((unsigned)chunks, (unsigned)by);
     cudaError_t e;
     if (u32) {
-        e = cudaFuncSetAttribute(swing_layer_kernel<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+        e = allow_dynamic(swing_layer_kernel<uint32_t>, dyn);
         if (e != cudaSuccess) return e;
         swing_layer_kernel<uint32_t><<<grid, kRowWarps * 32, dyn, st>>>((const uint32_t*)counts, coff, Nk, Nk1, staged,
                                                                        vk, Pnext, Pk, n, k, Qmin, Qmax);
     } else {
-        e = cudaFuncSetAttribute(swing_layer_kernel<long long>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+        e = allow_dynamic(swing_layer_kernel<long long>, dyn);
         if (e != cudaSuccess) return e;
         swing_layer_kernel<long long><<<grid, kRowWarps * 32, dyn, st>>>((const long long*)counts, coff, Nk, Nk1, staged,
                                                                         vk, Pnext, Pk, n, k, Qmin, Qmax);

@@ -131,3 +131,24 @@ def test_root_value_of_many_rows(ctx, B):
         w = blocks[0].sum(1)
         P0 = P.cpu().numpy()[:int(N[0])]
         assert abs(price - (w * P0).sum() / w.sum()) <= 1e-12 * price
+
+
+@pytest.mark.parametrize("N", [[3, 12289, 40], [1, 9, 13000, 64], [2, 30001, 2]])
+@pytest.mark.parametrize("u32", [False, True])
+@pytest.mark.parametrize("density,wide", [(0.02, False), (1.0, False), (0.3, True)])
+def test_backward_values_beyond_shared_memory(ctx, B, N, u32, density, wide):
+    """Layers of more than 12288 points: their values stay in device memory, the lists are the
+    same, and so is the sum of 30001 terms: (30001 + 3) 2^-53 < 4e-12."""
+    N = np.array(N, dtype=np.int64)
+    blocks, dev = _tree(N, u32, density, 1, wide)
+    phi = np.random.default_rng(4).random(int(N.sum())) * 10.0
+    ct = B.COUNTS_U32 if u32 else B.COUNTS_I64
+    for value in (None, np.inf, np.nan):
+        if value is not None:
+            phi[int(N[:2].sum()) - 5] = value
+        ref = _backward(blocks, N, phi)
+        V = ctx.backward(N, dev, torch.from_numpy(phi).cuda(), ct).cpu().numpy()
+        np.testing.assert_array_equal(np.isnan(V), np.isnan(ref))
+        np.testing.assert_array_equal(np.isinf(V), np.isinf(ref))
+        ok = np.isfinite(ref)
+        assert np.max(np.abs(V[ok] - ref[ok]) / np.abs(ref[ok])) < 4e-12
