@@ -628,12 +628,12 @@ __device__ __noinline__ int warp_window_nn(const float (&xs)[DM], float A, const
     const float rad = fmaxf(A2 + U + 0x1p-18f * (A2 + fabsf(U)) + eta, 0.0f);
     const float rho = Ap + __fsqrt_rn(rad);
     const float Erho = cd * (rho * rho + 2.0f * Ap * rho);
-    const float lim = b1 + (E1 + Erho + eta) * 1.25f + 0x1p-20f * fabsf(b1) + 0x1p-100f;
+    float lim = b1 + (E1 + Erho + eta) * 1.25f + 0x1p-20f * fabsf(b1) + 0x1p-100f;
     // exact distances on the window only; on every record where the scores bound nothing (a
     // sample so far out that they overflow).  A sample with no finite distance has no cell:
     // the index returned is out of range, and the callers refuse it
     constexpr int kNone = 0x7FFFFFFF;
-    const bool all = i1 >= N || !(lim < __int_as_float(0x7F800000));
+    if (i1 >= N || !(lim < __int_as_float(0x7F800000))) lim = __int_as_float(0x7F800000);
     double best = __longlong_as_double(0x7FF0000000000000LL);
     int bi = kNone;
     double zz[DM];
@@ -646,9 +646,7 @@ __device__ __noinline__ int warp_window_nn(const float (&xs)[DM], float A, const
             bi = j;
         }
     };
-    if (all) {
-        for (int j = lane; j < N; j += 32) exact(j);
-    } else if (!__any_sync(0xFFFFFFFFu, l3 <= lim)) {
+    if (!__any_sync(0xFFFFFFFFu, l3 <= lim)) {
         if (l1 <= lim) exact(k1);                      // lim is finite: a lane's own record
         if (l2 <= lim) exact(k2);
     } else {
@@ -658,7 +656,7 @@ __device__ __noinline__ int warp_window_nn(const float (&xs)[DM], float A, const
             for (int u = 0; u < kU; ++u) sc[u] = score(min(j0 + 32 * u, N - 1));
 #pragma unroll
             for (int u = 0; u < kU; ++u)
-                if (j0 + 32 * u < N && sc[u] <= lim) exact(j0 + 32 * u);
+                if (j0 + 32 * u < N && !(sc[u] > lim)) exact(j0 + 32 * u);
         }
     }
 #pragma unroll

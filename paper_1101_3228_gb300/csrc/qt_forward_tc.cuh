@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
     constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(kTcTileN >> 3) << 17) | ((uint32_t)(kTcTileM >> 4) << 24);
     extern __shared__ __align__(128) unsigned char dsm_tc[];
     __shared__ __align__(8) unsigned long long s_tfull[kTcMaxSlots], s_cfull[2];
-    __shared__ __align__(8) unsigned long long s_accfull;
+    __shared__ __align__(8) unsigned long long s_accfull, s_meet;
     __shared__ uint32_t s_arrived;
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
@@ -435,6 +435,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
         mbar_init(cfull, 1);
         mbar_init(cfull + 8, 1);
         mbar_init(accfull, 1);
+        mbar_init(smem_u32(&s_meet), kTcThreads / 32);
         s_arrived = 0;
         s_abort = 0;
         fence_proxy_async();
@@ -492,25 +493,12 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
         bulk_g2s(ring_u + (uint32_t)to * kTileBytes,
                  reinterpret_cast<const unsigned char*>(p.tc_tiles) + (long long)src * kTileBytes, kTileBytes, bar);
     };
-    // Samples of this CTA's next item with tiles, from item number ld_s on (thread 0);
-    // their number c picks the buffer.  An item whose grids both have one point needs no
-    // screen: it is skipped here and in the loop below, because nothing between its wait
-    // and the next load would hold the warps together (a warp two loads behind would wait
-    // for the wrong phase).
-    long long ld_s = 0;
-    auto load_samples = [&](long long c) {
-        for (;; ++ld_s) {
-            const long long item = p.item_lo + blockIdx.x + ld_s * G;
-            if (item >= p.item_hi) return;
-            const LayerDesc& L = p.layers[tc_layer(p, item)];
-            if (L.NA > 1 || L.NB > 1) break;
-            ld_s = max(ld_s, (L.item_begin + L.items - p.item_lo - blockIdx.x + G - 1) / G - 1);   // the layer's last
-        }
-        const long long item = p.item_lo + blockIdx.x + ld_s * G;
-        ++ld_s;
-        const uint32_t bar = cfull + (uint32_t)(8 * (c & 1));
+    auto load_samples = [&](long long n) {
+        const long long item = p.item_lo + blockIdx.x + n * G;
+        if (item >= p.item_hi) return;
+        const uint32_t bar = cfull + (uint32_t)(8 * (n & 1));
         mbar_arrive_expect_tx(bar, kCertBytes);
-        bulk_g2s(cert_u + (uint32_t)(c & 1) * kCertBytes,
+        bulk_g2s(cert_u + (uint32_t)(n & 1) * kCertBytes,
                  p.tc_items + (item - p.item_lo) * (long long)(TcItem<DM>::kFloats * 4), kCertBytes, bar);
     };
     if (t == 0) load_samples(0);
@@ -520,11 +508,11 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
     }
 
     int slot = 0;                                      // ring slot and parity of the next tile
-    uint32_t ph = 0, accph = 0;
+    uint32_t ph = 0, accph = 0, meetph = 0;
     long long lend = 0;
     int tA = 0, nT = 0, expA = 0, expB = 0;
-    long long c = 0;                                   // items with tiles before this one
-    for (long long n = 0;; ++n) {
+    long long n = 0;
+    for (;; ++n) {
         const long long item = p.item_lo + blockIdx.x + n * G;
         if (item >= p.item_hi) break;
         if (__shfl_sync(0xFFFFFFFFu, *(volatile int*)&s_abort, 0)) {
@@ -541,15 +529,14 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
             expA = GA.tc_exp;
             expB = GB.tc_exp;
         }
-        if (nT == 0) continue;
         // this item's samples have landed; the next item's go to the other buffer, which
         // every warp has left (all have read the last tile of the item before)
-        if (!warp_wait(cfull + (uint32_t)(8 * (c & 1)), (uint32_t)((c >> 1) & 1), budget)) {
+        if (!warp_wait(cfull + (uint32_t)(8 * (n & 1)), (uint32_t)((n >> 1) & 1), budget)) {
             ok = false;
             break;
         }
-        if (t == 0) load_samples(c + 1);
-        const float* cert = cert0 + (c & 1) * TcItem<DM>::kCert;
+        if (t == 0) load_samples(n + 1);
+        const float* cert = cert0 + (n & 1) * TcItem<DM>::kCert;
         float* state = reinterpret_cast<float*>(p.tc_items) + (item - p.item_lo) * (long long)TcItem<DM>::kFloats + TcItem<DM>::kCert + t;
         // operand rows of one grid: the MMAs of the grid before are complete (every warp
         // has waited for its last tile); fenced for the tensor core's reads
@@ -589,8 +576,19 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
             o[3 * kTcTileM] = KeyTrack::low(tr.B3);
             tr.reset();
         };
-        operands(tA > 0 ? 0 : 1);
-        ok = arrive_and_issue(0, -1);
+        if (nT > 0) {
+            operands(tA > 0 ? 0 : 1);
+            ok = arrive_and_issue(0, -1);
+        } else {
+            // two grids of one point: no tile holds the warps together, and a warp that still
+            // waited for these samples when those after the next arrive would wait for the wrong
+            // phase
+            const uint32_t meet = smem_u32(&s_meet);
+            if (elect_one()) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(meet) : "memory");
+            __syncwarp();
+            ok = warp_wait(meet, meetph, budget);
+            meetph ^= 1u;
+        }
 #pragma unroll 1
         for (int i = 0; i < nT; ++i) {
             ok = warp_wait(accfull, accph, budget) && ok;
@@ -630,7 +628,6 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
         }
         if (!ok) break;
         if (nT > tA) put(1);
-        ++c;
     }
     if (!ok && (t & 31) == 0) {
         record_error(p.status, 4 /* QT_ETIMEOUT */, 26);
@@ -644,7 +641,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
     if (t == 0 && s_abort) {
         // after a timeout the copies still in flight land too (a slot that nothing is
         // loading runs its second out)
-        for (int q = 0; q < 2; ++q) mbar_wait_bounded(cfull + (uint32_t)(8 * ((c + q) & 1)), (uint32_t)(((c + q) >> 1) & 1), 1000000);
+        for (int q = 0; q < 2; ++q) mbar_wait_bounded(cfull + (uint32_t)(8 * ((n + q) & 1)), (uint32_t)(((n + q) >> 1) & 1), 1000000);
         for (int q = 0; q < RS; ++q) {
             mbar_wait_bounded(tfull + (uint32_t)(8 * slot), ph, 1000000);
             if (++slot == RS) {
