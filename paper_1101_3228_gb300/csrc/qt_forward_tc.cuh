@@ -267,6 +267,31 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, long lo
     return __all_sync(0xFFFFFFFFu, mbar_wait_bounded(bar, parity, budget));
 }
 
+// The warps of a CTA meet at an mbarrier (one arrival each), bounded.  By the arrival's own
+// token, not a parity that the loop around it would carry (0.5% of the screen; as a function of
+// its own 10%).
+__device__ __forceinline__ bool warps_meet(uint32_t bar, long long budget_us)
+{
+    bool ok = false;
+    __syncwarp();
+    if (elect_one()) {
+        unsigned long long state;
+        asm volatile("mbarrier.arrive.shared::cta.b64 %0, [%1];" : "=l"(state) : "r"(bar) : "memory");
+        const unsigned long long t0 = global_ns();
+        while (budget_us >= 0 && !ok) {
+            uint32_t done;
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tmbarrier.try_wait.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(done)
+                : "r"(bar), "l"(state)
+                : "memory");
+            ok = done != 0;
+            if (!ok && global_ns() - t0 > (unsigned long long)budget_us * 1000ull) break;
+        }
+    }
+    return __any_sync(0xFFFFFFFFu, ok);
+}
+
 __device__ __forceinline__ int layer_of(const ForwardParams& p, long long item)
 {
     int lo = 0, hi = p.n - 1;
@@ -508,7 +533,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
     }
 
     int slot = 0;                                      // ring slot and parity of the next tile
-    uint32_t ph = 0, accph = 0, meetph = 0;
+    uint32_t ph = 0, accph = 0;
     long long lend = 0;
     int tA = 0, nT = 0, expA = 0, expB = 0;
     long long n = 0;
@@ -583,11 +608,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
             // two grids of one point: no tile holds the warps together, and a warp that still
             // waited for these samples when those after the next arrive would wait for the wrong
             // phase
-            const uint32_t meet = smem_u32(&s_meet);
-            if (elect_one()) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(meet) : "memory");
-            __syncwarp();
-            ok = warp_wait(meet, meetph, budget);
-            meetph ^= 1u;
+            ok = warps_meet(smem_u32(&s_meet), budget);
         }
 #pragma unroll 1
         for (int i = 0; i < nT; ++i) {
