@@ -429,7 +429,10 @@ __device__ __forceinline__ int tc_layer(const ForwardParams& p, long long item)
     return p.tc_ipl > 0 ? (int)(item / p.tc_ipl) : layer_of(p, item);
 }
 
-template <int DM, int KT>
+// SPLIT: the work units are not items but the two grids of an item (unit 2 i + g), where items
+// are so few that the SMs hold all of them at once and an item's tiles, one round trip after
+// another, are the launch (one item of 2 x 4000 points at d = 4: 27 -> 15 us).
+template <int DM, int KT, bool SPLIT>
 __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const __grid_constant__ ForwardParams p)
 {
     constexpr int K = 16 * KT;
@@ -484,7 +487,14 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
     // ---- tile loads: a cursor over the tiles of this CTA's items, grid A's then grid B's
     // of each (a one-point grid needs none), kept by every thread; whichever warp issues
     // a tile's MMAs starts the copy that refills the slot before it
-    long long ld_item = p.item_lo + blockIdx.x, ld_end = 0;
+    constexpr int kSplit = SPLIT ? 1 : 0;
+    const long long unit_lo = p.item_lo << kSplit, unit_hi = p.item_hi << kSplit;
+    // tiles of a unit's grid A, and of both
+    auto tiles_of = [&](long long unit, const GridInfo& GA, const GridInfo& GB, int& a, int& all) {
+        a = GA.N > 1 && !(SPLIT && (unit & 1) != 0) ? GA.tc_tiles : 0;
+        all = a + (GB.N > 1 && !(SPLIT && (unit & 1) == 0) ? GB.tc_tiles : 0);
+    };
+    long long ld_item = unit_lo + blockIdx.x, ld_end = 0;
     int ld_a = 0, ld_b = 0;                            // tile numbers of the cursor's layer
     int ld_i = 0, ld_tA = 0, ld_nT = 0;
     // number of the next tile to load, -1 after the last one
@@ -492,17 +502,16 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
         while (ld_i == ld_nT) {                        // the next item with tiles
             if (ld_nT > 0) ld_item += G;
             ld_i = 0;
-            if (ld_item >= p.item_hi) {
+            if (ld_item >= unit_hi) {
                 ld_nT = 0;
                 return -1;
             }
-            if (ld_nT == 0 || ld_item >= ld_end) {
-                const LayerDesc& L = p.layers[tc_layer(p, ld_item)];
+            if (SPLIT || ld_nT == 0 || ld_item >= ld_end) {
+                const LayerDesc& L = p.layers[tc_layer(p, ld_item >> kSplit)];
                 const GridInfo& GA = p.grids[L.gridA];
                 const GridInfo& GB = p.grids[L.gridB];
                 ld_end = L.item_begin + L.items;
-                ld_tA = GA.N > 1 ? GA.tc_tiles : 0;
-                ld_nT = ld_tA + (GB.N > 1 ? GB.tc_tiles : 0);
+                tiles_of(ld_item, GA, GB, ld_tA, ld_nT);
                 ld_a = (int)GA.tc_toff;
                 ld_b = (int)GB.tc_toff - ld_tA;
                 if (ld_nT == 0) ld_item += G;
@@ -519,8 +528,8 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
                  reinterpret_cast<const unsigned char*>(p.tc_tiles) + (long long)src * kTileBytes, kTileBytes, bar);
     };
     auto load_samples = [&](long long n) {
-        const long long item = p.item_lo + blockIdx.x + n * G;
-        if (item >= p.item_hi) return;
+        const long long unit = unit_lo + blockIdx.x + n * G, item = unit >> kSplit;
+        if (unit >= unit_hi) return;
         const uint32_t bar = cfull + (uint32_t)(8 * (n & 1));
         mbar_arrive_expect_tx(bar, kCertBytes);
         bulk_g2s(cert_u + (uint32_t)(n & 1) * kCertBytes,
@@ -538,19 +547,18 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
     int tA = 0, nT = 0, expA = 0, expB = 0;
     long long n = 0;
     for (;; ++n) {
-        const long long item = p.item_lo + blockIdx.x + n * G;
-        if (item >= p.item_hi) break;
+        const long long unit = unit_lo + blockIdx.x + n * G, item = unit >> kSplit;
+        if (unit >= unit_hi) break;
         if (__shfl_sync(0xFFFFFFFFu, *(volatile int*)&s_abort, 0)) {
             ok = false;
             break;
         }
-        if (n == 0 || item >= lend) {
+        if (SPLIT || n == 0 || item >= lend) {
             const LayerDesc& L = p.layers[tc_layer(p, item)];
             const GridInfo& GA = p.grids[L.gridA];
             const GridInfo& GB = p.grids[L.gridB];
             lend = L.item_begin + L.items;
-            tA = GA.N > 1 ? GA.tc_tiles : 0;
-            nT = tA + (GB.N > 1 ? GB.tc_tiles : 0);
+            tiles_of(unit, GA, GB, tA, nT);
             expA = GA.tc_exp;
             expB = GB.tc_exp;
         }
@@ -876,10 +884,10 @@ __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(cons
 }
 
 // Screen of the items [p.item_lo, p.item_hi).
-template <int DM, int KT>
+template <int DM, int KT, bool SPLIT>
 cudaError_t launch_tc(const ForwardParams& p, int dyn, int num_sms, int* bps, cudaStream_t st)
 {
-    auto kern = forward_tc_kernel<DM, KT>;
+    auto kern = forward_tc_kernel<DM, KT, SPLIT>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e != cudaSuccess) return e;
     if (p.tc_slots < 2 || p.tc_slots > kTcMaxSlots) return cudaErrorInvalidValue;
@@ -887,7 +895,8 @@ cudaError_t launch_tc(const ForwardParams& p, int dyn, int num_sms, int* bps, cu
     // and tensor memory (128 of 512 columns each) are taken so that they fit
     *bps = kTcCtas;
     long long grid = (long long)kTcCtas * num_sms;
-    if (grid > p.item_hi - p.item_lo) grid = p.item_hi - p.item_lo;
+    const long long units = (p.item_hi - p.item_lo) * (SPLIT ? 2 : 1);
+    if (grid > units) grid = units;
     if (grid < 1) return cudaSuccess;
     kern<<<(unsigned)grid, kTcThreads, dyn, st>>>(p);
     return cudaGetLastError();

@@ -77,3 +77,27 @@ def test_uneven_layers_over_windows(ctx, B, chunk):
             for k in range(n):
                 np.testing.assert_array_equal(got[k], ref[k], err_msg=f"layer {k}")
             assert st.device_status == 0
+
+
+@pytest.mark.parametrize("d", [4, 10])
+@pytest.mark.parametrize("Ns", [[1, 300, 200], [1, 1, 129, 1], [40, 700, 1, 1, 260]])
+def test_few_items_take_their_grids_apart(ctx, B, d, Ns):
+    """Up to twice as many items as SMs are screened grid by grid; item counts either side of
+    the line, in one window and in windows of 7."""
+    n = len(Ns) - 1
+    rng = np.random.default_rng(2)
+    L = np.concatenate([np.zeros((1, d, d)), np.repeat((np.eye(d) - 0.3 * np.tri(d, k=-1))[None], n, 0)])
+    g = np.concatenate([rng.standard_normal((k, d)) for k in Ns])
+    line = torch.cuda.get_device_properties(0).multi_processor_count * 2
+    for items in (1, line // n, line // n + 1, line + 3):
+        M = items * 128 - 5
+        model = W.Model("few", d, n, np.array(Ns, dtype=np.int64), np.repeat(0.9 * np.eye(d)[None], n, 0), np.zeros((n, d)),
+                        np.repeat(0.4 * np.eye(d)[None], n, 0), np.zeros((n + 1, d)), L, np.arange(n + 1.0), 0.0,
+                        "basket_put", 1.0, None, M, 31, W.PREC_F32, "kmeans")
+        ref = oracle.transitions(model, g, M, model.seed, W.PREC_F32)
+        for chunk in (0, 7):
+            counts, st, _ = ctx.transitions(model, _dev(g), M, model.seed, B.options(tc_chunk_items=chunk))
+            got = B.split_counts(model.N, counts.cpu().numpy())
+            for k in range(n):
+                np.testing.assert_array_equal(got[k], ref[k], err_msg=f"items {items} layer {k}")
+            assert st.device_status == 0 and st.form_used == B.FORM_TC_RECHECK
