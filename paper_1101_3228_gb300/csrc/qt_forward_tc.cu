@@ -90,7 +90,7 @@ static cudaError_t launch_window(const ForwardParams& p, int dyn, int num_sms, i
     if (e != cudaSuccess) return e;
     auto certify = tc_certify_kernel<DM>;
     const int rec2 = 2 * TcItem<DM>::kFloats * 4;
-    e = cudaFuncSetAttribute(certify, cudaFuncAttributeMaxDynamicSharedMemorySize, rec2);
+    e = allow_dynamic_smem(certify, rec2);
     if (e != cudaSuccess) return e;
     const long long ctas = (long long)num_sms * kCertifyCtas;
     certify<<<(unsigned)(n < ctas ? n : ctas), kTcTileM, rec2, st>>>(p);

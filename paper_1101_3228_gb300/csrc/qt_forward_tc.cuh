@@ -888,7 +888,7 @@ template <int DM, int KT, bool SPLIT>
 cudaError_t launch_tc(const ForwardParams& p, int dyn, int num_sms, int* bps, cudaStream_t st)
 {
     auto kern = forward_tc_kernel<DM, KT, SPLIT>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    cudaError_t e = allow_dynamic_smem(kern, dyn);
     if (e != cudaSuccess) return e;
     if (p.tc_slots < 2 || p.tc_slots > kTcMaxSlots) return cudaErrorInvalidValue;
     // four CTAs share an SM: registers (launch bounds), shared memory (make_plan_full)

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "qt_internal.h"
+#include "qt_launch.h"
 #include "qt_sampler.cuh"
 
 namespace qt {
@@ -235,14 +236,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) backward_layer_kernel(const C*
     }
 }
 
-// Dynamic shared memory beside the lists: up to 16 KB need no leave (a call of its own, 2 us).
-template <typename F>
-static cudaError_t allow_dynamic(F kernel, size_t dyn)
-{
-    constexpr size_t kLists = sizeof(uint32_t) * kRowWarps * kRowSlots * 32;
-    if (kLists + dyn <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-}
+constexpr size_t kListBytes = sizeof(uint32_t) * kRowWarps * kRowSlots * 32;   // the lists of a CTA
 
 cudaError_t launch_backward_layer(const void* counts, int u32, long long coff, int Nk, int Nk1, const double* phik,
                                   const double* Vnext, double* Vk, int num_sms, cudaStream_t st)
@@ -255,12 +249,12 @@ cudaError_t launch_backward_layer(const void* counts, int u32, long long coff, i
     if (blocks > num_sms * per_sm) blocks = num_sms * per_sm;
     cudaError_t e;
     if (u32) {
-        e = allow_dynamic(backward_layer_kernel<uint32_t>, dyn);
+        e = allow_dynamic_smem(backward_layer_kernel<uint32_t>, dyn, kListBytes);
         if (e != cudaSuccess) return e;
         backward_layer_kernel<uint32_t><<<(unsigned)blocks, kRowWarps * 32, dyn, st>>>((const uint32_t*)counts, coff, Nk,
                                                                                       Nk1, staged, phik, Vnext, Vk);
     } else {
-        e = allow_dynamic(backward_layer_kernel<long long>, dyn);
+        e = allow_dynamic_smem(backward_layer_kernel<long long>, dyn, kListBytes);
         if (e != cudaSuccess) return e;
         backward_layer_kernel<long long><<<(unsigned)blocks, kRowWarps * 32, dyn, st>>>((const long long*)counts, coff,
                                                                                        Nk, Nk1, staged, phik, Vnext, Vk);
@@ -622,12 +616,12 @@ cudaError_t launch_swing_layer(const void* counts, int u32, long long coff, int 
     const dim3 grid((unsigned)chunks, (unsigned)by);
     cudaError_t e;
     if (u32) {
-        e = allow_dynamic(swing_layer_kernel<uint32_t>, dyn);
+        e = allow_dynamic_smem(swing_layer_kernel<uint32_t>, dyn, kListBytes);
         if (e != cudaSuccess) return e;
         swing_layer_kernel<uint32_t><<<grid, kRowWarps * 32, dyn, st>>>((const uint32_t*)counts, coff, Nk, Nk1, staged,
                                                                        vk, Pnext, Pk, n, k, Qmin, Qmax);
     } else {
-        e = allow_dynamic(swing_layer_kernel<long long>, dyn);
+        e = allow_dynamic_smem(swing_layer_kernel<long long>, dyn, kListBytes);
         if (e != cudaSuccess) return e;
         swing_layer_kernel<long long><<<grid, kRowWarps * 32, dyn, st>>>((const long long*)counts, coff, Nk, Nk1, staged,
                                                                         vk, Pnext, Pk, n, k, Qmin, Qmax);

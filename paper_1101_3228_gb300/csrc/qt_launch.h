@@ -7,6 +7,15 @@
 
 namespace qt {
 
+// Leave for `dyn` bytes of dynamic shared memory beside `fixed` bytes that the kernel declares:
+// up to 48 KB in all need none (the call takes a host microsecond of every launch).
+template <typename F>
+cudaError_t allow_dynamic_smem(F kernel, size_t dyn, size_t fixed = 1024)
+{
+    if (fixed + dyn <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+}
+
 bool forward_variant_exists(int form, int dm, int S, bool streamed);
 
 // Launches one persistent grid (SM count x resident CTAs per SM).
