@@ -748,7 +748,6 @@ qt_status make_plan_full(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
         P.tc_item_bytes = (size_t)tc_item_bytes(P.dm);
         // more than a fifth, so that a fifth CTA never waits for tensor memory
         P.grid_bytes = std::max((size_t)fixed + (size_t)P.tc_slots * tile_bytes, (ctx->smem_optin + 1024) / 5);
-        P.hist_bytes = 0;
         P.dyn_smem = P.grid_bytes;
         P.layers.resize(n);
         long long item = 0, coff = 0;
@@ -769,6 +768,9 @@ qt_status make_plan_full(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
             L.coff = coff;
             L.item_begin = item;
             L.items = (int)items_per_layer;
+            const long long ent = (long long)L.NA * L.NB;
+            L.hist_smem = !(o->flags & QT_FLAG_GLOBAL_HIST) && ent <= 1024 && M >= 64 * ent;
+            if (L.hist_smem) P.hist_bytes = std::max(P.hist_bytes, (size_t)round_up(ent * 4, 16));
             item += items_per_layer;
             coff += (long long)L.NA * L.NB;
         }

@@ -89,7 +89,7 @@ static cudaError_t launch_window(const ForwardParams& p, int dyn, int num_sms, i
                                               : launch_tc<DM, KT, false>(p, dyn, num_sms, bps, st);
     if (e != cudaSuccess) return e;
     auto certify = tc_certify_kernel<DM>;
-    const int rec2 = 2 * TcItem<DM>::kFloats * 4;
+    const int rec2 = 2 * TcItem<DM>::kFloats * 4 + p.smem_hist_entries * 4;
     e = allow_dynamic_smem(certify, rec2);
     if (e != cudaSuccess) return e;
     const long long ctas = (long long)num_sms * kCertifyCtas;

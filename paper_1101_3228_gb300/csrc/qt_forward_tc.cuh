@@ -724,7 +724,7 @@ template <int DM>
 __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(const __grid_constant__ ForwardParams p)
 {
     constexpr uint32_t kBytes = TcItem<DM>::kFloats * 4;
-    extern __shared__ __align__(128) float dsm_cf[];   // two records
+    extern __shared__ __align__(128) float dsm_cf[];   // two records, then the counts of a small layer
     __shared__ __align__(8) unsigned long long s_full[2];
     __shared__ GridInfo s_G[2];
     __shared__ float s_sigma[2][2];                    // 2^tc_exp and its inverse
@@ -751,14 +751,26 @@ __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(cons
     __syncthreads();
     int k = -1;
     LayerDesc L;
+    // counts of a layer of a few hundred entries are gathered in shared memory first: the L2
+    // reductions of all CTAs meet on them (1e6 given pairs on 16 x 16 points: 375 -> 330 us)
+    uint32_t* hist = reinterpret_cast<uint32_t*>(dsm_cf + 2 * TcItem<DM>::kFloats);
+    int live = 0;                                      // entries gathered there, 0: none
+    auto flush = [&]() {
+        for (int e = t; e < live; e += kTcTileM)
+            if (hist[e]) count_add(p.counts, p.counts_u32, L.coff + e, hist[e]);
+    };
     const float sqrt_d = sqrtf((float)d);
     for (long long n = 0;; ++n) {
         const long long item = p.item_lo + blockIdx.x + n * (long long)gridDim.x;
         if (item >= p.item_hi) break;
         const int ki = tc_layer(p, item);
         if (ki != k) {
+            flush();                                   // (every warp is done with the item before)
             k = ki;
             L = p.layers[k];
+            live = L.hist_smem ? L.NA * L.NB : 0;
+            __syncthreads();
+            for (int e = t; e < live; e += kTcTileM) hist[e] = 0;
             for (int e = t; e < (int)(sizeof(GridInfo) / 4); e += kTcTileM) {
                 reinterpret_cast<int*>(&s_G[0])[e] = reinterpret_cast<const int*>(p.grids + L.gridA)[e];
                 reinterpret_cast<int*>(&s_G[1])[e] = reinterpret_cast<const int*>(p.grids + L.gridB)[e];
@@ -857,7 +869,8 @@ __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(cons
         if (valid && ((unsigned)ci >= (unsigned)L.NA || (unsigned)cj >= (unsigned)L.NB)) {
             record_error(p.status, 6 /* QT_EDEVICE */, 13);
         } else if (valid) {
-            count_add(p.counts, p.counts_u32, L.coff + (long long)ci * L.NB + cj, 1u);
+            if (live) atomicAdd(&hist[ci * L.NB + cj], 1u);
+            else count_add(p.counts, p.counts_u32, L.coff + (long long)ci * L.NB + cj, 1u);
             if (p.cellsA) {
                 p.cellsA[ms] = ci;
                 p.cellsB[ms] = cj;
@@ -881,6 +894,7 @@ __global__ void __launch_bounds__(kTcTileM, kCertifyCtas) tc_certify_kernel(cons
         __syncthreads();                               // every warp is done with this record (and s_G)
         if (t == 0) load(n + 2);
     }
+    flush();
 }
 
 // Screen of the items [p.item_lo, p.item_hi).

@@ -101,3 +101,25 @@ def test_few_items_take_their_grids_apart(ctx, B, d, Ns):
             for k in range(n):
                 np.testing.assert_array_equal(got[k], ref[k], err_msg=f"items {items} layer {k}")
             assert st.device_status == 0 and st.form_used == B.FORM_TC_RECHECK
+
+
+@pytest.mark.parametrize("Ns", [[1, 16, 16, 64, 17, 1, 40], [30, 34, 31, 33, 1024, 1, 1024]])
+@pytest.mark.parametrize("chunk", [0, 40])
+def test_small_layers_count_in_shared_memory(ctx, B, Ns, chunk):
+    """Layers of up to 1024 entries (and one more) between larger ones, with many samples."""
+    d, n, M = 4, len(Ns) - 1, 70001
+    rng = np.random.default_rng(2)
+    L = np.concatenate([np.zeros((1, d, d)), np.repeat((np.eye(d) - 0.3 * np.tri(d, k=-1))[None], n, 0)])
+    g = np.concatenate([rng.standard_normal((k, d)) for k in Ns])
+    model = W.Model("hist", d, n, np.array(Ns, dtype=np.int64), np.repeat(0.9 * np.eye(d)[None], n, 0), np.zeros((n, d)),
+                    np.repeat(0.4 * np.eye(d)[None], n, 0), np.zeros((n + 1, d)), L, np.arange(n + 1.0), 0.0,
+                    "basket_put", 1.0, None, M, 31, W.PREC_F32, "kmeans")
+    ref = oracle.transitions(model, g, M, model.seed, W.PREC_F32)
+    for ct in (B.COUNTS_I64, B.COUNTS_U32):
+        for flags in (0, B.FLAG_GLOBAL_HIST):
+            counts, st, _ = ctx.transitions(model, _dev(g), M, model.seed,
+                                            B.options(counts_type=ct, flags=flags, tc_chunk_items=chunk))
+            got = B.split_counts(model.N, counts.cpu().numpy())
+            for k in range(n):
+                np.testing.assert_array_equal(got[k], ref[k], err_msg=f"layer {k}")
+            assert st.device_status == 0
