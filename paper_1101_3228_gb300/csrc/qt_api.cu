@@ -1836,7 +1836,7 @@ extern "C" qt_status qt_build_grids(qt_ctx* ctx, const qt_model* model, int32_t 
                 const size_t z = (size_t)draws(end->first) * d;
                 if (nj > 0 && (zf + z) * sizeof(float) > ((size_t)1 << 30)) break;
                 zf += z;
-                sw += (size_t)end->first * (d + 1);
+                sw += (size_t)end->first * (d + 1) * km_copies(end->first);
             }
             void *dZ, *dsum;
             if ((s = dev_get(ctx, "km_Z", sizeof(float) * zf, &dZ))) return s;
@@ -1846,9 +1846,9 @@ extern "C" qt_status qt_build_grids(qt_ctx* ctx, const qt_model* model, int32_t 
                 const long long Nk = it->first;
                 jobs.j[i] = KmJob{(float*)dZ + zf, (float*)dC + it->second, (unsigned long long*)dsum + sw,
                                   seed ^ (0x9E3779B97F4A7C15ull * (unsigned long long)Nk), draws(Nk), (int)Nk,
-                                  (int)((Nk + 15) / 16 * 16)};
+                                  (int)((Nk + 15) / 16 * 16), km_copies(Nk), 0};
                 zf += (size_t)draws(Nk) * d;
-                sw += (size_t)Nk * (d + 1);
+                sw += (size_t)Nk * (d + 1) * km_copies(Nk);
             }
             QT_CUDA(launch_kmeans(jobs, nj, d, its, ctx->num_sms, st));
         }

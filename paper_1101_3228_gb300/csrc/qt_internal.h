@@ -186,11 +186,16 @@ struct ForwardParams {
 struct KmJob {
     float* Z;                      // training draws [d][S]
     float* C;                      // centres, pairs [Npad/2][dim class][2]
-    unsigned long long* sums;      // [N][d + 1]: fixed-point sums, count
+    unsigned long long* sums;      // [copies][N][d + 1]: fixed-point sums, count
     unsigned long long seed;
     long long S;
     int32_t N, Npad;
+    int32_t copies, pad;           // sums of CTAs taken modulo `copies`
 };
+// Copies of the sums: few centres have many draws each, whose additions would wait for one
+// another (1e5 draws, 10 centres, d = 8: 400 us an iteration, 250 before each launch served all
+// draws of four CTAs an SM at once)
+__host__ __device__ constexpr int km_copies(long long N) { return N <= 64 ? 16 : 1; }
 constexpr int kKmJobs = 32;        // grid sizes per launch
 struct KmJobs {
     KmJob j[kKmJobs];

@@ -92,7 +92,8 @@ __global__ void __launch_bounds__(256) km_draw_kernel(const __grid_constant__ Km
         for (int l = 0; l < kDMax; ++l)
             if (l < dm) c[2 * l] = t < J.N ? (l < d ? g[l] : 0.0f) : __int_as_float(0x7F800000);
         if (t < J.N)
-            for (int l = 0; l <= d; ++l) J.sums[t * (d + 1) + l] = 0ull;
+            for (int c = 0; c < J.copies; ++c)
+                for (int l = 0; l <= d; ++l) J.sums[((long long)c * J.N + t) * (d + 1) + l] = 0ull;
     }
 }
 
@@ -152,6 +153,8 @@ __global__ void __launch_bounds__(kKmBlock) km_assign_kernel(const __grid_consta
                 }
         }
     }
+    unsigned long long* sums = J.sums;
+    if (J.copies > 1) sums += (long long)(blockIdx.x % (unsigned)J.copies) * J.N * (d + 1);
     // the first centre of the best group that has its minimum: the same distances again
     const float* base = groups <= kTile ? s_c : J.C;
 #pragma unroll
@@ -168,7 +171,7 @@ __global__ void __launch_bounds__(kKmBlock) km_assign_kernel(const __grid_consta
             if (a == best[r]) idx = 2 * q;
         }
         if (t0 + r * kKmBlock < J.S) {
-            unsigned long long* s = J.sums + (long long)(bg[r] * 16 + idx) * (d + 1);
+            unsigned long long* s = sums + (long long)(bg[r] * 16 + idx) * (d + 1);
 #pragma unroll
             for (int l = 0; l < DM; ++l)
                 if (l < d) {
@@ -188,14 +191,19 @@ __global__ void __launch_bounds__(128) km_update_kernel(const __grid_constant__ 
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= J.N) return;
     unsigned long long* s = J.sums + (long long)j * (d + 1);
-    const unsigned long long c = s[d];
+    const long long copy = (long long)J.N * (d + 1);
+    // of all copies, left at zero
+    auto total = [&](int l) {
+        unsigned long long v = 0;
+#pragma unroll 4
+        for (int q = 0; q < J.copies; ++q) v += s[q * copy + l];
+        for (int q = 0; q < J.copies; ++q) s[q * copy + l] = 0ull;
+        return v;
+    };
+    const unsigned long long c = total(d);
     if (c == 0) return;
     float* ctr = J.C + (long long)(j >> 1) * 2 * dm + (j & 1);
-    for (int l = 0; l < d; ++l) {
-        ctr[2 * l] = (float)(((double)(long long)s[l] / 68719476736.0) / (double)c);
-        s[l] = 0ull;
-    }
-    s[d] = 0ull;
+    for (int l = 0; l < d; ++l) ctr[2 * l] = (float)(((double)(long long)total(l) / 68719476736.0) / (double)c);
 }
 
 template <int DM>
