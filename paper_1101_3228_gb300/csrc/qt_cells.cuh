@@ -199,10 +199,12 @@ __device__ __forceinline__ int cell_search(const CellGrid& G, const unsigned cha
     uint32_t b = cell_bin(a[0], axes.x, axes.z);
     bool in = b < (uint32_t)G.nb0;
     if constexpr (DM == 1) {
-        // the last bins serve what lies up to 2^20 bins beyond them
-        const float v = __fmaf_rn(a[0], axes.x, axes.z);
-        b = (uint32_t)__float_as_int(fminf(fmaxf(v, 8388608.0f), 8388607.0f + (float)G.nb0)) - 0x4B000000u;
-        in = fabsf(v - 8388608.0f) <= 1048576.0f;
+        if (!in) {
+            // beside the table: the first and last bins go on for 2^20 more
+            const float v = __fmaf_rn(a[0], axes.x, axes.z) - 8388608.0f;
+            in = fabsf(v) <= 1048576.0f;
+            b = v > 0.0f ? (uint32_t)G.nb0 - 1u : 0u;
+        }
     } else {
         uint32_t b1 = cell_bin(a[1], axes.y, axes.w);
         in = in && b1 < (uint32_t)G.nb1;
@@ -251,8 +253,10 @@ __device__ __forceinline__ int cell_search(const CellGrid& G, const unsigned cha
 // all, so the points in doubt are put into an entry first and evaluated side by side).  A
 // sample without a finite distance has no cell: the index is out of range, and the callers
 // refuse it, as in the other forms.
-template <int DM>
-__device__ __noinline__ int cell_exact(const CellGrid& G, const float* __restrict__ rec, const float (&a)[DM], float f,
+// a: the sample z in FP32, centred.  KNOWN: an entry that stands for the whole grid has the
+// smallest distance from it in its low word.
+template <int DM, bool KNOWN>
+__device__ __noinline__ int cell_exact(const CellGrid& G, const float* __restrict__ rec, const float (&a)[DM],
                                        const double (&z)[DM], uint64_t e, const uint16_t* __restrict__ pool,
                                        const double* __restrict__ g64)
 {
@@ -262,13 +266,13 @@ __device__ __noinline__ int cell_exact(const CellGrid& G, const float* __restric
         return kind == kCellScan ? q : (kind == kCellPool ? (int)pool[(uint32_t)e + q] : (int)((e >> (10 * q)) & 1023u));
     };
     float b = __int_as_float(0x7F800000);
-    if (kind == kCellScan) {
+    if (KNOWN && kind == kCellScan) {
         b = __uint_as_float((uint32_t)e);
     } else {
 #pragma unroll 4
         for (int q = 0; q < cnt; ++q) b = fminf(b, cell_dist(rec, at(q), a));
     }
-    const float lim = b + cell_doubt<DM>(G, a, f).window(b);
+    const float lim = b + cell_doubt<DM>(G, a, 0.0f).window(b);   // rounding alone: a is z's own
     uint64_t in_doubt = 0;
     int n = 0;
     auto look = [&](int j) {

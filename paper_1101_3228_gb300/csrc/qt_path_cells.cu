@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) path_cells_kernel(const __gri
 #pragma unroll
                         for (int l = 0; l < DM; ++l) z[l] = (double)x[s][l];
                         atomicAdd(&p.status->rechecks, 1ull);
-                        j = cell_exact<DM>(s_G, cell_records(s_G, sm), a, 1.0f, z, e, p.cell_pool, p.g64 + G.goff * DM);
+                        j = cell_exact<DM, true>(s_G, cell_records(s_G, sm), a, z, e, p.cell_pool, p.g64 + G.goff * DM);
                     }
                 }
                 if ((unsigned)j >= (unsigned)N) {
