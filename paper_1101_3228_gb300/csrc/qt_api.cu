@@ -137,10 +137,12 @@ struct DeviceGuard {
 };
 
 // Host-side fault injection for the allocation-failure tests: QT_FAULT=alloc
-// makes the next workspace allocation fail as if the device were out of memory.
-bool injected_alloc_failure()
+// makes the next workspace allocation fail as if the device were out of memory,
+// QT_FAULT=alloc_above:B every one of more than B bytes.
+bool injected_alloc_failure(size_t bytes)
 {
     const char* f = getenv("QT_FAULT");
+    if (f && strncmp(f, "alloc_above:", 12) == 0) return bytes > strtoull(f + 12, nullptr, 10);
     return f && strcmp(f, "alloc") == 0;
 }
 
@@ -165,7 +167,7 @@ qt_status dev_get(qt_ctx* ctx, const char* name, size_t bytes, void** out)
 {
     DevBuf& b = ctx->dev[name];
     if (b.bytes < bytes) {
-        if (injected_alloc_failure()) return fail(ctx, QT_ENOMEM, "workspace '%s': injected allocation failure", name);
+        if (injected_alloc_failure(bytes)) return fail(ctx, QT_ENOMEM, "workspace '%s': injected allocation failure", name);
         if (b.p) cudaFree(b.p);
         b.p = nullptr;
         b.bytes = 0;
@@ -1101,6 +1103,7 @@ qt_status run_plan(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long M, uns
         key_append(key, &P.streamed, sizeof P.streamed);
         key_append(key, &P.seg_records, sizeof P.seg_records);
         key_append(key, &P.euler, sizeof P.euler);
+        key_append(key, &P.tc_chunk_items, sizeof P.tc_chunk_items);
         key_append(key, &M, sizeof M);
         key_append(key, &seed, sizeof seed);
         key_append(key, &source, sizeof source);
@@ -1283,7 +1286,25 @@ qt_status forward_common(qt_ctx* ctx, int d, int n, const int64_t* Ns, const dou
                                              : QT_FORM_F32_RECHECK;
     // one layer at a time (fused backward) launches directly: each layer would be a new graph
     const bool use_graph = !(o->flags & QT_FLAG_NO_GRAPH) && !capturing && only_layer < 0;
-    if ((s = run_plan(ctx, P, io, M, seed, o, source, params_d_host, st, use_graph, ""))) return s;
+    const std::string err = ctx->err;
+    s = run_plan(ctx, P, io, M, seed, o, source, params_d_host, st, use_graph, "");
+    // no memory for the windows of the tensor-core form: smaller ones
+    while (s == QT_ENOMEM && P.form == kTcRecheck && P.tc_chunk_items > kTcCtas * ctx->num_sms) {
+        P.tc_chunk_items = std::max<long long>(kTcCtas * ctx->num_sms, P.tc_chunk_items / 4);
+        s = run_plan(ctx, P, io, M, seed, o, source, params_d_host, st, use_graph, "");
+    }
+    // none for the tables of the located search: brute force
+    if (s == QT_ENOMEM && (P.form == kCells || P.form == kPathCells) && !capturing) {
+        qt_options brute = *o;
+        brute.form = QT_FORM_F32_RECHECK;
+        if ((s = forward_common(ctx, d, n, Ns, mus, params_d_host, M, seed, &brute, source, io, stats, st, only_layer, algo,
+                                euler)))
+            return s;
+        ctx->err = err;
+        return QT_OK;
+    }
+    if (s) return s;
+    ctx->err = err;
     if (stats) return read_status(ctx, st, stats, (long long)n * M, (algo == 2 ? n + 1ll : 2ll * n) * M);
     return QT_OK;
 }
@@ -1827,6 +1848,8 @@ extern "C" qt_status qt_build_grids(qt_ctx* ctx, const qt_model* model, int32_t 
         if ((s = dev_get(ctx, "km_C", sizeof(float) * (size_t)centres, &dC))) return s;
         // as many sizes in each launch as keep their draws within 1 GiB (one at least),
         // the largest first
+        const std::string err = ctx->err;
+        size_t most = (size_t)1 << 30;
         for (auto it = at.rbegin(); it != at.rend();) {
             KmJobs jobs;
             int nj = 0;
@@ -1834,13 +1857,18 @@ extern "C" qt_status qt_build_grids(qt_ctx* ctx, const qt_model* model, int32_t 
             auto end = it;
             for (; end != at.rend() && nj < kKmJobs; ++end, ++nj) {
                 const size_t z = (size_t)draws(end->first) * d;
-                if (nj > 0 && (zf + z) * sizeof(float) > ((size_t)1 << 30)) break;
+                if (nj > 0 && (zf + z) * sizeof(float) > most) break;
                 zf += z;
                 sw += (size_t)end->first * (d + 1) * km_copies(end->first);
             }
             void *dZ, *dsum;
-            if ((s = dev_get(ctx, "km_Z", sizeof(float) * zf, &dZ))) return s;
-            if ((s = dev_get(ctx, "km_sum", sizeof(unsigned long long) * sw, &dsum))) return s;
+            if ((s = dev_get(ctx, "km_Z", sizeof(float) * zf, &dZ)) ||
+                (s = dev_get(ctx, "km_sum", sizeof(unsigned long long) * sw, &dsum))) {
+                if (s != QT_ENOMEM || nj == 1) return s;
+                most = 0;                              // no memory for several sizes at once: one by one
+                ctx->err = err;
+                continue;
+            }
             zf = sw = 0;
             for (int i = 0; i < nj; ++i, ++it) {
                 const long long Nk = it->first;
