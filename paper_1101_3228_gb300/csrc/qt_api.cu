@@ -986,6 +986,7 @@ qt_status enqueue_forward(qt_ctx* ctx, const Plan& P, const FwdIO& io, long long
         // draw, screen and certificate, window by window
         fp.tc_items = (unsigned char*)dtcitems;
         fp.tc_ipl = P.only_layer < 0 ? P.layers[0].items : 0;
+        for (const LayerDesc& L : P.layers) fp.tc_one_point |= L.items > 0 && L.NA == 1 && L.NB == 1;
         for (long long lo = 0; lo < P.total_items; lo += P.tc_chunk_items) {
             fp.item_lo = lo;
             fp.item_hi = std::min(P.total_items, lo + P.tc_chunk_items);

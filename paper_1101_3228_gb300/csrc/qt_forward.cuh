@@ -632,16 +632,15 @@ __device__ __noinline__ int warp_window_nn(const float (&xs)[DM], float A, const
     // exact distances on the window only; on every record where the scores bound nothing (a
     // sample so far out that they overflow).  A sample with no finite distance has no cell:
     // the index returned is out of range, and the callers refuse it
-    constexpr int kNone = 0x7FFFFFFF;
     if (i1 >= N || !(lim < __int_as_float(0x7F800000))) lim = __int_as_float(0x7F800000);
     double best = __longlong_as_double(0x7FF0000000000000LL);
-    int bi = kNone;
+    int bi = 0x7FFFFFFF;
     double zz[DM];
 #pragma unroll
     for (int l = 0; l < DM; ++l) zz[l] = __shfl_sync(0xFFFFFFFFu, z[l], src);
     auto exact = [&](int j) {
         const double dj = dist64<DM>(zz, g64 + (long long)j * d, d);
-        if (dj < best || (dj == best && j < bi && bi != kNone)) {
+        if (dj < best || (dj == best && j < bi)) {
             best = dj;
             bi = j;
         }
@@ -669,7 +668,7 @@ __device__ __noinline__ int warp_window_nn(const float (&xs)[DM], float A, const
         }
     }
     (void)Npad;
-    return bi;
+    return best < __longlong_as_double(0x7FF0000000000000LL) ? bi : 0x7FFFFFFF;
 }
 
 // ------------------------------------------------------------------ the kernel

@@ -84,9 +84,10 @@ static cudaError_t launch_window(const ForwardParams& p, int dyn, int num_sms, i
     tc_draw_kernel<DM><<<(unsigned)n, kTcTileM, 0, st>>>(p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // an item's grids apart while all of them are resident at once
-    e = 2 * n <= (long long)kTcCtas * num_sms ? launch_tc<DM, KT, true>(p, dyn, num_sms, bps, st)
-                                              : launch_tc<DM, KT, false>(p, dyn, num_sms, bps, st);
+    // an item's grids apart while all of them are resident at once, and with layers of one point
+    e = p.tc_one_point || 2 * n <= (long long)kTcCtas * num_sms
+            ? launch_tc<DM, KT, true>(p, dyn, num_sms, bps, st)
+            : launch_tc<DM, KT, false>(p, dyn, num_sms, bps, st);
     if (e != cudaSuccess) return e;
     auto certify = tc_certify_kernel<DM>;
     const int rec2 = 2 * TcItem<DM>::kFloats * 4 + p.smem_hist_entries * 4;

@@ -35,10 +35,10 @@
 // tensor memory (193 scores per SM and cycle: 85 cycles per 128 x 128 tile) and the
 // issue slots of the chunk tracking (about 50 half-rate instructions per thread and
 // tile); what is left is the round trip of the 512 columns of tensor memory (issue,
-// MMA, arrival, read, hand-over: about 1700 cycles for the SM's four tiles, 420 a tile).
+// MMA, arrival, read, hand-over: 1350 cycles for the SM's four tiles at d = 8, 337 a tile).
 // 8-d tree, 12 dates of 4000 points, 2e6 paths: 21.3 -> 19.3 ms; 4-d, 50 dates of
-// 2000 points on average, 1e6 paths: 19.1 -> 13.8 ms (draw 1.35, screen 9.7, certify
-// 2.9 ms of it); 10-d, 6 dates of 8000 points, 1e6 paths: 9.7 -> 8.7 ms; 3-d given
+// 200 to 2000 points, 1e6 paths: 19.1 -> 13.7 ms (draw 1.35, screen 9.7, certify
+// 2.6 ms of it); 10-d, 6 dates of 8000 points, 1e6 paths: 9.7 -> 8.7 ms; 3-d given
 // samples: 0.55 -> 0.38 ms.
 // The hand-over costs 2 (8 DM + 40) bytes of traffic per pair and reads of
 // them, 0.3 KB at d = 8, and buys kernels that each fit their registers: one kernel
@@ -268,8 +268,8 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, long lo
 }
 
 // The warps of a CTA meet at an mbarrier (one arrival each), bounded.  By the arrival's own
-// token, not a parity that the loop around it would carry (0.5% of the screen; as a function of
-// its own 10%).
+// token, not a parity that the loop around it would carry (as a function of its own it costs
+// the screen 10%).
 __device__ __forceinline__ bool warps_meet(uint32_t bar, long long budget_us)
 {
     bool ok = false;
@@ -431,7 +431,9 @@ __device__ __forceinline__ int tc_layer(const ForwardParams& p, long long item)
 
 // SPLIT: the work units are not items but the two grids of an item (unit 2 i + g), where items
 // are so few that the SMs hold all of them at once and an item's tiles, one round trip after
-// another, are the launch (one item of 2 x 4000 points at d = 4: 27 -> 15 us).
+// another, are the launch (one item of 2 x 4000 points at d = 4: 27 -> 15 us).  Units without a
+// tile (grids of one point) make the warps meet, which costs the screen's loop 0.3% and
+// is left out of the other variant: that one takes no layers of one point by one.
 template <int DM, int KT, bool SPLIT>
 __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const __grid_constant__ ForwardParams p)
 {
@@ -612,10 +614,9 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas) forward_tc_kernel(const _
         if (nT > 0) {
             operands(tA > 0 ? 0 : 1);
             ok = arrive_and_issue(0, -1);
-        } else {
-            // two grids of one point: no tile holds the warps together, and a warp that still
-            // waited for these samples when those after the next arrive would wait for the wrong
-            // phase
+        } else if constexpr (SPLIT) {
+            // no tile holds the warps together, and a warp that still waited for these samples
+            // when those after the next arrive would wait for the wrong phase
             ok = warps_meet(smem_u32(&s_meet), budget);
         }
 #pragma unroll 1

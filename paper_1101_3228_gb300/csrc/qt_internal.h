@@ -156,6 +156,7 @@ struct ForwardParams {
     int32_t tc_k;                  // 16 or 32
     int32_t tc_slots;              // ring slots of operand tiles in shared memory
     long long item_lo, item_hi;    // tensor-core form: work items [item_lo, item_hi) of this launch
+    int32_t tc_one_point;          // tensor-core form: some layer has one point by one
     long long tc_ipl;              // tensor-core form: work items of every layer (0: one layer has them all)
     unsigned char* tc_items;       // tensor-core form: records of the window's items
     // located search (d <= 2)
