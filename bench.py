@@ -60,7 +60,7 @@ def parse():
                     help="count histogram: library choice, shared-memory privatised, or L2 reductions")
     ap.add_argument("--spt", type=int, default=0, help="samples per thread (0 = library choice)")
     ap.add_argument("--tc-draw", type=int, default=0, choices=[0, 1, 2],
-                    help="tensor-core form's sample-draw layout: 0 autotuned, 1 draw pass, 2 in the screen kernel")
+                    help="tensor-core form: qt_options.tc_draw (every value runs the draw pass before each screen)")
     ap.add_argument("--router-samples", type=int, default=10**7, help="labelled pairs for the router form")
     return ap.parse_args()
 
@@ -361,7 +361,7 @@ def extra_workloads(ctx, B, dev, stream, flush, peaks, n_sm):
         if st.form_used == B.FORM_ROUTER_CERT:
             r["candidates_per_search"] = st.candidates / (2 * units)
         if st.form_used == B.FORM_TC_RECHECK and not pathwise:
-            r["tc_draw"] = {1: "draw pass", 2: "in the screen kernel"}.get(st.tc_draw)
+            r["tc_draw"] = {1: "draw pass"}.get(st.tc_draw)
             r["roofline"] = tensor_roofline(model, units, kmean, peaks)
         else:
             r["roofline"] = alu_roofline(model, units, kmean, peaks, n_sm, pathwise, o.form == B.FORM_AUTO)
@@ -511,8 +511,8 @@ def main():
            "h2d_bytes_per_step": int(gh.nbytes + phi.nbytes), "d2h_bytes_per_step": 8,
            "ms_per_step": statistics.mean(e2e_ms), "price": price}
 
-    # roofline of the dominant kernel: the forward region (screen launches and, with
-    # the draw-pass layout, the draw passes), timed by the library's CUDA events on
+    # roofline of the dominant kernel: the forward region (the screen, and in the
+    # tensor-core form its draw and certificate), timed by the library's CUDA events on
     # the launching stream at every timed step
     peaks = json.load(open(MEASURED)) if os.path.exists(MEASURED) else {}
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
@@ -521,7 +521,7 @@ def main():
         roofline = tensor_roofline(model, units, kmean, peaks)
     else:
         roofline = alu_roofline(model, units, kmean, peaks, n_sm)
-    layout = {1: "draw pass", 2: "in the screen kernel"}.get(st.tc_draw)
+    layout = {1: "draw pass"}.get(st.tc_draw)
     traffic = None
     if os.path.exists(TRAFFIC):
         # DRAM bytes of one ncu capture of this kernel, kept only while the sources,

@@ -75,7 +75,8 @@ typedef int32_t qt_status;
                                  3 <= d <= 10, F32_RECHECK otherwise; for d <= 2 and grids
                                  of at most 1024 points the FP32 screen runs only over the
                                  few points that a table of the grid leaves (located search,
-                                 Algorithms II and III and given samples)                  */
+                                 Algorithms II and III and given samples), where the layers
+                                 have pairs enough to pay for the tables                   */
 #define QT_FORM_PLAIN_F64 1   /* brute force, exact FP64 distances                       */
 #define QT_FORM_F32_RECHECK 2 /* FP32 brute-force screen, FP64 recheck of near ties      */
 #define QT_FORM_TC_RECHECK 3  /* tensor-core (tcgen05) screen, FP64 recheck              */
@@ -134,7 +135,8 @@ typedef struct {
     const void* router;    /* qt_router* for QT_FORM_ROUTER_CERT, else NULL                */
     int32_t tile_samples_per_thread; /* 0 = autotuned                                       */
     int32_t tc_chunk_items; /* tensor-core form: most work items (128 samples each) per window
-                              of launches; 0 = as many as 1 GiB of their records holds     */
+                              of launches; 0 = as many as 1 GiB of their records holds, or
+                              as the device's free memory does                             */
     int32_t tc_draw;       /* tensor-core form: named two layouts of the sample draw (1, 2;
                               0 = autotuned).  Every value runs the one layout there is: a
                               draw pass before each screen                                */

@@ -36,9 +36,10 @@
 //
 // Why bins: brute force spends 2 d flops on each of N_k + N_{k+1} candidates (1000
 // on the 2-factor workload), and only the few points around a sample can be its
-// cell.  About 20 bins per point (104 x 104 at most: two tables fit one CTA's
-// shared memory) leave 2.6 candidates per search on average and 4 for the slowest
-// lane of a warp on the 2-factor grids; 64 x 64 bins leave 4.3 and 6.6.
+// cell.  About 20 bins per point (104 x 104 at most, split by the grid's extents: two
+// tables fit one CTA's shared memory) leave 3.2 candidates per search on average and 5.5
+// for the slowest lane of a warp (samples of N(0, I) on a quantizer of 500 points, counted on
+// the CPU); 64 x 64 bins leave 6.1 and 12.6.
 #pragma once
 #include "qt_forward.cuh"
 

@@ -42,6 +42,9 @@ __device__ __forceinline__ float warp_max(float v)
 //            + 8 u slack.
 // Twice that is allowed for.  (A bound of 2^-18 S^2 for every bin, S the size of the box,
 // kept 16 points in every bin of a 1-d grid of 1000.)
+//
+// What bounds it: latency with few grids (a warp has one patch: 30 us for two grids of 1000
+// points, 9 for five of 64), issue slots with many (366 grids of 500 points: 275 us, 66%).
 template <int DM>
 __global__ void __launch_bounds__(kBuildThreads) build_cells_kernel(const __grid_constant__ ForwardParams p)
 {
@@ -453,8 +456,8 @@ static __device__ __noinline__ int cell_recheck(const ForwardParams& p, const fl
 // qt_cells.cuh), 2: given samples.  A work item is (layer, blockDim.x samples), one
 // sample per thread; a CTA takes a contiguous run of items, so that it loads the
 // two tables of a layer (170 KB at most) once or twice per launch instead of once
-// per item and layer.  What bounds it: issue slots (87% busy, 640 instructions a
-// pair at d = 2, most of them the draw).  2-factor workload, 10^9 pairs: 19.5 ms,
+// per item and layer.  What bounds it: issue slots (83% busy, 580 instructions a
+// pair at d = 2, most of them the draw).  2-factor workload, 10^9 pairs: 17.7 ms,
 // against 142.9 ms for brute force over 1000 candidates a pair.
 template <int DM, int MODE>
 __global__ void __launch_bounds__(kCellThreads, 1) forward_cells_kernel(const __grid_constant__ ForwardParams p)

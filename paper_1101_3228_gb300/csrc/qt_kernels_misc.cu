@@ -1,6 +1,6 @@
 // qt_kernels_misc.cu -- small kernels around the forward step: preparation of
-// the screened grid records, the backward induction of Sec. 2, the root price,
-// and the sample-Lloyd (k-means) steps of the grid builder.
+// the screened grid records, the backward induction of Sec. 2, the swing recursion
+// and the root price.
 #include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
