@@ -94,7 +94,7 @@ struct qt_ctx {
     int last_tc_draw = 0;              // sample-draw layout of the last tensor-core step
     void* status_buf = nullptr;   // status block of the last forward call
     void* tree_status = nullptr;  // that of the one-launch backward induction after it, if any
-    DevStatus* status_host = nullptr;   // pinned: both as read
+    DevStatus* status_host = nullptr;   // pinned: both as read, and a price
 };
 
 namespace {
@@ -281,7 +281,7 @@ extern "C" qt_status qt_create(qt_ctx** out, int32_t device)
         cudaEventCreateWithFlags(&ctx->ev_tree, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_up_tree[0], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&ctx->ev_up_tree[1], cudaEventDisableTiming) != cudaSuccess ||
-        cudaMallocHost(&ctx->status_host, 2 * sizeof(DevStatus)) != cudaSuccess ||
+        cudaMallocHost(&ctx->status_host, 2 * sizeof(DevStatus) + sizeof(double)) != cudaSuccess ||
         cudaEventCreate(&ctx->ev_k0) != cudaSuccess || cudaEventCreate(&ctx->ev_k1) != cudaSuccess) {
         delete ctx;
         return QT_ECUDA;
@@ -1487,9 +1487,10 @@ extern "C" qt_status qt_transitions_workspace(const qt_model* model, const qt_op
 // ------------------------------------------------------------------ backward induction and price
 
 namespace {
-// qt_backward with the bound of the waits inside its kernels (microseconds, 0 = 10 s)
+// qt_backward with the bound of the waits inside its kernels (microseconds, 0 = 10 s) and the
+// status block they record in (NULL: one of its own)
 qt_status backward_impl(qt_ctx* ctx, int32_t n, const int64_t* N, const void* counts, int32_t counts_type,
-                        const double* phi, double* V, long long spin_budget, void* stream)
+                        const double* phi, double* V, long long spin_budget, DevStatus* status, void* stream)
 {
     if (n < 1 || !N || !counts || !phi || !V) return fail(ctx, QT_EINVAL, "bad arguments to qt_backward");
     if (counts_type != QT_COUNTS_I64 && counts_type != QT_COUNTS_U32)
@@ -1534,9 +1535,9 @@ qt_status backward_impl(qt_ctx* ctx, int32_t n, const int64_t* N, const void* co
             ctx->up_tree ^= 1;
             const cudaError_t e =
                 launch_backward_tree(counts, u32, n, maxN, (unsigned char*)dt + kHead, phi, V, (double*)dx,
-                                     (DevStatus*)dt, budget, ctx->num_sms, st);
+                                     status ? status : (DevStatus*)dt, budget, ctx->num_sms, st);
             QT_CUDA(cudaEventRecord(ctx->ev_tree, st));
-            ctx->tree_status = dt;
+            if (!status) ctx->tree_status = dt;
             if (e != cudaErrorCooperativeLaunchTooLarge) {
                 QT_CUDA(e);
                 return QT_OK;
@@ -1559,7 +1560,7 @@ extern "C" qt_status qt_backward(qt_ctx* ctx, int32_t n, const int64_t* N, const
                                  const double* phi, double* V, void* stream)
 {
     if (!ctx) return QT_EINVAL;
-    return backward_impl(ctx, n, N, counts, counts_type, phi, V, 0, stream);
+    return backward_impl(ctx, n, N, counts, counts_type, phi, V, 0, nullptr, stream);
 }
 
 extern "C" qt_status qt_swing(qt_ctx* ctx, int32_t n, const int64_t* N, const void* counts, int32_t counts_type,
@@ -1656,7 +1657,8 @@ extern "C" qt_status qt_price(qt_ctx* ctx, const qt_model* model, const double* 
     }
     if (!fused) {
         if ((s = qt_transitions(ctx, model, dgrids, M, seed, &o, dcounts, nullptr, nullptr, stream))) return s;
-        if ((s = backward_impl(ctx, n, model->N, dcounts, o.counts_type, dphi, (double*)dV, o.spin_budget, stream)))
+        if ((s = backward_impl(ctx, n, model->N, dcounts, o.counts_type, dphi, (double*)dV, o.spin_budget,
+                               (DevStatus*)ctx->status_buf, stream)))
             return s;
     } else {
         // layers in reverse order: the counts of pair (k, k + 1), then V_k from
@@ -1688,8 +1690,12 @@ extern "C" qt_status qt_price(qt_ctx* ctx, const qt_model* model, const double* 
     root_price_kernel<<<1, 1024, 0, st>>>(dcounts, o.counts_type == QT_COUNTS_U32, (int)model->N[0], (int)model->N[1],
                                         (const double*)dV, (double*)dout);
     QT_CUDA(cudaGetLastError());
-    QT_CUDA(cudaMemcpyAsync(price, dout, sizeof(double), cudaMemcpyDeviceToHost, st));
-    return read_status(ctx, st, stats, (long long)n * M, 2ll * n * M);
+    // one wait for the value and the status
+    double* const value = (double*)(ctx->status_host + 2);
+    QT_CUDA(cudaMemcpyAsync(value, dout, sizeof(double), cudaMemcpyDeviceToHost, st));
+    s = read_status(ctx, st, stats, (long long)n * M, 2ll * n * M);
+    *price = *value;
+    return s;
 }
 
 // ------------------------------------------------------------------ grid builder

@@ -369,7 +369,12 @@ __global__ void __launch_bounds__(kTreeThreads) backward_tree_kernel(const C* __
         return;
     }
     const int t = threadIdx.x;
-    bool gave_up = false;
+    // a negative budget gives up without waiting, as every bounded wait does
+    bool gave_up = budget_us < 0;
+    auto record = [&]() {
+        if (atomicCAS(&status->code, 0, 4 /* QT_ETIMEOUT */) == 0) status->where = 60;
+    };
+    if (gave_up) record();
     TreeLayer Ln = layers[n], L = layers[n - 1];
     for (int i = blockIdx.x * kHalf + t; i < Ln.N; i += gridDim.x * kHalf) V[Ln.goff + i] = phi[Ln.goff + i];
     for (int s = 0; s < n; ++s) {
@@ -380,8 +385,6 @@ __global__ void __launch_bounds__(kTreeThreads) backward_tree_kernel(const C* __
 #pragma unroll
         for (int q = 0; q < kTreeMaxN / kHalf; ++q) v[q] = t + q * kHalf < Ln.N ? kUnset : 0ull;
         unsigned long long t0 = 0;
-        // a negative budget gives up without waiting, as every bounded wait does
-        bool give_up = s > 0 && !gave_up && budget_us < 0;
         for (int polls = 0;; ++polls) {
 #pragma unroll
             for (int q = 0; q < kTreeMaxN / kHalf; ++q) {
@@ -393,17 +396,13 @@ __global__ void __launch_bounds__(kTreeThreads) backward_tree_kernel(const C* __
             bool missing = false;
 #pragma unroll
             for (int q = 0; q < kTreeMaxN / kHalf; ++q) missing |= v[q] == kUnset;
-            if ((!missing && !give_up) || s == 0 || gave_up) break;
+            if (!missing || s == 0 || gave_up) break;
             if ((polls & 255) == 255) {
                 unsigned long long now;
                 asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
                 if (t0 == 0) t0 = now;
-                give_up = give_up || now - t0 > (unsigned long long)budget_us * 1000ull;
-            }
-            if (give_up) {
-                gave_up = true;
-                if (atomicCAS(&status->code, 0, 4 /* QT_ETIMEOUT */) == 0) status->where = 60;
-                break;
+                gave_up = now - t0 > (unsigned long long)budget_us * 1000ull;
+                if (gave_up) record();
             }
         }
         bool odd = false;
